@@ -270,12 +270,6 @@ template <class S, class R> __device__ __forceinline__ bool store_overflow(R v, 
     if constexpr (std::is_same<S, __half>::value) return fabsf(float(v)) * sp.st_scale[q] > 60000.0f;
     else return false;
 }
-// the same for the density plane
-template <class S, class R> __device__ __forceinline__ bool store_overflow_c(R v, const SimParams &sp) {
-    if constexpr (std::is_same<S, __half>::value) return fabsf(float(v)) * sp.ct_scale > 60000.0f;
-    else return false;
-}
-
 __device__ __forceinline__ bool allowed_cell(const SimParams &sp, int gx, int gy) {
     if (sp.wall_x && (gx < -2 || gx > sp.nx + 1)) return false;
     if (sp.wall_y && (gy < -2 || gy > sp.ny + 1)) return false;
@@ -1793,6 +1787,14 @@ struct LbArgs {
     unsigned *err;
 };
 
+// v / 3 to a rounding of the result: 1/3 as a float pair in FP32.
+template <class R> __device__ __forceinline__ R third(R v);
+template <> __device__ __forceinline__ float third<float>(float v) {
+    constexpr float hi = 1.0f / 3.0f, lo = (float)(1.0 / 3.0 - (double)hi);
+    return __fmaf_rn(v, hi, __fmul_rn(v, lo));
+}
+template <> __device__ __forceinline__ double third<double>(double v) { return v * (1.0 / 3.0); }
+
 // The arithmetic of one node of K1 once its inputs are loaded: moments, SFC
 // equilibrium, Guo forcing and BGK collision.  f: the stored populations (f[0]
 // becomes relative to this step's Delta rho); fh: the post-collision values in
@@ -1826,8 +1828,6 @@ __device__ __forceinline__ R lb_collide(const SimParams &sp, R (&f)[9], R (&fh)[
     }
     if (!(ux + uy == ux + uy)) atomicOr(err, ERR_NAN);  // a NaN rho makes both velocities NaN
     const R omega = pick<R>(sp.omega, sp.omega_f), kf = pick<R>(sp.kf, sp.kf_f);
-    const R u2 = ux * ux + uy * uy;
-    const R uF = ux * Fx + uy * Fy;
     R dde;
     const R dds = two_diff<R>(dro, drt, dde);
     const R dd = dds + (dde + (dro_lo - drt_lo));  // change of the rest base over the step (small)
@@ -1835,26 +1835,36 @@ __device__ __forceinline__ R lb_collide(const SimParams &sp, R (&f)[9], R (&fh)[
     f[0] += dd;                  // rest population relative to this step's Delta rho
     // Collision f^ = f - omega (f - f^eq) + (1 - omega/2) F_i (Eq. 2_2_bgk_force) with
     // f^eq of Eq. 2_3_feq_sfc in the stored form (minus w rho_f, minus Delta rho for
-    // q = 0) and the Guo term of Eq. 2_2_Fi times rho.  Opposite directions share the
-    // even parts (in c) of f^eq and F_i and differ in the sign of the odd parts.
+    // q = 0) and the Guo term of Eq. 2_2_Fi times rho.  Written out, direction q adds
+    //   w_q (E + 4.5 rho (c.u)(c.h)) + 3 w_q c.g,  g = rho (omega u + kf F),
+    //   h = omega u + 2 kf F,  E = omega (rho - rho_t) - 1.5 rho u.h,
+    // and with the weights 4/9, 1/9, 1/36 everything follows from E / 9, P = rho u / 2,
+    // Px hx, Py hy, Px hy + Py hx and g / 3 by additions and factors of 4: about 52
+    // operations where a sum per direction took 97.  The FP64 and the 16-bit kernel
+    // are bound by their instructions (1024^2 FP64 274 -> 207 us, 4096^2 FP16 staged
+    // 275 -> 254 us); the FP32 one by HBM (4096^2 245 -> 242 us).  The thirds and ninths
+    // are applied in two parts in FP32: a rounded 1/9 scales every equilibrium by
+    // 1 + 7e-9, the same way at every node and step, which was most of the velocity's
+    // error (80^2 cavity, 250 steps: 2.6e-6 -> 3e-7 of u).
     const R om1 = R(1) - omega;
-    const R r15u2 = R(1.5) * u2, r3uF = R(3) * uF;
-    {
-        const R w = R(4) / R(9), rw = rho * w;
-        fh[0] = om1 * f[0] + omega * (w * ddr - rw * r15u2) - kf * rw * r3uF;
-    }
-#pragma unroll
-    for (int pr = 0; pr < 4; pr++) {
-        const int q = pr + 1 + (pr >= 2 ? 2 : 0);  // 1, 2, 5, 6; partners 3, 4, 7, 8
-        const int qo = oppq(q);
-        const R w = wq<R>(q), rw = rho * w;
-        const R cu = R(cxq(q)) * ux + R(cyq(q)) * uy;
-        const R cF = R(cxq(q)) * Fx + R(cyq(q)) * Fy;
-        const R even = omega * (w * ddr + rw * (R(4.5) * cu * cu - r15u2)) + kf * rw * (R(9) * cu * cF - r3uF);
-        const R odd = R(3) * rw * (omega * cu + kf * cF);
-        fh[q] = om1 * f[q] + even + odd;
-        fh[qo] = om1 * f[qo] + even - odd;
-    }
+    const R hr = R(0.5) * rho, px = hr * ux, py = hr * uy;
+    const R ox = omega * ux, oy = omega * uy, kf2 = kf + kf;
+    const R hx = fma_rn<R>(kf2, Fx, ox), hy = fma_rn<R>(kf2, Fy, oy);
+    const R gx = third<R>(rho * fma_rn<R>(kf, Fx, ox)), gy = third<R>(rho * fma_rn<R>(kf, Fy, oy));
+    const R ax = px * hx, ay = py * hy, s2 = ax + ay, xy = fma_rn<R>(px, hy, mul_rn<R>(py, hx));
+    const R E = third<R>(third<R>(omega * ddr) - s2);
+    fh[0] = fma_rn<R>(om1, f[0], R(4) * E);
+    const R ex = E + ax, ey = E + ay;
+    fh[1] = fma_rn<R>(om1, f[1], ex + gx);
+    fh[3] = fma_rn<R>(om1, f[3], ex - gx);
+    fh[2] = fma_rn<R>(om1, f[2], ey + gy);
+    fh[4] = fma_rn<R>(om1, f[4], ey - gy);
+    const R q4 = R(0.25), e4 = q4 * (E + s2), x4 = q4 * xy, a4 = q4 * (gx + gy), b4 = q4 * (gy - gx);
+    const R ep = e4 + x4, em = e4 - x4;
+    fh[5] = fma_rn<R>(om1, f[5], ep + a4);
+    fh[7] = fma_rn<R>(om1, f[7], ep - a4);
+    fh[6] = fma_rn<R>(om1, f[6], em + b4);
+    fh[8] = fma_rn<R>(om1, f[8], em - b4);
     return dr;
 }
 
@@ -1907,11 +1917,12 @@ __device__ __forceinline__ R lb_node(const SimParams &sp, const LbArgs<R, S> &a,
     } else {
         stC<S, R>(a.carry + c, dr, sp);
     }
-    if constexpr (is16<S>()) {
-        bool ov = store_overflow_c<S, R>(dr, sp);
+    if constexpr (std::is_same<S, __half>::value) {
+        // a stored value beyond FP16's range: one maximum and one test (a NaN raises nothing here)
+        float top = fabsf(float(dr)) * sp.ct_scale;
 #pragma unroll
-        for (int q = 0; q < 9; q++) ov = ov || store_overflow<S, R>(fh[q], sp, q);
-        if (ov) atomicOr(a.err, ERR_OVERFLOW16);
+        for (int q = 0; q < 9; q++) top = fmaxf(top, fabsf(float(fh[q])) * sp.st_scale[q]);
+        if (top > 60000.0f) atomicOr(a.err, ERR_OVERFLOW16);
     }
     stS<S, R>(a.fout_push[0] + c, fh[0], sp, 0);
     if (interior) {
