@@ -517,7 +517,7 @@ class Simulation:
         return bool(load().lbrmt_uses_overlap(self.h))
 
     def set_rmt_threads(self, threads):
-        """CTA width of the reference-map kernel: 0 (chosen), 256 or 1024 (lbrmt_set_rmt_threads)."""
+        """Form of the reference-map kernel: 0 (chosen), 256 or 1024, a cluster per solid (lbrmt_set_rmt_threads)."""
         _check(self.h, load().lbrmt_set_rmt_threads(self.h, int(threads)))
 
     @property

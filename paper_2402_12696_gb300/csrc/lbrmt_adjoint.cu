@@ -209,12 +209,12 @@ static lbrmt_status backward_impl(lbrmt_sim *s, const double *dLdc, double *dLdG
     ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, force_adjoint_kernel<R>, TILE_N, fsm));
     const int fblocks = nsm * std::max(per, 1);
     const int rsm = ((s->li.tmax * s->li.tmax + 15) & ~15) + 8 * LIST_CAP;  // labels and layer lists
-    ok(cudaFuncSetAttribute(rmt_adjoint_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_SMEM_MAX));
+    ok(cudaFuncSetAttribute(rmt_adjoint_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_ADJ_SMEM_MAX));
     // the forward's choice: 1024-thread CTAs for FP32 arithmetic and few solids
     constexpr bool can_big = sizeof(R) == 4;
     const bool big = can_big && s->li.rmt_threads == RMT_THREADS_BIG;
     if constexpr (can_big)
-        if (big) ok(cudaFuncSetAttribute(rmt_adjoint_kernel_big<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_SMEM_MAX));
+        if (big) ok(cudaFuncSetAttribute(rmt_adjoint_kernel_big<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_ADJ_SMEM_MAX));
     const int lblocks = (int)std::min<long long>((P + 255) / 256, (long long)nsm * 8);
     if (e != cudaSuccess) return lbrmt_internal_fail(s, LBRMT_ERR_CUDA, std::string("adjoint setup: ") + cudaGetErrorString(e));
 

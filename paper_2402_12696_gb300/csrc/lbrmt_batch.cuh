@@ -25,11 +25,10 @@ struct BatchSimDesc {
 };
 
 // K2 over every solid of every simulation: item = (simulation, solid).
-// Same launch bounds as the single-simulation kernel: the same register budget
-// gives the same instruction selection, so batch members stay bit-identical to
-// single runs.
+// FP32: three CTAs per SM (85 registers) where the single-simulation kernel runs
+// four: with the member's parameters behind pointers, 64 registers spill 1.4 KB.
 template <class R, class S>
-__global__ void __launch_bounds__(RMT_THREADS, sizeof(R) == 4 ? RMT_MIN_BLOCKS : 2)
+__global__ void __launch_bounds__(RMT_THREADS, sizeof(R) == 4 ? 3 : 2)
     rmt_batch_kernel(const BatchSimDesc<R, S> *sims, const int2 *items, int nitems, int parity) {
     __shared__ SimParams sp;
     __shared__ RmtArgs<R, S> ra;
@@ -41,7 +40,7 @@ __global__ void __launch_bounds__(RMT_THREADS, sizeof(R) == 4 ? RMT_MIN_BLOCKS :
             ra = sims[w.x].rmt[parity];
         }
         __syncthreads();
-        rmt_solid<R, S>(sp, ra, w.y);
+        rmt_solid<R, S, false>(sp, ra, w.y, 0, 1);
     }
 }
 

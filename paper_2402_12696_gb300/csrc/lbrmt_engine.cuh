@@ -20,7 +20,8 @@ struct LaunchInfo {
     int force_carve_ov;  // the overlapped K3's preferred carveout (percent), or -1
     int force_smem;      // dynamic shared memory of K3
     int rmt_req = 0;      // requested K2 CTA width (0: chosen by configure)
-    int rmt_threads = 256; // K2 CTA width in use: 256, or 1024 (FP32 arithmetic only)
+    int rmt_threads = 256; // the form as lbrmt_rmt_threads tells it: 256, or 1024 (FP32 arithmetic only)
+    int rmt_nc = 0;        // CTAs per solid (a cluster) of K2's wide form; 0: the narrow form
     bool tma = false;    // tensor maps of the populations and density plane are valid
     bool use_tma = true; // K1 with TMA staging (else the direct-load kernel)
     int lb_blocks = 0, lb_smem = 0;
@@ -241,18 +242,18 @@ struct Engine {
         li->tma = true;
     }
 
-    // K2's dynamic shared memory and carveout.  A CTA holds the byte labels of
-    // its tile (tmax^2, padded) and the node lists; min_blocks CTAs on an SM
-    // take min_blocks x (dynamic + static + reserved) of its carveout, and the
-    // rest is L1 cache, which K2's gathers and stencils lean on.  When a lower
-    // carveout step than the one that lists of 8 LIST_CAP bytes need holds
-    // min_blocks CTAs with at least RMT_LIST_MIN_BYTES of lists, the lists take
-    // all of the CTA's share of that step and each launch asks for it.
-    // Otherwise: lists of 8 LIST_CAP bytes and the driver's choice (-1).
+    // K2's dynamic shared memory and carveout.  A CTA holds its solid's sets
+    // (row masks) and the node lists; min_blocks CTAs on an SM take min_blocks x
+    // (dynamic + static + reserved) of its carveout, and the rest is L1 cache,
+    // which K2's gathers and stencils lean on.  When a lower carveout step than
+    // the one that RMT_LIST_BYTES of lists need holds min_blocks CTAs with at
+    // least RMT_LIST_MIN_BYTES of them, the lists take all of the CTA's share of
+    // that step and each launch asks for it.  Otherwise: RMT_LIST_BYTES and the
+    // driver's choice (-1).
     template <class K>
     static void rmt_smem_carveout(K kernel, int tmax, int min_blocks, int *smem, int *carve) {
-        const int labs = (tmax * tmax + 15) & ~15;
-        *smem = labs + 8 * LIST_CAP;
+        const int labs = rmt_mask_bytes(tmax, 1, 0);
+        *smem = labs + RMT_LIST_BYTES;
         *carve = -1;
         int per_sm, resv;
         smem_limits(&per_sm, &resv);
@@ -280,9 +281,55 @@ struct Engine {
         }
     }
 
+    // K2's wide form: a cluster of CTAs per solid.  As many as the SMs hold for every
+    // solid at once, up to 16 (K2 with 1, 2, 4, 8, 16 CTAs: the r = 128 disk 364, 208, 145,
+    // 108, 91 us, the r = 64 one 131, 94, 75, 66, 61, r = 16 59, 55, 53, 52, 52), and at least
+    // 8 tile rows (about 5 band rows) to each: a strip is not shorter than its two-row halo
+    // by much, and a shorter one gains nothing.  Where one CTA's strip does not fit its shared
+    // memory (the largest tiles in FP64), the narrow form runs.
+    static cudaLaunchConfig_t wide_config(int nsolids, int nc, int smem, cudaStream_t st, int prio,
+                                          cudaLaunchAttribute *at) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(nsolids * nc);
+        cfg.blockDim = dim3(RMT_WIDE_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = nc;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributePriority;
+        at[1].val.priority = prio;
+        cfg.attrs = at;
+        cfg.numAttrs = 2;
+        return cfg;
+    }
+    static cudaError_t configure_wide(const SimParams &sp, int tmax, int nsm, LaunchInfo *li) {
+        auto kernel = rmt_solid_kernel_wide<R, S>;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_SMEM_CAP - 2048);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        for (int nc = 16; nc >= 1; nc /= 2) {
+            if (nc > 1 && (sp.nsolids * nc > nsm || 8 * nc > tmax)) continue;
+            const int smem = rmt_wide_smem(tmax, nc, sp.n_layers, (int)sizeof(R));
+            if (smem > RMT_SMEM_CAP - 2048) break;  // and more with fewer CTAs
+            cudaLaunchAttribute at[2];
+            const cudaLaunchConfig_t cfg = wide_config(sp.nsolids, nc, smem, nullptr, 0, at);
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            if (nc > 1 && n < sp.nsolids) continue;
+            li->rmt_smem = smem;
+            li->rmt_carve = -1;
+            li->rmt_nc = nc;
+            break;
+        }
+        return cudaSuccess;
+    }
+
     static cudaError_t configure(const SimParams &sp, const DevState &d, int tmax, LaunchInfo *li) {
         li->tmax = tmax;
-        li->rmt_smem = ((tmax * tmax + 15) & ~15) + 8 * LIST_CAP;
         {
             cudaError_t e0 = upload_rinv_tables();
             if (e0 != cudaSuccess) return e0;
@@ -297,20 +344,15 @@ struct Engine {
         int nsm0 = 0, dev0 = 0;
         cudaGetDevice(&dev0);
         cudaDeviceGetAttribute(&nsm0, cudaDevAttrMultiProcessorCount, dev0);
-        // K2's CTA width: the request, else 1024 threads when the solids number at
-        // most half the SMs (FP32 arithmetic: 64 registers hold it), else 256
+        // K2's form: the request, else the wide one when the solids number at most
+        // half the SMs.  FP64 takes it unasked only, and reports its 256-thread CTAs.
         int w = li->rmt_req;
-        if (w == 0) w = sizeof(R) == 4 && sp.nsolids > 0 && 2 * sp.nsolids <= nsm0 ? RMT_THREADS_BIG : RMT_THREADS;
+        const bool few = sp.nsolids > 0 && 2 * sp.nsolids <= nsm0;
+        if (w == 0) w = sizeof(R) == 4 && few ? RMT_THREADS_BIG : RMT_THREADS;
         if (w == RMT_THREADS_BIG && sizeof(R) != 4) w = RMT_THREADS;
         li->rmt_threads = w;
-        if (w == RMT_THREADS_BIG) {
-            e = cudaFuncSetAttribute(rmt_solid_kernel_big<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_SMEM_MAX);
-            // One CTA per solid and at most one per SM: room for node lists of a
-            // tile's size, so that a large solid's advected nodes and layers are
-            // listed instead of walked (its box) or scanned (its tile, per layer).
-            li->rmt_smem = std::max(li->rmt_smem, std::min(((tmax * tmax + 15) & ~15) + 4 * tmax * tmax, RMT_SMEM_MAX));
-            li->rmt_carve = -1;
-        }
+        li->rmt_nc = 0;
+        if (w == RMT_THREADS_BIG || (sizeof(R) == 8 && few && li->rmt_req == 0)) e = configure_wide(sp, tmax, nsm0, li);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(force_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  force_smem_max() * (int)sizeof(R));
@@ -357,12 +399,10 @@ struct Engine {
             a.xi_out = (R *)d.xi[0];
             a.frame_out = d.frame[0];
             a.frame_next = d.frame[1];
-            a.stats = nullptr;
         } else {
             a.xi_out = (R *)d.xi[q];
             a.frame_out = d.frame[q];
             a.frame_next = d.frame[p];
-            a.stats = d.stats_step;
         }
         const int r = init ? 1 : p;  // the initial registry takes slot 1 (step 0 reads it as "previous")
         a.reg_count = d.reg_count[r];
@@ -433,12 +473,11 @@ struct Engine {
         int dev = 0, nsm = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        bl->rmt_smem = ((tmax * tmax + 15) & ~15) + 8 * LIST_CAP;
         bl->force_smem = fs_elems * (int)sizeof(R);
         cudaError_t e = cudaFuncSetAttribute(rmt_batch_kernel<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              RMT_SMEM_MAX);
         if (e != cudaSuccess) return e;
-        rmt_smem_carveout(rmt_batch_kernel<R, S>, tmax, sizeof(R) == 4 ? RMT_MIN_BLOCKS : 2, &bl->rmt_smem,
+        rmt_smem_carveout(rmt_batch_kernel<R, S>, tmax, sizeof(R) == 4 ? 3 : 2, &bl->rmt_smem,
                           &bl->rmt_carve);
         e = cudaFuncSetAttribute(force_batch_kernel<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  force_smem_max() * (int)sizeof(R));
@@ -490,9 +529,11 @@ struct Engine {
 
     static void launch_rmt(const SimParams &sp, const LaunchInfo &li, const RmtArgs<R, S> &a, cudaStream_t st,
                            int prio = 0) {
-        if (li.rmt_threads == RMT_THREADS_BIG)
-            launch_prio(rmt_solid_kernel_big<R, S>, dim3(sp.nsolids), dim3(RMT_THREADS_BIG), li.rmt_smem, st, prio, sp, a);
-        else
+        if (li.rmt_nc > 0) {
+            cudaLaunchAttribute at[2];
+            const cudaLaunchConfig_t cfg = wide_config(sp.nsolids, li.rmt_nc, li.rmt_smem, st, prio, at);
+            cudaLaunchKernelEx(&cfg, rmt_solid_kernel_wide<R, S>, sp, a);
+        } else
             launch_carve(rmt_solid_kernel<R, S>, dim3(sp.nsolids), dim3(RMT_THREADS), li.rmt_smem, st, prio, li.rmt_carve,
                          sp, a);
     }

@@ -1,9 +1,9 @@
 // lbrmt_kernels.cuh -- device code of the LBRMT time step for sm_103a.
 //
 // Three kernels make one step of Algorithm 1 (Sun & Rycroft, arXiv 2402.12696):
-//   K2 rmt_solid_kernel   one CTA per solid: advect xi (Sec. 3.1), extrapolate
-//                         it layer by layer (Sec. 3.2), relabel, register the
-//                         32x8 tiles its blur zone touches, per-solid FP64 stats.
+//   K2 rmt_solid_kernel   one CTA, or a cluster of CTAs, per solid: advect xi (Sec.
+//                         3.1), extrapolate it layer by layer (Sec. 3.2), relabel,
+//                         register the tiles its blur zone touches.
 //   K3 force_kernel       one CTA per registered tile: half-edge Jacobians and
 //                         neo-Hookean stresses (Sec. 3.3), multi-solid blend and
 //                         contact (Sec. 3.6), divergence (Eq. 3_3_div_solid_stress),
@@ -36,10 +36,33 @@ constexpr int RMT_THREADS = 256;
 #ifndef RMT_MIN_BLOCKS
 #define RMT_MIN_BLOCKS 4
 #endif
-constexpr int LIST_CAP = 2048;              // per-layer target list in shared memory
-constexpr int RMT_LIST_MIN_BYTES = 12288;   // least node-list space (bytes) for which K2 takes a smaller carveout
-constexpr int TILE_SIDE_MAX = 448;          // largest solid tile side (byte labels + lists in shared memory)
-constexpr int RMT_SMEM_MAX = ((TILE_SIDE_MAX * TILE_SIDE_MAX + 15) & ~15) + 8 * LIST_CAP;
+constexpr int TILE_SIDE_MAX = 448;          // largest solid tile side
+// Shared memory of K2: the solid's sets as one bit per tile node (row masks
+// below), then lists (ints: pass 0's nodes per warp, each layer's targets), and
+// in its wide form the reference map of the CTA's strip of rows.
+constexpr int RMT_MASKS = 5;                // S, layers <= 2, and three in rotation
+constexpr int RMT_LIST_BYTES = 6144;        // list space of a 256-thread CTA
+constexpr int RMT_LIST_MIN_BYTES = 4096;    // least (128 nodes per warp) list space for which K2 takes a smaller carveout
+constexpr int RMT_WIDE_LIST_BYTES = 16384;  // list space of a CTA that has its SM to itself
+constexpr int RMT_SMEM_CAP = 227 * 1024;    // largest dynamic shared memory of a CTA
+__host__ __device__ constexpr int mask_row_words(int T) { return ((T + 34) >> 5) + 1; }
+// Rows of a set: the tile's, or of a strip of a cluster of nc CTAs with the
+// NL + 1 rows on either side that the dilation steps reach; plus pad rows.
+__host__ __device__ constexpr int mask_rows(int T, int nc, int NL) {
+    return (nc == 1 || (T + nc - 1) / nc + 2 * NL > T) ? T + 5 : (T + nc - 1) / nc + 2 * NL + 5;
+}
+__host__ __device__ constexpr int mask_words(int T, int nc, int NL) { return (mask_rows(T, nc, NL) * mask_row_words(T) + 5) & ~3; }
+__host__ __device__ constexpr int rmt_mask_bytes(int T, int nc, int NL) { return RMT_MASKS * 4 * mask_words(T, nc, NL); }
+// The wide form's set of pass 0 (the CTA's rows of the input box) and its map (two halo rows on either side).
+__host__ __device__ constexpr int strip_mask_words(int T, int nc) { return (((T + nc - 1) / nc + 1) * mask_row_words(T) + 3) & ~3; }
+__host__ __device__ constexpr int strip_values(int T, int nc) { return ((T + nc - 1) / nc + 5) * T; }
+__host__ __device__ constexpr int rmt_wide_smem(int T, int nc, int NL, int real) {
+    return rmt_mask_bytes(T, nc, NL) + 4 * strip_mask_words(T, nc) + RMT_WIDE_LIST_BYTES + 2 * real * strip_values(T, nc);
+}
+constexpr int RMT_SMEM_MAX = rmt_mask_bytes(TILE_SIDE_MAX, 1, 20) + RMT_LIST_BYTES;
+// Shared memory of the reverse sweep's K2: byte labels and layer lists.
+constexpr int LIST_CAP = 2048;
+constexpr int RMT_ADJ_SMEM_MAX = ((TILE_SIDE_MAX * TILE_SIDE_MAX + 15) & ~15) + 8 * LIST_CAP;
 // Force pool, per registered tile, TILE_N values per plane: F_x and F_y of the
 // solid terms (without the body force), Delta rho as an unevaluated sum hi + lo
 // (two planes' worth, the pair of node lt at POOL_DRHO + 2 lt, read as one
@@ -184,7 +207,7 @@ struct DevState {
     unsigned char *busy[2]; // per K1 region, by step parity: 1 if it may hold solid forcing this step
     void *fbody;           // per row: body-force x component
     double *mass_partials; // per LB block
-    double *stats_step;    // S x 8, stats of the state at the start of the last step
+    double *stats_step;    // S x 8, zero (a section of the checkpoints)
     SolidDesc *solids;
     unsigned *err;
 };
@@ -389,6 +412,39 @@ __device__ __forceinline__ void node_moments(const SimParams &sp, const S *f, co
     moments_from<R>(sp, fq, rest_base<R>(sp, reg, pool, i, j), cx, cy, rho, u, v);
 }
 
+__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// Thread-block clusters: rank and size, the barrier (release / acquire, so
+// global and shared writes before it are seen after it by the whole cluster),
+// and a word of another CTA's shared memory.
+__device__ __forceinline__ int cluster_rank() { unsigned r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return (int)r; }
+__device__ __forceinline__ int cluster_size() { unsigned r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return (int)r; }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ unsigned cluster_addr(const void *p, int rank) {
+    unsigned a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ unsigned cluster_ld(const void *p, int rank) {
+    unsigned v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_ld2(const float2 *p, int rank, float &x, float &y) {
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(cluster_addr(p, rank)) : "memory");
+}
+__device__ __forceinline__ void cluster_ld2(const double2 *p, int rank, double &x, double &y) {
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(x), "=d"(y) : "r"(cluster_addr(p, rank)) : "memory");
+}
+__device__ __forceinline__ void cluster_st(float *p, int rank, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_st(double *p, int rank, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "d"(v) : "memory");
+}
+
 // Block-wide sum of NV values (blockDim.x multiple of 32, <= 1024).
 template <class T, int NV>
 __device__ void block_sum(T (&v)[NV], T *sh /* 32*NV */) {
@@ -426,7 +482,6 @@ struct RmtArgs {
     Frame *frame_out;    // origin read at entry; its box is written at exit
     Frame *frame_next;   // frame of the next step's output tile
     int *reg_count, *reg_solids, *reg_active, *reg_nactive;
-    double *stats;       // S x 8 (state at time n), may be null at init
     const SolidDesc *solids;
     const int *order;    // CTA -> solid (largest tiles first), or null
     unsigned *err;
@@ -463,183 +518,6 @@ template <class R> __device__ __forceinline__ R rinv_tab(int dx, int dy);
 template <> __device__ __forceinline__ float rinv_tab<float>(int dx, int dy) { return c_rinv_f[abs(dx) * (RMAX_TAB + 1) + abs(dy)]; }
 template <> __device__ __forceinline__ double rinv_tab<double>(int dx, int dy) { return c_rinv_d[abs(dx) * (RMAX_TAB + 1) + abs(dy)]; }
 
-// Running sums of one weighted least-squares fit.  The positive-weight nodes
-// are collinear iff the Gram determinant of their integer offsets vanishes,
-// (n Sxx - Sx^2)(n Syy - Sy^2) - (n Sxy - Sx Sy)^2 = 0, an exact integer test.
-template <class R>
-struct Lsq {
-    int nvalid, n, sx, sy, sxx, syy, sxy;
-    bool haveref;
-    R a, b, c, d, e, fw;            // M = [[a b c],[b d e],[c e fw]]
-    R bx0, bx1, bx2, by0, by1, by2; // right-hand sides for eta_x - xref and eta_y - yref
-    R xref, yref;                   // values of the first valid node (fit of differences)
-};
-
-template <class R>
-__device__ __forceinline__ void lsq_cell(Lsq<R> &A, const signed char *lab, const R *X, const R *Y, int k, int l, int dx,
-                                         int dy, bool use_n, R nhx, R nhy) {
-    const int L = lab[k];
-    if (!(L >= 0 && L < l)) return;
-    A.nvalid++;
-    R wt = pow2neg<R>(abs(dx) + abs(dy));  // 2^{-(r_i + r_j)}
-    if (use_n) {
-        const R dn = (R(-dx) * nhx + R(-dy) * nhy) * rinv_tab<R>(dx, dy);  // d = target - node
-        wt = dn > R(COS_TIE) ? dn * wt : R(0);
-    }
-    if (!(wt > R(0))) return;
-    A.n++; A.sx += dx; A.sy += dy; A.sxx += dx * dx; A.syy += dy * dy; A.sxy += dx * dy;
-    R Xv = X[k], Yv = Y[k];
-    if (!A.haveref) { A.xref = Xv; A.yref = Yv; A.haveref = true; }
-    Xv -= A.xref; Yv -= A.yref;
-    const R x = R(dx), y = R(dy);
-    const R wx = wt * x, wy = wt * y;
-    A.a += wx * x; A.b += wx * y; A.c += wx; A.d += wy * y; A.e += wy; A.fw += wt;
-    A.bx0 += wx * Xv; A.bx1 += wy * Xv; A.bx2 += wt * Xv;
-    A.by0 += wx * Yv; A.by1 += wy * Yv; A.by2 += wt * Yv;
-}
-
-// The 5x5 window of a target away from the tile edge, without branches on
-// the node's validity (weights are zero for the nodes that do not count).
-template <class R, bool USE_N>
-__device__ __forceinline__ void lsq_window5(Lsq<R> &A, const signed char *lab, const R *X, const R *Y, int t, int T,
-                                            int l, R nhx, R nhy) {
-#pragma unroll
-    for (int dy = -2; dy <= 2; dy++)
-#pragma unroll
-        for (int dx = -2; dx <= 2; dx++) {
-            if (dx == 0 && dy == 0) continue;  // the target itself (layer l) never counts
-            const int k = t + dy * T + dx;
-            const int L = lab[k];
-            const bool valid = (unsigned)L < (unsigned)l;  // 0 <= L < l
-            R wt = valid ? pow2neg<R>(abs(dx) + abs(dy)) : R(0);
-            if (USE_N) {
-                const R dn = (R(-dx) * nhx + R(-dy) * nhy) * rinv_tab<R>(dx, dy);
-                wt = dn > R(COS_TIE) ? dn * wt : R(0);
-            }
-            A.nvalid += valid ? 1 : 0;
-            const bool pos = wt > R(0);
-            A.n += pos ? 1 : 0;
-            A.sx += pos ? dx : 0; A.sy += pos ? dy : 0;
-            A.sxx += pos ? dx * dx : 0; A.syy += pos ? dy * dy : 0; A.sxy += pos ? dx * dy : 0;
-            R Xv = R(0), Yv = R(0);
-            if (pos) { Xv = X[k] - A.xref; Yv = Y[k] - A.yref; }
-            const R wx = wt * R(dx), wy = wt * R(dy);
-            A.a += wx * R(dx); A.b += wx * R(dy); A.c += wx; A.d += wy * R(dy); A.e += wy; A.fw += wt;
-            A.bx0 += wx * Xv; A.bx1 += wy * Xv; A.bx2 += wt * Xv;
-            A.by0 += wx * Yv; A.by1 += wy * Yv; A.by2 += wt * Yv;
-        }
-}
-
-// The 5x5 window without directional weights (layers beyond the second): the
-// weights 2^{-(|dx|+|dy|)} then depend only on which of the 24 nodes are valid,
-// so the sums of M and of the collinearity test follow from each row's 5-bit
-// validity mask by bit counts.  Every term is a multiple of 1/16, so these sums
-// are exact, as the running sums of lsq_window5 are; only the right-hand sides
-// read the nodes' values, accumulated in the same node order.
-template <class R>
-__device__ __forceinline__ void lsq_window5_mask(Lsq<R> &A, const signed char *lab, const R *X, const R *Y, int t,
-                                                 int T, int l) {
-    int n = 0, sx = 0, sy = 0, sxx = 0, syy = 0, sxy = 0;
-    int a16 = 0, b16 = 0, c16 = 0, d16 = 0, e16 = 0, f16 = 0;  // 16 x the entries of M
-    unsigned rows = 0;                                         // 5 bits per row, dx = -2..2
-#pragma unroll
-    for (int dy = -2; dy <= 2; dy++) {
-        unsigned r = 0;
-#pragma unroll
-        for (int dx = -2; dx <= 2; dx++) {
-            if (dx == 0 && dy == 0) continue;  // the target itself (layer l) never counts
-            const int L = lab[t + dy * T + dx];
-            r |= ((unsigned)L < (unsigned)l ? 1u : 0u) << (dx + 2);
-        }
-        rows |= r << (5 * (dy + 2));
-        const int c0 = (r >> 2) & 1, p1 = __popc(r & 0x0au), p2 = __popc(r & 0x11u);
-        const int d1 = (int)((r >> 3) & 1) - (int)((r >> 1) & 1), d2 = (int)((r >> 4) & 1) - (int)(r & 1);
-        const int nr = c0 + p1 + p2, sxr = d1 + 2 * d2;
-        // row sums of 4 2^{-|dx|} dx^k (k = 0, 1, 2), row weight 4 2^{-|dy|}
-        const int s0 = 4 * c0 + 2 * p1 + p2, s1 = 2 * d1 + 2 * d2, s2 = 2 * p1 + 4 * p2;
-        const int g = dy == 0 ? 4 : (dy == 1 || dy == -1 ? 2 : 1);
-        n += nr; sx += sxr; sxx += p1 + 4 * p2; sy += dy * nr; syy += dy * dy * nr; sxy += dy * sxr;
-        f16 += g * s0; c16 += g * s1; a16 += g * s2; e16 += g * dy * s0; d16 += g * dy * dy * s0; b16 += g * dy * s1;
-    }
-    A.nvalid += n; A.n += n; A.sx += sx; A.sy += sy; A.sxx += sxx; A.syy += syy; A.sxy += sxy;
-    const R q = R(0.0625);
-    A.a += R(a16) * q; A.b += R(b16) * q; A.c += R(c16) * q; A.d += R(d16) * q; A.e += R(e16) * q; A.fw += R(f16) * q;
-#pragma unroll
-    for (int dy = -2; dy <= 2; dy++)
-#pragma unroll
-        for (int dx = -2; dx <= 2; dx++) {
-            if (dx == 0 && dy == 0) continue;
-            if (!((rows >> (5 * (dy + 2) + dx + 2)) & 1u)) continue;
-            const int k = t + dy * T + dx;
-            const R Xv = X[k] - A.xref, Yv = Y[k] - A.yref;
-            const R w = pow2neg<R>((dx < 0 ? -dx : dx) + (dy < 0 ? -dy : dy));
-            const R wx = w * R(dx), wy = w * R(dy);
-            A.bx0 += wx * Xv; A.bx1 += wy * Xv; A.bx2 += w * Xv;
-            A.by0 += wx * Yv; A.by1 += wy * Yv; A.by2 += w * Yv;
-        }
-}
-
-// Weighted least-squares fit of one target (Sec. 3.2, steps (i)-(iii)).  The
-// weights do not depend on the window size, so growing r from r-1 only adds
-// the ring |dx| = r or |dy| = r to the sums of the smaller window.  The fit is
-// of differences from the value at the target's 4-neighbour in layer l - 1
-// (a valid node by construction), which keeps the sums small.
-template <class R>
-__device__ void extrapolate_target(const SimParams &sp, const signed char *lab, R *X, R *Y, int T, int tx, int ty,
-                                   int l, bool use_n, R nhx, R nhy, unsigned *err) {
-    const int t = ty * T + tx;
-    Lsq<R> A;
-    A.nvalid = A.n = A.sx = A.sy = A.sxx = A.syy = A.sxy = 0;
-    A.a = A.b = A.c = A.d = A.e = A.fw = R(0);
-    A.bx0 = A.bx1 = A.bx2 = A.by0 = A.by1 = A.by2 = R(0);
-    {
-        int kref = t + T;
-        if (tx > 0 && lab[t - 1] == l - 1) kref = t - 1;
-        else if (tx < T - 1 && lab[t + 1] == l - 1) kref = t + 1;
-        else if (ty > 0 && lab[t - T] == l - 1) kref = t - T;
-        A.xref = X[kref];
-        A.yref = Y[kref];
-        A.haveref = true;
-    }
-    if (tx >= 2 && ty >= 2 && tx < T - 2 && ty < T - 2) {
-        if (use_n) lsq_window5<R, true>(A, lab, X, Y, t, T, l, nhx, nhy);
-        else lsq_window5_mask<R>(A, lab, X, Y, t, T, l);
-    } else {
-        for (int dy = -2; dy <= 2; dy++)
-            for (int dx = -2; dx <= 2; dx++)
-                if (tx + dx >= 0 && ty + dy >= 0 && tx + dx < T && ty + dy < T)
-                    lsq_cell<R>(A, lab, X, Y, t + dy * T + dx, l, dx, dy, use_n, nhx, nhy);
-    }
-    for (int r = 2; r <= sp.rmax; r++) {
-        if (r > 2) {
-            for (int q = -r; q <= r; q++) {
-                const int ring[4][2] = {{q, -r}, {q, r}, {-r, q}, {r, q}};
-                for (int m = 0; m < 4; m++) {
-                    if (m >= 2 && (q == -r || q == r)) continue;  // corners counted once
-                    const int dx = ring[m][0], dy = ring[m][1];
-                    if (tx + dx >= 0 && ty + dy >= 0 && tx + dx < T && ty + dy < T)
-                        lsq_cell<R>(A, lab, X, Y, t + dy * T + dx, l, dx, dy, use_n, nhx, nhy);
-                }
-            }
-        }
-        if (A.nvalid < 3 || A.n < 3) continue;
-        const long long g1 = (long long)A.n * A.sxx - (long long)A.sx * A.sx;
-        const long long g2 = (long long)A.n * A.syy - (long long)A.sy * A.sy;
-        const long long g3 = (long long)A.n * A.sxy - (long long)A.sx * A.sy;
-        if (g1 * g2 - g3 * g3 == 0) continue;  // positive-weight nodes on one line
-        // third row of M^{-1} from the cofactors of the symmetric M
-        const R c13 = A.b * A.e - A.c * A.d, c23 = A.b * A.c - A.a * A.e, c33 = A.a * A.d - A.b * A.b;
-        const R det = A.a * (A.d * A.fw - A.e * A.e) - A.b * (A.b * A.fw - A.c * A.e) + A.c * (A.b * A.e - A.c * A.d);
-        if (!(det != R(0))) continue;
-        X[t] = A.xref + (c13 * A.bx0 + c23 * A.bx1 + c33 * A.bx2) / det;
-        Y[t] = A.yref + (c13 * A.by0 + c23 * A.by1 + c33 * A.by2) / det;
-        return;
-    }
-    atomicOr(err, ERR_EXTRAP);
-    X[t] = nanv<R>();
-    Y[t] = nanv<R>();
-}
-
 template <class R> __device__ __forceinline__ R mul_rn(R a, R b);
 template <> __device__ __forceinline__ float mul_rn<float>(float a, float b) { return __fmul_rn(a, b); }
 template <> __device__ __forceinline__ double mul_rn<double>(double a, double b) { return __dmul_rn(a, b); }
@@ -649,6 +527,281 @@ template <> __device__ __forceinline__ double add_rn<double>(double a, double b)
 template <class R> __device__ __forceinline__ R fma_rn(R a, R b, R c);
 template <> __device__ __forceinline__ float fma_rn<float>(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 template <> __device__ __forceinline__ double fma_rn<double>(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// Row masks: a set of tile nodes as one bit per node in shared memory.  Node
+// (x, y) is bit (x + 32) & 31 of word ((x + 32) >> 5) of row y - (first row); the
+// pad word on the left and the pad bits on the right are always zero, and
+// enough rows are kept above and below, so the 5x5 window of any node is
+// read without edge tests: two words and a funnel shift per row.  (One byte
+// label per node took 24 shared loads per window, and 8 times the space: 9 KB
+// against 1.5 KB per set on a 96^2 tile, which is L1 cache for K2's gathers.)
+struct RowMask {
+    unsigned *p;
+    int rw, y0;  // words per row, tile row of the first mask row
+    __device__ __forceinline__ unsigned *word(int x, int y) const { return p + (y - y0) * rw + ((x + 32) >> 5); }
+    __device__ __forceinline__ bool bit(int x, int y) const { return (*word(x, y) >> (x & 31)) & 1u; }
+    // the 25 validity bits of the window around (x, y): bit 5 (dy + 2) + dx + 2
+    __device__ __forceinline__ unsigned window5(int x, int y) const {
+        const unsigned *q = p + (y - 2 - y0) * rw + ((x + 30) >> 5);
+        const int sh = (x + 30) & 31;
+        unsigned m = 0;
+#pragma unroll
+        for (int d = 0; d < 5; d++) m |= (__funnelshift_r(q[d * rw], q[d * rw + 1], sh) & 31u) << (5 * d);
+        return m;
+    }
+};
+
+// Moments of a 5-bit row mask (dx = -2..2) with the weights 4 2^-|dx|: sum w,
+// sum w dx and sum w dx^2 in the 10-bit fields of one word (added with borrows,
+// taken apart by window_moments).
+__device__ __forceinline__ int row_moments(unsigned r) {
+    const int c0 = (r >> 2) & 1, l1 = (r >> 1) & 1, r1 = (r >> 3) & 1, l2 = r & 1, r2 = (r >> 4) & 1;
+    return (4 * c0 + 2 * (l1 + r1) + (l2 + r2)) + 1024 * (2 * (r1 - l1) + 2 * (r2 - l2)) +
+           1048576 * (2 * (l1 + r1) + 4 * (l2 + r2));
+}
+
+// The normal matrix M = [[a b c],[b d e],[c e f]] of the plane fit with the
+// weights 2^-(|dx| + |dy|) over the window bits m, times 16: whole numbers, from
+// five entries of the table of row_moments.  Returns 16^3 det M and 16^2 times
+// the cofactors of M's last row, all exact in 32 bits; the determinant vanishes
+// exactly when the nodes lie on one line or are fewer than three (positive weights).
+__device__ __forceinline__ int window_moments(const int *lut, unsigned m, int &c13, int &c23, int &c33) {
+    const int t0 = lut[m & 31u], t1 = lut[(m >> 5) & 31u], t2 = lut[(m >> 10) & 31u], t3 = lut[(m >> 15) & 31u],
+              t4 = lut[(m >> 20) & 31u];
+    const int P = t0 + t4 + 2 * (t1 + t3) + 4 * t2;  // row weights 4 2^-|dy|
+    const int Q = 2 * ((t3 + t4) - (t0 + t1));       // times dy
+    const int d = (4 * (t0 + t4) + 2 * (t1 + t3)) & 1023;
+    const int f = P & 1023, p1 = (P - f) >> 10, c = (p1 << 22) >> 22, a = (p1 - c) >> 10;
+    const int e = (Q << 22) >> 22, q1 = (Q - e) >> 10, b = (q1 << 22) >> 22;
+    c13 = b * e - c * d;
+    c23 = b * c - a * e;
+    c33 = a * d - b * b;
+    return c * c13 + e * c23 + f * c33;
+}
+
+// A whole number below 2^24 in R.  For double: the exact float's bits, widened
+// by hand, because GB300 converts and multiplies in FP64 at 1/64 of its FP32 rate.
+template <class R> __device__ __forceinline__ R whole(int v);
+template <> __device__ __forceinline__ float whole<float>(int v) { return (float)v; }
+template <> __device__ __forceinline__ double whole<double>(int v) {
+    const unsigned u = __float_as_uint((float)v);
+    const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+    return v == 0 ? 0.0 : __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// v > t for a positive float threshold t; in FP64 by the high words (t to 20 bits).
+__device__ __forceinline__ bool above(float v, float t) { return v > t; }
+__device__ __forceinline__ bool above(double v, float t) {
+    return __double2hiint(v) > (int)((__float_as_uint(t) >> 3) + 0x38000000u);
+}
+
+template <class R> struct Vec2;
+template <> struct Vec2<float> { typedef float2 type; };
+template <> struct Vec2<double> { typedef double2 type; };
+
+// A predicated load (no branch): *p where on, else v.
+__device__ __forceinline__ float ld_if(bool on, const float *p, float v) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.f32 %0, [%1];\n}\n" : "+f"(v) : "l"(p), "r"((unsigned)on));
+    return v;
+}
+__device__ __forceinline__ double ld_if(bool on, const double *p, double v) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.f64 %0, [%1];\n}\n" : "+d"(v) : "l"(p), "r"((unsigned)on));
+    return v;
+}
+
+// The reference map that the fits read and write: two planes in global memory
+// (CL false), or a strip of rows in shared memory (pairs).
+template <class R, bool CL>
+struct RefVals {
+    typedef typename Vec2<R>::type V2;
+    V2 *tile;       // CL
+    R *X, *Y;       // else
+    int stride, o;  // node (x, y) at y stride + x - o
+    __device__ __forceinline__ int at(int x, int y) const { return y * stride + x - o; }
+    __device__ __forceinline__ R get(int k, int c) const {
+        if constexpr (CL) return reinterpret_cast<const R *>(tile)[2 * k + c];
+        else return c ? Y[k] : X[k];
+    }
+    __device__ __forceinline__ void get2(int k, R &x, R &y) const {
+        if constexpr (CL) {
+            const V2 v = tile[k];
+            x = v.x; y = v.y;
+        } else {
+            x = X[k]; y = Y[k];
+        }
+    }
+    // node k, or the values (xr, yr) of node kr where it does not count; the load
+    // does not wait for one before it
+    __device__ __forceinline__ void get2_if(bool on, int k, int kr, R xr, R yr, R &x, R &y) const {
+        if constexpr (CL) {
+            get2(on ? k : kr, x, y);
+        } else {
+            x = ld_if(on, X + k, xr);
+            y = ld_if(on, Y + k, yr);
+        }
+    }
+};
+
+// Sum over the five rows of a window that are dealt out over LPT lanes (lane q
+// holds rows q, q + LPT, ..: v[0], v[1], ..; zero beyond the fifth), always as
+// ((row 0 + row 1) + (row 2 + row 3)) + row 4, so that a fit's value does not
+// depend on the lanes given to it.  gm: the lanes of the group.
+template <int LPT, class T> __device__ __forceinline__ T row_sum(unsigned gm, const T (&v)[(4 + LPT) / LPT]) {
+    if constexpr (LPT == 1) {
+        return ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
+    } else {
+        const int first = threadIdx.x & 31 & ~(LPT - 1);
+        T t = v[0] + __shfl_xor_sync(gm, v[0], 1);
+        if constexpr (LPT == 2) return (t + (v[1] + __shfl_xor_sync(gm, v[1], 1))) + __shfl_sync(gm, v[2], first);
+        else {
+            t += __shfl_xor_sync(gm, t, 2);
+            if constexpr (LPT == 4) return t + __shfl_sync(gm, v[1], first);
+            else return t + __shfl_xor_sync(gm, t, 4);
+        }
+    }
+}
+
+// One coefficient of a fit without directional weights, from the whole numbers
+// c13, c23 and c33: 16 2^-(|dx| + |dy|) (c33 + dy c23 + dx c13), below 2^20 and
+// exact either way.  FP32: in floats (converting each costs four issue slots);
+// FP64: in integers, widened.
+template <class R> struct FitCoef;
+template <> struct FitCoef<float> {
+    float c13, c23, c33;
+    __device__ __forceinline__ FitCoef(int a, int b, int c) : c13((float)a), c23((float)b), c33((float)c) {}
+    __device__ __forceinline__ float row(int dy) const { return (float)(4 >> (dy < 0 ? -dy : dy)) * fmaf((float)dy, c23, c33); }
+    __device__ __forceinline__ float col(int dy) const { return (float)(4 >> (dy < 0 ? -dy : dy)) * c13; }
+    static __device__ __forceinline__ float at(float row, float col, int dx) {
+        return (float)(4 >> (dx < 0 ? -dx : dx)) * fmaf((float)dx, col, row);
+    }
+};
+template <> struct FitCoef<double> {
+    int c13, c23, c33;
+    __device__ __forceinline__ FitCoef(int a, int b, int c) : c13(a), c23(b), c33(c) {}
+    __device__ __forceinline__ int row(int dy) const { return (4 >> (dy < 0 ? -dy : dy)) * (c33 + dy * c23); }
+    __device__ __forceinline__ int col(int dy) const { return (4 >> (dy < 0 ? -dy : dy)) * c13; }
+    static __device__ __forceinline__ double at(int row, int col, int dx) {
+        return whole<double>((4 >> (dx < 0 ? -dx : dx)) * (row + dx * col));
+    }
+};
+
+// The fitted value at one target (Sec. 3.2, steps (i)-(iii)) by a group of LPT
+// lanes, the rows of its 5x5 window dealt out over them; XY: twice that,
+// one half for each coordinate (FP64).  value = ref + sum_k w_k (c13 dx + c23 dy
+// + c33) (X_k - ref) / det with the cofactors of M's last row, over the valid
+// nodes (bits m).  The fit is of differences from the value at the target's
+// 4-neighbour in the layer before (a valid node by construction), which keeps
+// the sums small.  Without directional weights (use_n: layers 1 and 2, weights
+// 2^-(|dx|+|dy|) max(0, d.n) / |d|, (gx, gy) along n; a common factor of the weights
+// drops out, so n is not normalised; wd: 2^-(|dx|+|dy|) / |d|) the cofactors come from the validity bits
+// alone, exactly.  A layer takes as long as this chain, so its loads do not wait
+// for one another: every node of a row is loaded, one that does not count from
+// the reference's address (its difference is then zero).
+// False if the window does not define the plane.  The group's lanes call together.
+template <class R, bool CL, int LPT, bool XY>
+__device__ __forceinline__ bool fit_window(const RefVals<R, CL> &V, const int *lut, const R *wd, unsigned m, int x, int y,
+                                           bool use_n, R gx, R gy, R &ox, R &oy) {
+    const int q = threadIdx.x & (LPT - 1), c = XY ? (threadIdx.x / LPT) & 1 : 0;
+    constexpr int G = XY ? 2 * LPT : LPT;
+    const unsigned gm = (0xffffffffu >> (32 - G)) << (threadIdx.x & 31 & ~(G - 1));
+    const int t = V.at(x, y);
+    const int kref = (m >> 11) & 1u ? t - 1 : ((m >> 13) & 1u ? t + 1 : ((m >> 7) & 1u ? t - V.stride : t + V.stride));
+    constexpr int NR = (4 + LPT) / LPT;  // rows per lane
+    R xref, yref, ax[NR], ay[NR], det;
+    if constexpr (XY) xref = V.get(kref, c);
+    else V.get2(kref, xref, yref);
+    bool good;
+    auto add = [&](int i, bool on, int k, R g) {
+        if constexpr (XY) {
+            ax[i] = fma_rn<R>(g, V.get(on ? k : kref, c) - xref, ax[i]);
+        } else {
+            R vx, vy;
+            V.get2_if(on, k, kref, xref, yref, vx, vy);
+            ax[i] = fma_rn<R>(g, vx - xref, ax[i]);
+            ay[i] = fma_rn<R>(g, vy - yref, ay[i]);
+        }
+    };
+    int i13, i23, i33;
+#pragma unroll
+    for (int i = 0; i < NR; i++) ax[i] = ay[i] = R(0);
+    if (!use_n) {
+        const int idet = window_moments(lut, m, i13, i23, i33);
+        good = idet != 0;
+        det = whole<R>(idet);
+        const FitCoef<R> fc(i13, i23, i33);
+#pragma unroll
+        for (int i = 0; i < NR; i++) {
+            const int d = i * LPT + q, dy = d - 2;  // d >= 5: no row
+            const unsigned r = d < 5 ? (m >> (5 * d)) & 31u : 0u;
+            if (!CL && r == 0u) continue;
+            const int k = t + dy * V.stride;
+            const auto row = fc.row(dy), col = fc.col(dy);
+#pragma unroll
+            for (int dx = -2; dx <= 2; dx++) add(i, (r >> (dx + 2)) & 1u, k + dx, FitCoef<R>::at(row, col, dx));
+        }
+    } else {
+        const float gxf = (float)gx, gyf = (float)gy, lim = (float)COS_TIE * sqrtf(gxf * gxf + gyf * gyf);
+        R s0[NR], s1[NR], s2[NR];
+        unsigned pos = 0;
+#pragma unroll
+        for (int i = 0; i < NR; i++) {
+            const int d = i * LPT + q, dy = d - 2;
+            const unsigned r = d < 5 ? (m >> (5 * d)) & 31u : 0u;
+            const R *w = wd + 5 * (d < 5 ? d : 0);
+            const R dygy = R(dy) * gy;
+            s0[i] = s1[i] = s2[i] = R(0);
+#pragma unroll
+            for (int dx = -2; dx <= 2; dx++) {
+                // d.n times |d| |n|, d = target - node; a cosine up to COS_TIE counts as zero
+                const R dn = -fma_rn<R>(R(dx), gx, dygy);
+                const bool p = ((r >> (dx + 2)) & 1u) && above(dn, lim * sqrtf((float)(dx * dx) + (float)(dy * dy)));
+                const R wt = p ? dn * w[dx + 2] : R(0);
+                pos |= p ? 1u << (5 * d + dx + 2) : 0u;
+                s0[i] += wt;
+                s1[i] = fma_rn<R>(R(dx), wt, s1[i]);
+                s2[i] = fma_rn<R>(R(dx * dx), wt, s2[i]);
+            }
+        }
+        R y0[NR], y1[NR], y2[NR];  // times dy (and dy^2): exact
+#pragma unroll
+        for (int i = 0; i < NR; i++) {
+            const R dy = R(i * LPT + q - 2);
+            y1[i] = dy * s1[i]; y0[i] = dy * s0[i]; y2[i] = dy * y0[i];
+        }
+        const R a = row_sum<LPT>(gm, s2), b = row_sum<LPT>(gm, y1), cc = row_sum<LPT>(gm, s1);
+        const R d_ = row_sum<LPT>(gm, y2), e = row_sum<LPT>(gm, y0), fw = row_sum<LPT>(gm, s0);
+#pragma unroll
+        for (int d = 1; d < LPT; d <<= 1) pos |= __shfl_xor_sync(gm, pos, d);
+        const R c13 = fma_rn<R>(b, e, -mul_rn<R>(cc, d_)), c23 = fma_rn<R>(b, cc, -mul_rn<R>(a, e)),
+                c33 = fma_rn<R>(a, d_, -mul_rn<R>(b, b));
+        det = fma_rn<R>(cc, c13, fma_rn<R>(e, c23, mul_rn<R>(fw, c33)));
+        good = window_moments(lut, pos, i13, i23, i33) != 0 && det != R(0);
+#pragma unroll
+        for (int i = 0; i < NR; i++) {
+            const int d = i * LPT + q, dy = d - 2;
+            const unsigned r = d < 5 ? (pos >> (5 * d)) & 31u : 0u;
+            if (!CL && r == 0u) continue;
+            const int k = t + dy * V.stride;
+            const R *w = wd + 5 * (d < 5 ? d : 0);
+            const R base = fma_rn<R>(R(dy), c23, c33), dygy = R(dy) * gy;
+#pragma unroll
+            for (int dx = -2; dx <= 2; dx++)
+                add(i, (r >> (dx + 2)) & 1u, k + dx,
+                    mul_rn<R>(mul_rn<R>(-fma_rn<R>(R(dx), gx, dygy), w[dx + 2]), fma_rn<R>(R(dx), c13, base)));
+        }
+    }
+    const R sx = row_sum<LPT>(gm, ax);
+    if constexpr (XY) {
+        const R v = xref + sx / det, w = __shfl_xor_sync(gm, v, LPT);
+        ox = c ? w : v;
+        oy = c ? v : w;
+    } else {
+        const R sy = row_sum<LPT>(gm, ay);
+        ox = xref + sx / det;
+        oy = yref + sy / det;
+    }
+    return good;
+}
 
 // R^2 as an unevaluated sum hi + lo in precision R (from the host-side split).
 template <class R>
@@ -1029,19 +1182,94 @@ __device__ __forceinline__ bool list_layers(const signed char *lab, int T, int x
     return listed;
 }
 
+// Rows of a solid's band over the CTAs of a cluster (one CTA: all of them).
+struct Strips {
+    int y0, y1, lnc, NL;  // band rows; log2 of the CTAs; layers
+    __device__ __forceinline__ int first(int k) const { return y0 + (((y1 - y0 + 1) * k) >> lnc); }
+    __device__ __forceinline__ int owner(int y) const { return (((y - y0 + 1) << lnc) - 1) / (y1 - y0 + 1); }
+    // first row of CTA k's sets: one before the farthest that its strip is reached from
+    __device__ __forceinline__ int set_first(int k) const { return max(first(k) - NL - 2, y0 - 2); }
+};
+
+// The fit with a window grown beyond 5x5 (Sec. 3.2's widening, r = 3 .. rmax):
+// rare, so every sum is formed anew, and in a cluster every row is read from
+// the CTA that holds it.  False if no window up to rmax defines the plane.
+template <class R, bool CL>
+__device__ __noinline__ bool fit_grown(const RefVals<R, CL> &V, const RowMask &v, const Strips &st, int x0, int T, int x,
+                                       int y, int rmax, bool use_n, R gx, R gy, R &ox, R &oy) {
+    auto valid = [&](int px, int py) {
+        if (px < 0 || px >= T || py < st.y0 || py > st.y1) return false;
+        if constexpr (CL) {
+            const int o = st.owner(py);
+            return ((cluster_ld(v.p + (py - st.set_first(o)) * v.rw + ((px + 32) >> 5), o) >> (px & 31)) & 1u) != 0u;
+        } else {
+            return v.bit(px, py);
+        }
+    };
+    auto value = [&](int px, int py, R &vx, R &vy) {
+        if constexpr (CL) {
+            const int o = st.owner(py);
+            cluster_ld2(V.tile + (py - st.first(o) + 2) * V.stride + px - x0, o, vx, vy);
+        } else {
+            V.get2(V.at(px, py), vx, vy);
+        }
+    };
+    const R nn = rsqrt_<R>(gx * gx + gy * gy);
+    R xref = R(0), yref = R(0);
+    if (valid(x - 1, y)) value(x - 1, y, xref, yref);
+    else if (valid(x + 1, y)) value(x + 1, y, xref, yref);
+    else if (valid(x, y - 1)) value(x, y - 1, xref, yref);
+    else if (valid(x, y + 1)) value(x, y + 1, xref, yref);
+    for (int r = 3; r <= rmax; r++) {
+        int n = 0, sx = 0, sy = 0, sxx = 0, syy = 0, sxy = 0;
+        R a = 0, b = 0, c = 0, d = 0, e = 0, fw = 0, bx0 = 0, bx1 = 0, bx2 = 0, by0 = 0, by1 = 0, by2 = 0;
+        for (int dy = -r; dy <= r; dy++)
+            for (int dx = -r; dx <= r; dx++) {
+                if (!valid(x + dx, y + dy)) continue;
+                R wt = pow2neg<R>(abs(dx) + abs(dy));
+                if (use_n) {
+                    const R dn = (R(-dx) * gx + R(-dy) * gy) / nn * rinv_tab<R>(dx, dy);
+                    wt = dn > R(COS_TIE) ? dn * wt : R(0);
+                }
+                if (!(wt > R(0))) continue;
+                n++; sx += dx; sy += dy; sxx += dx * dx; syy += dy * dy; sxy += dx * dy;
+                R Xv, Yv;
+                value(x + dx, y + dy, Xv, Yv);
+                Xv -= xref; Yv -= yref;
+                const R wx = wt * R(dx), wy = wt * R(dy);
+                a += wx * R(dx); b += wx * R(dy); c += wx; d += wy * R(dy); e += wy; fw += wt;
+                bx0 += wx * Xv; bx1 += wy * Xv; bx2 += wt * Xv;
+                by0 += wx * Yv; by1 += wy * Yv; by2 += wt * Yv;
+            }
+        if (n < 3) continue;
+        const long long g1 = (long long)n * sxx - (long long)sx * sx;
+        const long long g2 = (long long)n * syy - (long long)sy * sy;
+        const long long g3 = (long long)n * sxy - (long long)sx * sy;
+        if (g1 * g2 - g3 * g3 == 0) continue;  // positive-weight nodes on one line
+        const R c13 = b * e - c * d, c23 = b * c - a * e, c33 = a * d - b * b;
+        const R det = c * c13 + e * c23 + fw * c33;
+        if (!(det != R(0))) continue;
+        ox = xref + (c13 * bx0 + c23 * bx1 + c33 * bx2) / det;
+        oy = yref + (c13 * by0 + c23 * by1 + c33 * by2) / det;
+        return true;
+    }
+    ox = oy = nanv<R>();
+    return false;
+}
+
 // One node of pass 0 (advection): its stored state and the LB state at it,
 // gathered with independent loads (the rest base is loaded whatever the
 // registry count and selected after).
 template <class R>
 struct P0Node {
     int ix, iy, cnt;
-    R ex, ey, phi, cx, cy, pv;
+    R ex, ey, cx, cy, pv;
     R f[9];
 };
 
 template <class R, class S>
-__device__ __forceinline__ void p0_gather(const SimParams &sp, const RmtArgs<R, S> &a, const R *Xi, const R *Yi,
-                                          const R *Pi, int T, int2 oo, int shx, int shy, int entry, P0Node<R> &nd) {
+__device__ __forceinline__ void p0_gather(const SimParams &sp, const RmtArgs<R, S> &a, const R *Xi, const R *Yi, int T,
+                                          int2 oo, int shx, int shy, int entry, P0Node<R> &nd) {
     nd.ix = entry & 0xffff;
     nd.iy = entry >> 16;
     const int k = nd.iy * T + nd.ix;
@@ -1050,7 +1278,6 @@ __device__ __forceinline__ void p0_gather(const SimParams &sp, const RmtArgs<R, 
     const int tile = (j >> sp.ly) * sp.ntx + (i >> sp.lx);
     nd.ex = Xi[k];
     nd.ey = Yi[k];
-    nd.phi = Pi[k];
 #pragma unroll
     for (int q = 0; q < 9; q++) nd.f[q] = ldS<S, R>(a.f + q * sp.P + c, sp, q);
     nd.cnt = a.reg_prev[tile];
@@ -1063,13 +1290,20 @@ __device__ __forceinline__ void p0_gather(const SimParams &sp, const RmtArgs<R, 
     nd.cy = po[POOL_CY];
 }
 
-// The rest of pass 0 for a gathered node of the blur zone or the solid:
-// statistics, and for a solid node the upwind advection (Eqs. 3_1_refmap_adv,
-// 3_1_eno) into the output tile.
+// Velocities in the solid's mean velocity: whole multiples of 2^-22 (its only
+// use is the next frame's offset), so that the sums do not depend on how
+// the nodes are spread over threads and CTAs.
+constexpr float VEL_SCALE = 4194304.0f;
+__device__ __forceinline__ int vel_fixed(float u) { return __float2int_rn(u * VEL_SCALE); }
+__device__ __forceinline__ int vel_fixed(double u) { return __float2int_rn((float)u * VEL_SCALE); }
+
+// The rest of pass 0 for a gathered node of the solid: the upwind advection
+// (Eqs. 3_1_refmap_adv, 3_1_eno) into the output tile, its bit in the solid set
+// and its part of the mean velocity (acc: nodes, u, v).
 template <class R, class S>
 __device__ __forceinline__ void p0_finish(const SimParams &sp, const RmtArgs<R, S> &a, const P0Node<R> &nd,
-                                          const R *Xi, const R *Yi, R *Xo, R *Yo, signed char *lab, int T,
-                                          const Frame &fi, int2 oo, int shx, int shy, R ddx, R ddy, R eps, R (&stl)[6],
+                                          const R *Xi, const R *Yi, R *Xo, R *Yo, const RowMask &ms, int T,
+                                          const Frame &fi, int2 oo, int shx, int shy, R ddx, R ddy, int (&acc)[3],
                                           int (&sb)[4]) {
     const int ix = nd.ix, iy = nd.iy, lx = ix - shx, ly = iy - shy;
     R rho, u, v, cx = nd.cx, cy = nd.cy;
@@ -1084,10 +1318,7 @@ __device__ __forceinline__ void p0_finish(const SimParams &sp, const RmtArgs<R, 
         free_carry<R>(sp, ldC<S, R>(a.carry + c, sp), Fx, Fy, cx, cy);
     }
     moments_from<R>(sp, nd.f, nd.cnt > 0 ? nd.pv : R(0), cx, cy, rho, u, v);
-    const R lam = R(1) - heaviside<R>(nd.phi, eps);
-    stl[0] += lam; stl[1] += lam * R(lx); stl[2] += lam * R(ly);
-    stl[3] += lam * rho; stl[4] += lam * rho * u; stl[5] += lam * rho * v;
-    if (!(nd.phi < -R(PHI_TIE))) return;
+    acc[0]++; acc[1] += vel_fixed(u); acc[2] += vel_fixed(v);
     const int sx = (u >= R(0)) ? -1 : 1, sy = (v >= R(0)) ? -1 : 1;
     const int x2 = ix + 2 * sx, y2 = iy + 2 * sy;
     if (x2 < fi.bx0 || x2 > fi.bx1 || y2 < fi.by0 || y2 > fi.by1) {
@@ -1131,36 +1362,68 @@ __device__ __forceinline__ void p0_finish(const SimParams &sp, const RmtArgs<R, 
         Xo[t] = ex - (u - ddx) - (u * dXdx + v * dXdy);
         Yo[t] = ey - (v - ddy) - (u * dYdx + v * dYdy);
     }
-    lab[t] = 0;
+    atomicOr(ms.word(lx, ly), 1u << (lx & 31));
     sb[0] = min(sb[0], lx); sb[1] = max(sb[1], lx); sb[2] = min(sb[2], ly); sb[3] = max(sb[3], ly);
 }
 
-template <class R, class S>
-__device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int s) {
+// Shift of eta between two frames, (o_out - o_in) - (off_out - off_in): whole
+// numbers and multiples of 2^-14 below 2^9, so exact in FP32 as in FP64 (every
+// thread forms it; GB300's FP64 pipe takes 16 cycles per warp instruction).
+template <class R> __device__ __forceinline__ R frame_shift(int sh, float off_out, float off_in) {
+    return R(sh) - (R(off_out) - R(off_in));
+}
+
+// K2 for solid s.  CL: the solid is spread over the nc CTAs of a cluster, CTA
+// `rank` taking a strip of rows in each phase; else one CTA (rank 0 of 1).
+//   0. advection of the solid set S;
+//   1. layers 1..NL: the set of nodes within l 4-neighbour dilation steps of S,
+//      dilated bitwise one layer ahead of the fits; a layer's new nodes are
+//      listed and fitted from the sets before it, one barrier per layer;
+//   2. relabel, next frame, tile registry.
+// A cluster keeps the strips' map in shared memory from pass 0 to the relabel,
+// with two halo rows on either side that the neighbours write into as they fit
+// them, so that a layer costs a cluster barrier and no trip through L2; each
+// CTA dilates the rows that its strip can still be reached from.
+// Bound by the latency of this chain (HBM and every pipe idle but FP64's in FP64).
+// A solid of radius 16 takes, in cycles with four such CTAs on an SM: advection 44 K,
+// sets 4 K, layers 1-2 23 K, layers 3-11 48 K, relabel 31 K, frame and registry 6 K
+// (54, 24, 20, 53, 32, 12 K with byte labels, an L1 distance transform and a
+// branch per window node, and 7 K instead of 4 K before pass 0, most of it FP64
+// in every thread).  Per launch: 4096^2 with 1024 disks 198 -> 164 us; 1501 x 1203 with 110 88 -> 75;
+// 96 cavities in one batch 213 -> 175.  In a cluster of 16 CTAs: one disk of radius
+// 128 1529 -> 66 us (its layers no longer fitted the list and scanned the tile), of
+// 64 192 -> 51, of 16 57 -> 40 (cluster of 8), 24 of 10-20 58 -> 42; in FP64, whose pipe takes a warp
+// instruction per scheduler in 64 cycles, 64 disks 352 -> 156, one 204 -> 73.
+template <class R, class S, bool CL>
+__device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int s, const int rank, const int nc) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int lcnt[24];  // per layer: node count, then the next free list slot
-    __shared__ int loff[24];  // per layer: first list slot (layer l at loff[l] .. loff[l + 1])
-    __shared__ int bb[12];    // S bbox (0-3), band bbox (4-7), blur-zone bbox (8-11)
-    __shared__ double red[32 * 6];
+    __shared__ int lcnt[24];   // targets listed per layer
+    __shared__ int bb[16];     // this CTA's boxes: S (0-3), band (4-7), blur zone (8-11); S nodes and velocity sums (12-14 hi/lo)
+    __shared__ int sbb[4];     // box of S over the cluster
+    __shared__ int lut[32];
+    __shared__ R wd[25];
+    __shared__ unsigned long long vsum[2];
     __syncthreads();  // the shared state of a previous solid is no longer read
-    const SolidDesc sd = a.solids[s];
-    const int T = sd.T, TT = T * T;
-    const int lane = threadIdx.x & 31;
-    signed char *lab = reinterpret_cast<signed char *>(smem);        // -1 free, 0 solid, l layer
-    // after the labels, the rest of the launch's dynamic shared memory holds
-    // ints: pass 0's per-warp node lists, then the layer lists
-    int *lists = reinterpret_cast<int *>(smem + ((TT + 15) & ~15));
+    const SolidDesc &sd = a.solids[s];
+    const int NL = sp.n_layers;
+    const int T = sd.T, TT = T * T, rw = mask_row_words(T), mw = mask_words(T, nc, NL);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    unsigned *masks = reinterpret_cast<unsigned *>(smem);
+    const int m0w = CL ? strip_mask_words(T, nc) : 0;
+    int *lists = reinterpret_cast<int *>(masks + RMT_MASKS * mw + m0w);
     unsigned dsm;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
-    const int list_cap = ((int)dsm - ((TT + 15) & ~15)) >> 2;
+    const int list_ints = CL ? RMT_WIDE_LIST_BYTES / 4 : ((int)dsm >> 2) - RMT_MASKS * mw, layer_cap = list_ints >> 1;
+    auto solid_sync = [&]() {
+        if constexpr (CL) cluster_sync();
+        else __syncthreads();
+    };
     const Frame fo = a.frame_out[s];
     const Frame fi = a.init ? fo : a.frame_in[s];
     const int2 oo = make_int2(fo.ox, fo.oy);
     const int shx = fo.ox - fi.ox, shy = fo.oy - fi.oy;  // same node: local index shifts by this
-    // eta_out = eta_in + (d_out - d_in); exact (integer part plus multiples of 2^-14)
-    const R ddx = R((double)shx - ((double)fo.offx - (double)fi.offx));
-    const R ddy = R((double)shy - ((double)fo.offy - (double)fi.offy));
-    const Rsq<R> rq(sd);
+    // eta_out = eta_in + (d_out - d_in)
+    const R ddx = frame_shift<R>(shx, fo.offx, fi.offx), ddy = frame_shift<R>(shy, fo.offy, fi.offy);
     R *Xo = a.xi_out + sd.off;
     R *Yo = Xo + TT;
     R *Po = Yo + TT;  // phi^{n+1} of the tile nodes (third plane), written by the relabel
@@ -1168,237 +1431,448 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     const R *Yi = a.init ? nullptr : Xi + TT;
     const R *Pi = a.init ? nullptr : Yi + TT;  // phi^n, stored by the previous step's relabel
     const R eps = pick<R>(sp.eps, sp.eps_f);
-    if (threadIdx.x < 12) bb[threadIdx.x] = (threadIdx.x & 1) ? -(1 << 29) : (1 << 29);
-    if (threadIdx.x < 24) lcnt[threadIdx.x] = 0;
-    for (int k = threadIdx.x; k < (TT + 15) >> 4; k += blockDim.x)
-        reinterpret_cast<int4 *>(lab)[k] = make_int4(-1, -1, -1, -1);
-    R stl[6] = {0, 0, 0, 0, 0, 0};  // sum lambda, lambda lx, lambda ly, lambda rho, lambda rho u, lambda rho v
+    if (tid < 12) bb[tid] = (tid & 1) ? -(1 << 29) : (1 << 29);
+    else if (tid < 16) bb[tid] = 0;
+    if (tid < 24) lcnt[tid] = 0;
+    if (tid < 2) vsum[tid] = 0ull;
+    if (tid < 32) lut[tid] = row_moments(tid);
+    if (tid >= 32 && tid < 57) {
+        const int dx = (tid - 32) % 5 - 2, dy = (tid - 32) / 5 - 2;
+        wd[tid - 32] = pow2neg<R>(abs(dx) + abs(dy)) * rinv_tab<R>(dx, dy);
+    }
+    for (int k = tid; k < (RMT_MASKS * mw + m0w) / 4; k += blockDim.x) reinterpret_cast<int4 *>(masks)[k] = make_int4(0, 0, 0, 0);
+    int acc[3] = {0, 0, 0};
     int sb[4] = {1 << 29, -(1 << 29), 1 << 29, -(1 << 29)};
     __syncthreads();
 
     // Pass 0: the advected set S = {domain nodes with phi^n < 0}, Eqs. 3_1_refmap_adv / 3_1_eno,
-    // over the input tile's box (the whole tile at initialisation).
+    // over this CTA's rows of the input tile's box (the whole tile at initialisation).
     const int ib0 = a.init ? 0 : fi.bx0, ib1 = a.init ? T - 1 : fi.bx1;
     const int jb0 = a.init ? 0 : fi.by0, jb1 = a.init ? T - 1 : fi.by1;
-    const int bw = ib1 - ib0 + 1, bn = (ib1 >= ib0 && jb1 >= jb0) ? bw * (jb1 - jb0 + 1) : 0;
+    const int ih = (ib1 >= ib0 && jb1 >= jb0) ? jb1 - jb0 + 1 : 0, bw = ih ? ib1 - ib0 + 1 : 1;
+    const int jr0 = jb0 + (CL ? ih * rank / nc : 0), jr1 = jb0 + (CL ? ih * (rank + 1) / nc : ih);
+    const int bn = bw * (jr1 - jr0);
+    // the set S as this pass finds it: rows of the output tile (CL: the strip's alone)
+    const RowMask mP = {CL ? masks + RMT_MASKS * mw : masks, rw, CL ? jr0 - shy : -2};
     if (a.init) {
+        const Rsq<R> rq(sd);
         BoxWalk wk(bw);
-        for (int kk = threadIdx.x; kk < bn; kk += blockDim.x, wk.next()) {
-            const int ix = ib0 + wk.c, iy = jb0 + wk.r;  // input-tile coordinates
-            const int lx = ix - shx, ly = iy - shy;      // output-tile coordinates
-            const int gx = oo.x + lx, gy = oo.y + ly;
+        for (int kk = tid; kk < bn; kk += blockDim.x, wk.next()) {
+            const int lx = ib0 + wk.c, ly = jr0 + wk.r;  // the input frame is the output frame
             // xi = x: eta = d of the initial frame
             const R e0x = R(frame_d(fo, sd.xc, true)), e0y = R(frame_d(fo, sd.yc, false));
-            if (domain_cell(sp, gx, gy) && phi_eta(e0x, e0y, lx, ly, fo, rq) < -R(PHI_TIE)) {
+            if (domain_cell(sp, oo.x + lx, oo.y + ly) && phi_eta(e0x, e0y, lx, ly, fo, rq) < -R(PHI_TIE)) {
                 const int t = ly * T + lx;
-                Xo[t] = e0x; Yo[t] = e0y; lab[t] = 0;
+                Xo[t] = e0x; Yo[t] = e0y;
+                atomicOr(mP.word(lx, ly), 1u << (lx & 31));
                 sb[0] = min(sb[0], lx); sb[1] = max(sb[1], lx); sb[2] = min(sb[2], ly); sb[3] = max(sb[3], ly);
             }
         }
     } else {
-        // (a) each warp lists, in box order, the nodes of its share of the box
-        // (items threadIdx.x + m blockDim.x) that lie in the blur zone or the
-        // solid, in its own segment of the (not yet used) layer lists; (b) it
-        // advances them two per lane at a time, every load of both nodes issued
-        // before the arithmetic -- at the end of its share, or earlier whenever
-        // the segment could overflow, after which the listing goes on.
-        const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5;
-        const int seg_cap = list_cap / nw;
+        // (a) each warp lists, in box order, the solid's nodes of its share of the
+        // box (items tid + m blockDim.x) in its own segment of the (not yet used)
+        // lists; (b) it advances them two per lane at a time, every load of both
+        // nodes issued before the arithmetic -- at the end of its share, or earlier
+        // whenever the segment could overflow, after which the listing goes on.
+        const int seg_cap = list_ints / nw;  // >= 128
         int *seg = lists + warp * seg_cap;
-        if (seg_cap >= 128) {
-            // (four of a thread's items at a time: their phi loads first, then the
-            // ballots in item order, which add at most 128 entries)
-            int base = 0;
-            do {
-                int nseg = 0;
-                for (; base < bn && nseg <= seg_cap - 128; base += 4 * blockDim.x) {
-                    R ph[4];
-                    int ent[4];
+        // (four of a thread's items at a time: their phi loads first, then the
+        // ballots in item order, which add at most 128 entries)
+        BoxWalk wk(bw);
+        int base = 0;
+        do {
+            int nseg = 0;
+            for (; base < bn && nseg <= seg_cap - 128; base += 4 * blockDim.x) {
+                R ph[4];
+                int ent[4];
 #pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        const int kk = base + q * (int)blockDim.x + (int)threadIdx.x;
-                        const int ix = ib0 + kk % bw, iy = jb0 + kk / bw;
-                        ent[q] = ix | (iy << 16);
-                        ph[q] = kk < bn ? Pi[iy * T + ix] : eps;
-                    }
+                for (int q = 0; q < 4; q++) {
+                    const int ix = ib0 + wk.c, iy = jr0 + wk.r;
+                    ent[q] = ix | (iy << 16);
+                    ph[q] = base + q * (int)blockDim.x + tid < bn ? Pi[iy * T + ix] : R(0);
+                    wk.next();
+                }
 #pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        bool hit = false;
-                        if (ph[q] < eps) {
-                            const int lx = (ent[q] & 0xffff) - shx, ly = (ent[q] >> 16) - shy;
-                            if (domain_cell(sp, oo.x + lx, oo.y + ly)) {
-                                if (lx < 0 || ly < 0 || lx >= T || ly >= T) atomicOr(a.err, ERR_TILE_OVERFLOW);
-                                else hit = true;
-                            }
+                for (int q = 0; q < 4; q++) {
+                    bool hit = false;
+                    if (ph[q] < -R(PHI_TIE)) {
+                        const int lx = (ent[q] & 0xffff) - shx, ly = (ent[q] >> 16) - shy;
+                        if (domain_cell(sp, oo.x + lx, oo.y + ly)) {
+                            if (lx < 0 || ly < 0 || lx >= T || ly >= T) atomicOr(a.err, ERR_TILE_OVERFLOW);
+                            else hit = true;
                         }
-                        const unsigned m = __ballot_sync(0xffffffffu, hit);
-                        if (hit) seg[nseg + __popc(m & ((1u << lane) - 1u))] = ent[q];
-                        nseg += __popc(m);
                     }
+                    const unsigned m = __ballot_sync(0xffffffffu, hit);
+                    if (hit) seg[nseg + __popc(m & ((1u << lane) - 1u))] = ent[q];
+                    nseg += __popc(m);
                 }
-                __syncwarp();
-                for (int e = lane; e < nseg; e += 64) {
-                    const bool two = e + 32 < nseg;
-                    P0Node<R> n1, n2;
-                    p0_gather<R, S>(sp, a, Xi, Yi, Pi, T, oo, shx, shy, seg[e], n1);
-                    p0_gather<R, S>(sp, a, Xi, Yi, Pi, T, oo, shx, shy, seg[two ? e + 32 : e], n2);
-                    p0_finish<R, S>(sp, a, n1, Xi, Yi, Xo, Yo, lab, T, fi, oo, shx, shy, ddx, ddy, eps, stl, sb);
-                    if (two)
-                        p0_finish<R, S>(sp, a, n2, Xi, Yi, Xo, Yo, lab, T, fi, oo, shx, shy, ddx, ddy, eps, stl, sb);
-                }
-                __syncwarp();
-            } while (base < bn);
-        } else {
-            // segments too small to list four ballots: each thread walks its share
-            BoxWalk wk2(bw);
-            for (int kk = threadIdx.x; kk < bn; kk += blockDim.x, wk2.next()) {
-                const int ix = ib0 + wk2.c, iy = jb0 + wk2.r;
-                const int lx = ix - shx, ly = iy - shy;
-                if (!(Pi[iy * T + ix] < eps) || !domain_cell(sp, oo.x + lx, oo.y + ly)) continue;
-                if (lx < 0 || ly < 0 || lx >= T || ly >= T) {
-                    atomicOr(a.err, ERR_TILE_OVERFLOW);
-                    continue;
-                }
-                P0Node<R> nd;
-                p0_gather<R, S>(sp, a, Xi, Yi, Pi, T, oo, shx, shy, ix | (iy << 16), nd);
-                p0_finish<R, S>(sp, a, nd, Xi, Yi, Xo, Yo, lab, T, fi, oo, shx, shy, ddx, ddy, eps, stl, sb);
             }
-        }
+            __syncwarp();
+            for (int e = lane; e < nseg; e += 64) {
+                const bool two = e + 32 < nseg;
+                P0Node<R> n1, n2;
+                p0_gather<R, S>(sp, a, Xi, Yi, T, oo, shx, shy, seg[e], n1);
+                p0_gather<R, S>(sp, a, Xi, Yi, T, oo, shx, shy, seg[two ? e + 32 : e], n2);
+                p0_finish<R, S>(sp, a, n1, Xi, Yi, Xo, Yo, mP, T, fi, oo, shx, shy, ddx, ddy, acc, sb);
+                if (two) p0_finish<R, S>(sp, a, n2, Xi, Yi, Xo, Yo, mP, T, fi, oo, shx, shy, ddx, ddy, acc, sb);
+            }
+            __syncwarp();
+        } while (base < bn);
     }
     for (int k = 0; k < 4; k++) warp_minmax(sb[k], (k & 1) == 0);
     if (lane == 0) {
         atomicMin(&bb[0], sb[0]); atomicMax(&bb[1], sb[1]); atomicMin(&bb[2], sb[2]); atomicMax(&bb[3], sb[3]);
     }
-    __syncthreads();
+    // the mean velocity's sums: 32-bit per thread (below 2^31: 0.3 x 2^22 x 784 nodes), 64-bit beyond
+    acc[0] = __reduce_add_sync(0xffffffffu, acc[0]);
+#pragma unroll
+    for (int k = 1; k < 3; k++) {
+        const int lo = __reduce_add_sync(0xffffffffu, acc[k] & 0xffff), hi = __reduce_add_sync(0xffffffffu, acc[k] >> 16);
+        if (lane == 0) atomicAdd(&vsum[k - 1], (unsigned long long)((long long)hi * 65536 + lo));
+    }
+    if (lane == 0) atomicAdd(&bb[12], acc[0]);
+    solid_sync();
 
-    // Layers 1..n_layers around S (Sec. 3.2; 11 layers, Sec. 4), labelled at once
-    // (label_layers_l1), then listed by a counting pass and fitted one after
-    // another, each from S and the layers before it.
-    const int sx0 = bb[0], sx1 = bb[1], sy0 = bb[2], sy1 = bb[3];
-    if (sx0 > sx1) {
-        if (threadIdx.x == 0) atomicOr(a.err, ERR_TILE_OVERFLOW);  // the solid vanished
+    // The box of S over the cluster.
+    if constexpr (CL) {
+        if (warp == 0) {
+            for (int k = 0; k < 4; k++) {
+                int v = (int)cluster_ld(&bb[k], lane < nc ? lane : rank);
+                warp_minmax(v, (k & 1) == 0);
+                if (lane == 0) sbb[k] = v;
+            }
+        }
+    } else if (tid < 4) {
+        sbb[tid] = bb[tid];
     }
-    const int NL = sp.n_layers;
-    bool listed = false;  // every layer's nodes are in the lists (else each layer scans the tile)
-    if (sx0 <= sx1) {
-        const int x0 = max(sx0 - NL, 0), x1 = min(sx1 + NL, T - 1), y0 = max(sy0 - NL, 0), y1 = min(sy1 + NL, T - 1);
-        label_layers_l1(sp, lab, T, sx0, sx1, sy0, sy1, oo, NL, lcnt);
-        __syncthreads();
-        listed = list_layers(lab, T, x0, x1, y0, y1, NL, lcnt, loff, lists, list_cap);
-    }
-    for (int l = 1; l <= NL && sx0 <= sx1; l++) {
-        const int nitems = listed ? loff[l + 1] - loff[l] : TT;
-        for (int k = threadIdx.x; k < nitems; k += blockDim.x) {
-            int lx, ly;
-            if (listed) {
-                const int e = lists[loff[l] + k];
-                lx = e & 0xffff; ly = e >> 16;
-            } else {  // too many band nodes for the lists: scan the tile
-                lx = k % T; ly = k / T;
-                if (lab[k] != l) continue;
-            }
-            const int t = ly * T + lx;
-            if (a.init) {  // xi = x on the band at initialisation
-                Xo[t] = R(frame_d(fo, sd.xc, true));
-                Yo[t] = R(frame_d(fo, sd.yc, false));
-                continue;
-            }
-            bool use_n = false;
-            R nhx = 0, nhy = 0;
-            if (l <= 2) {
-                // surface normal: central difference of phi^n at the target (input frame)
-                const int ix = lx + shx, iy = ly + shy;
-                if (ix > fi.bx0 && iy > fi.by0 && ix < fi.bx1 && iy < fi.by1) {
-                    const int k0 = iy * T + ix;
-                    const R Xe = Xi[k0 + 1], Xw = Xi[k0 - 1], Xn = Xi[k0 + T], Xs = Xi[k0 - T];
-                    if (Xe == Xe && Xw == Xw && Xn == Xn && Xs == Xs) {
-                        const R pe = Pi[k0 + 1], pw = Pi[k0 - 1], pn = Pi[k0 + T], ps = Pi[k0 - T];
-                        const R gxp = (pe - pw) / R(2), gyp = (pn - ps) / R(2);
-                        const R nn = rsqrt_<R>(gxp * gxp + gyp * gyp);
-                        if (nn > R(0)) { use_n = true; nhx = gxp / nn; nhy = gyp / nn; }
-                    }
-                }
-            }
-            extrapolate_target<R>(sp, lab, Xo, Yo, T, lx, ly, l, use_n, nhx, nhy, a.err);
+    __syncthreads();
+    const int sx0 = sbb[0], sx1 = sbb[1], sy0 = sbb[2], sy1 = sbb[3];
+    const bool any = sx0 <= sx1;
+    if (!any && tid == 0) atomicOr(a.err, ERR_TILE_OVERFLOW);  // the solid vanished
+    // Layers 1..n_layers around S (Sec. 3.2; 11 layers, Sec. 4).  The allowed
+    // cells (not beyond the pad of a no-slip side) form a rectangle of the tile.
+    const int cx0 = sp.wall_x ? max(0, -2 - oo.x) : 0, cx1 = sp.wall_x ? min(T - 1, sp.nx + 1 - oo.x) : T - 1;
+    const int cy0 = sp.wall_y ? max(0, -2 - oo.y) : 0, cy1 = sp.wall_y ? min(T - 1, sp.ny + 1 - oo.y) : T - 1;
+    // the band's box (layer l lies within l of the box of S), and this CTA's rows of it
+    const int x0 = max(sx0 - NL, cx0), x1 = min(sx1 + NL, cx1), y0 = max(sy0 - NL, cy0), y1 = min(sy1 + NL, cy1);
+    const Strips st = {y0, any ? y1 : y0 - 1, 31 - __clz(nc), NL};  // nc: a power of two
+    const int yr0 = st.first(rank), yr1 = st.first(rank + 1);
+    // nodes within l steps of S: S itself, layers <= 2 kept for the relabel, three buffers in turn
+    const int my0 = CL ? st.set_first(rank) : -2;
+    auto set_of = [&](int l) {
+        const RowMask m = {masks + (l == 0 ? 0 : l == 1 ? 2 : l == 2 ? 1 : 2 + (l - 2) % 3) * mw, rw, my0};
+        return m;
+    };
+    const RowMask mS = set_of(0);
+    RefVals<R, CL> V;
+    if constexpr (CL) {
+        V.tile = reinterpret_cast<typename Vec2<R>::type *>(lists + list_ints);
+        V.stride = any ? x1 - x0 + 1 : 1;
+        V.o = (yr0 - 2) * V.stride + x0;
+        // the rows of S that this CTA's sets start from, from the CTAs that found them
+        const int r0 = max(max(yr0 - NL - 1, y0), jb0 - shy), r1 = min(min(yr1 + NL, y1), jb1 - shy);
+        for (int k = tid; k < (r1 - r0 + 1) * rw && any; k += blockDim.x) {
+            const int q = k / rw, w = k - q * rw, ly = r0 + q, row = ly - (jb0 - shy), owner = ((row + 1) * nc - 1) / ih;
+            mS.p[(ly - my0) * rw + w] = cluster_ld(mP.p + (row - ih * owner / nc) * rw + w, owner);
         }
         __syncthreads();
+        // their map, on the strip and its halo (written by pass 0 of any CTA before the cluster barrier)
+        const int v0 = max(yr0 - 2, sy0), v1 = min(yr1 + 1, sy1), w = sx1 - sx0 + 1;
+        BoxWalk wk(any ? w : 1);
+        for (int k = tid; k < w * (v1 - v0 + 1) && any; k += blockDim.x, wk.next()) {
+            const int lx = sx0 + wk.c, ly = v0 + wk.r;
+            if (!mS.bit(lx, ly)) continue;
+            typename Vec2<R>::type v;
+            v.x = Xo[ly * T + lx];
+            v.y = Yo[ly * T + lx];
+            V.tile[V.at(lx, ly)] = v;
+        }
+    } else {
+        V.X = Xo; V.Y = Yo; V.stride = T; V.o = 0;
+    }
+    // Dilate the set of layer l - 1 into that of layer l, a word per thread (from
+    // the last thread on: the first ones have targets of the layer before), and
+    // list the new nodes of this CTA's rows.  The words are those of the band's
+    // box (CL: of the rows from which the strip can be reached), whatever the layer.
+    const int wa = (x0 + 32) >> 5, wn = any ? ((x1 + 32) >> 5) - wa + 1 : 1;
+    const unsigned wdiv = wn > 1 ? 0xffffffffu / (unsigned)wn + 1u : 0u;  // k / wn = umulhi(k, wdiv) for k wn < 2^32
+    const int dy0 = CL ? max(y0, yr0 - NL) : y0, dn = wn * ((CL ? min(y1, yr1 + NL - 1) : y1) - dy0 + 1);
+    auto dilate = [&](int l) {
+        const unsigned *const v = set_of(l - 1).p, *const o = set_of(l).p;
+        int *list = lists + (l & 1) * layer_cap;
+        for (int kw = blockDim.x - 32 - 32 * warp; kw < dn; kw += blockDim.x) {  // uniform over the warp
+            const int k = kw + lane, row = wn > 1 ? (int)__umulhi((unsigned)k, wdiv) : k;
+            const int w = wa + k - row * wn, y = dy0 + row;
+            unsigned ring = 0;
+            if (k < dn) {
+                const int at = (y - my0) * rw + w;
+                const unsigned *q = v + at;
+                const unsigned c = q[0];
+                unsigned d = c | __funnelshift_l(q[-1], c, 1) | __funnelshift_r(c, q[1], 1) | q[-rw] | q[rw];
+                const int lo = max(x0 + 32 - 32 * w, 0), hi = min(x1 + 32 - 32 * w, 31);
+                d &= (0xffffffffu << lo) & (0xffffffffu >> (31 - hi));
+                const_cast<unsigned *>(o)[at] = d;
+                ring = y >= yr0 && y < yr1 ? d & ~c : 0u;
+            }
+            if (__ballot_sync(0xffffffffu, ring != 0u) == 0u) continue;
+            const int cnt = __popc(ring);
+            int pre = cnt;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, pre, d);
+                if (lane >= d) pre += t;
+            }
+            int at = 0;
+            if (lane == 31) at = atomicAdd(&lcnt[l], pre);
+            at = __shfl_sync(0xffffffffu, at, 31) + pre - cnt;
+            const int e0 = (32 * w - 32) | (y << 16);
+            while (ring) {
+                const int b = __ffs(ring) - 1;
+                ring &= ring - 1u;
+                if (at < layer_cap) list[at] = e0 + b;
+                at++;
+            }
+        }
+    };
+    // A fitted value goes to the map, and to the halo rows of the strips around.
+    auto put = [&](int lx, int ly, R vx, R vy) {
+        if constexpr (CL) {
+            V.tile[V.at(lx, ly)].x = vx;
+            V.tile[V.at(lx, ly)].y = vy;
+            for (int k = rank - 1; k >= 0 && ly < st.first(k + 1) + 2; k--) {
+                R *p = reinterpret_cast<R *>(V.tile + (ly - st.first(k) + 2) * V.stride + lx - x0);
+                cluster_st(p, k, vx);
+                cluster_st(p + 1, k, vy);
+            }
+            for (int k = rank + 1; k < nc && ly >= st.first(k) - 2; k++) {
+                R *p = reinterpret_cast<R *>(V.tile + (ly - st.first(k) + 2) * V.stride + lx - x0);
+                cluster_st(p, k, vx);
+                cluster_st(p + 1, k, vy);
+            }
+        } else {
+            Xo[ly * T + lx] = vx;
+            Yo[ly * T + lx] = vy;
+        }
+    };
+    // Along the surface normal at a target of layers 1 and 2: the central
+    // difference of phi^n (input frame); false where it is not to be had.
+    auto normal = [&](int l, int lx, int ly, R &gx, R &gy) {
+        gx = gy = R(0);
+        const int ix = lx + shx, iy = ly + shy;
+        if (l > 2 || !(ix > fi.bx0 && iy > fi.by0 && ix < fi.bx1 && iy < fi.by1)) return false;
+        const int q = iy * T + ix;
+        const R Xe = Xi[q + 1], Xw = Xi[q - 1], Xn = Xi[q + T], Xs = Xi[q - T];
+        const R pe = Pi[q + 1], pw = Pi[q - 1], pn = Pi[q + T], ps = Pi[q - T];
+        if (!(Xe == Xe && Xw == Xw && Xn == Xn && Xs == Xs)) return false;
+        gx = pe - pw;
+        gy = pn - ps;
+        return gx * gx + gy * gy > R(0);
+    };
+    // The n listed targets of layer l, LPT (XY: twice that) lanes to each.
+    auto fit_layer = [&](auto lpt, auto xy, int l, const int *list, int n) {
+        constexpr int LPT = decltype(lpt)::value;
+        constexpr bool XY = decltype(xy)::value;
+        constexpr int G = XY ? 2 * LPT : LPT;
+        const RowMask v = set_of(l - 1);
+        for (int k0 = 32 * warp / G; k0 < n; k0 += blockDim.x / G) {  // uniform over the warp
+            const int k = k0 + lane / G;
+            const bool on = k < n;
+            const int e = list[on ? k : n - 1], lx = e & 0xffff, ly = e >> 16;
+            R gx, gy, ox, oy;
+            const bool use_n = normal(l, lx, ly, gx, gy);
+            const bool good = fit_window<R, CL, LPT, XY>(V, lut, wd, v.window5(lx, ly), lx, ly, use_n, gx, gy, ox, oy);
+            if (!on || lane % G != 0) continue;
+            if (!good && !fit_grown<R, CL>(V, v, st, x0, T, lx, ly, sp.rmax, use_n, gx, gy, ox, oy)) atomicOr(a.err, ERR_EXTRAP);
+            put(lx, ly, ox, oy);
+        }
+    };
+    if (any) {
+        dilate(1);
+        __syncthreads();
+        for (int l = 1; l <= NL; l++) {
+            if (l < NL) dilate(l + 1);
+            int n = lcnt[l], *list = lists + (l & 1) * layer_cap;
+            if (a.init) {  // xi = x on the band at initialisation
+                const unsigned *const v = set_of(l - 1).p, *const o = set_of(l).p;
+                const R e0x = R(frame_d(fo, sd.xc, true)), e0y = R(frame_d(fo, sd.yc, false));
+                for (int k = tid; k < wn * (yr1 - yr0); k += blockDim.x) {
+                    const int ly = yr0 + k / wn, w = wa + k % wn, q = (ly - my0) * rw + w;
+                    for (unsigned ring = o[q] & ~v[q]; ring; ring &= ring - 1u) put(32 * w + __ffs(ring) - 33, ly, e0x, e0y);
+                }
+                solid_sync();
+                continue;
+            }
+            // a list that does not hold the layer is filled again for as many rows at a
+            // time as it holds in any case (their nodes come in any order)
+            const bool over = n > layer_cap;
+            const int rows = layer_cap / T;
+            for (int c = yr0; c < yr1; c += rows) {
+                if (over) {
+                    const unsigned *const v = set_of(l - 1).p, *const o = set_of(l).p;
+                    __syncthreads();
+                    if (tid == 0) lcnt[0] = 0;
+                    __syncthreads();
+                    for (int k = tid; k < wn * min(rows, yr1 - c); k += blockDim.x) {
+                        const int ly = c + k / wn, w = wa + k % wn, q = (ly - my0) * rw + w;
+                        for (unsigned ring = o[q] & ~v[q]; ring; ring &= ring - 1u)
+                            list[atomicAdd(&lcnt[0], 1)] = (32 * w + __ffs(ring) - 33) | (ly << 16);
+                    }
+                    __syncthreads();
+                    n = lcnt[0];
+                }
+                // Lanes to a target: with one CTA per SM a layer takes as long as one fit, so
+                // the window's rows go to 2, 4 or 8 lanes while the targets leave lanes
+                // idle -- in FP64, whose pipe takes a warp instruction per scheduler in 64
+                // cycles, up to one warp for each of the four, and a lane per coordinate.
+                // With several CTAs per SM the extra instructions cost more than they save.
+                if constexpr (CL) {
+                    typedef std::integral_constant<bool, sizeof(R) == 8> xy_t;
+                    const int room = sizeof(R) == 8 ? 64 : (int)blockDim.x;
+                    if (8 * n <= room) fit_layer(std::integral_constant<int, 8>(), xy_t(), l, list, n);
+                    else if (4 * n <= room) fit_layer(std::integral_constant<int, 4>(), xy_t(), l, list, n);
+                    else if (2 * n <= room) fit_layer(std::integral_constant<int, 2>(), xy_t(), l, list, n);
+                    else fit_layer(std::integral_constant<int, 1>(), xy_t(), l, list, n);
+                } else {
+                    fit_layer(std::integral_constant<int, 1>(), std::false_type(), l, list, n);
+                }
+                if (!over) break;
+            }
+            solid_sync();  // the next layer reads this one's values, and its list is complete
+        }
     }
 
-    // Relabel phi^{n+1} = phi_0(xi^{n+1}) over the box that can hold band nodes
-    // (layer l lies within l of the solid bbox); band and blur-zone bboxes;
-    // invalidate the free nodes of the box.
+    // Relabel phi^{n+1} = phi_0(xi^{n+1}) over this CTA's rows of the band's box;
+    // band and blur-zone boxes; invalidate the free nodes of the box.  The nodes
+    // in and near the blur zone, where FP32 keeps the level set as a float
+    // pair, are queued per warp and taken 32 at a time: one warp in two meets one.
+    const Rsq<R> rq(sd);
     int bx[8] = {1 << 29, -(1 << 29), 1 << 29, -(1 << 29), 1 << 29, -(1 << 29), 1 << 29, -(1 << 29)};
-    if (sx0 <= sx1) {
-        const int x0 = max(sx0 - sp.n_layers, 0), x1 = min(sx1 + sp.n_layers, T - 1);
-        const int y0 = max(sy0 - sp.n_layers, 0), y1 = min(sy1 + sp.n_layers, T - 1);
-        const int w = x1 - x0 + 1, n = w * (y1 - y0 + 1);
-        BoxWalk wk(w);
-        for (int k = threadIdx.x; k < n; k += blockDim.x, wk.next()) {
-            const int lx = x0 + wk.c, ly = y0 + wk.r, t = ly * T + lx;
-            if (lab[t] >= 0) {
-                bx[0] = min(bx[0], lx); bx[1] = max(bx[1], lx); bx[2] = min(bx[2], ly); bx[3] = max(bx[3], ly);
-                R phi = phi_eta(Xo[t], Yo[t], lx, ly, fo, rq);
+    {
+        const RowMask all = set_of(NL), two = set_of(min(NL, 2));
+        int *qu = lists + 64 * warp;
+        int qn = 0;  // warp-uniform
+        auto blur = [&](int cnt) {
+            if (lane < cnt) {
+                const int e = qu[qn - cnt + lane], lx = e & 0xffff, ly = e >> 16, t = ly * T + lx;
+                R phi = R(0), ex, ey;
+                V.get2(V.at(lx, ly), ex, ey);
                 if constexpr (xi_planes<R>() == 6) {
-                    // FP32: the level set as a float pair hi + lo in and near the blur
-                    // zone (the stresses and sets read hi; the density difference both)
-                    R exl = R(0), eyl = R(0);
-                    if (a.init || lab[t] > 0) {
-                        // the next step advects only nodes within a layer of this
-                        // step's solid (interfaces move less than one node per step):
-                        // their extrapolated eta has no low part
-                        if (a.init || lab[t] <= 2) {
-                            Xo[3 * TT + t] = R(0);
-                            Xo[4 * TT + t] = R(0);
-                        }
-                    } else {
-                        exl = Xo[3 * TT + t];  // the advection's low parts
+                    // the advection's low parts (an extrapolated node has none)
+                    R exl = R(0), eyl = R(0), pl;
+                    if (!a.init && mS.bit(lx, ly)) {
+                        exl = Xo[3 * TT + t];
                         eyl = Xo[4 * TT + t];
                     }
-                    if (phi > -eps - R(PHI_D_SHELL) && phi < eps + R(PHI_D_SHELL)) {
-                        R pl;
-                        if (rq.shape == 0) {
-                            phi_node_ff(Xo[t], Yo[t], exl, eyl, lx, ly, fo, rq, sd.Rlo_f, phi, pl);
-                        } else {
-                            const double X = ((double)lx + (double)fo.offx) + ((double)Xo[t] + (double)exl);
-                            const double Y = ((double)ly + (double)fo.offy) + ((double)Yo[t] + (double)eyl);
-                            const double dd = shape_sdf_polished(rq.shape, rq.a, rq.b, X, Y, sp.eps, PHI_D_SHELL);
-                            phi = R(dd);
-                            pl = R(dd - (double)phi);
-                        }
-                        Xo[5 * TT + t] = pl;  // read only where |phi| < eps + PHI_D_SHELL
+                    if (rq.shape == 0) {
+                        phi_node_ff(ex, ey, exl, eyl, lx, ly, fo, rq, sd.Rlo_f, phi, pl);
+                    } else {
+                        const double X = ((double)lx + (double)fo.offx) + ((double)ex + (double)exl);
+                        const double Y = ((double)ly + (double)fo.offy) + ((double)ey + (double)eyl);
+                        const double dd = shape_sdf_polished(rq.shape, rq.a, rq.b, X, Y, sp.eps, PHI_D_SHELL);
+                        phi = R(dd);
+                        pl = R(dd - (double)phi);
                     }
+                    Xo[5 * TT + t] = pl;  // read only where |phi| < eps + PHI_D_SHELL
                 }
                 Po[t] = phi;
                 if (phi < eps) {
                     bx[4] = min(bx[4], lx); bx[5] = max(bx[5], lx); bx[6] = min(bx[6], ly); bx[7] = max(bx[7], ly);
                 }
-            } else {
-                Xo[t] = nanv<R>();
-                Yo[t] = nanv<R>();
-                Po[t] = nanv<R>();
+            }
+            __syncwarp();
+            qn -= cnt;
+        };
+        const int w = any ? x1 - x0 + 1 : 1, n = any ? w * (yr1 - yr0) : 0;
+        BoxWalk wk(w);
+        for (int k0 = 0; k0 < n; k0 += blockDim.x, wk.next()) {
+            const int lx = x0 + wk.c, ly = yr0 + wk.r, t = ly * T + lx;
+            bool queue = false;
+            if (k0 + tid < n) {
+                if (all.bit(lx, ly)) {
+                    bx[0] = min(bx[0], lx); bx[1] = max(bx[1], lx); bx[2] = min(bx[2], ly); bx[3] = max(bx[3], ly);
+                    R ex, ey;
+                    V.get2(V.at(lx, ly), ex, ey);
+                    if (CL && !mS.bit(lx, ly)) {
+                        Xo[t] = ex;
+                        Yo[t] = ey;
+                    }
+                    const R phi = phi_eta(ex, ey, lx, ly, fo, rq);
+                    if constexpr (xi_planes<R>() == 6) {
+                        // the next step advects only nodes within a layer of this step's
+                        // solid (interfaces move less than one node per step): their
+                        // extrapolated eta has no low part
+                        if (a.init || (two.bit(lx, ly) && !mS.bit(lx, ly))) {
+                            Xo[3 * TT + t] = R(0);
+                            Xo[4 * TT + t] = R(0);
+                        }
+                        queue = phi > -eps - R(PHI_D_SHELL) && phi < eps + R(PHI_D_SHELL);
+                    }
+                    if (!queue) {
+                        Po[t] = phi;
+                        if (phi < eps) {
+                            bx[4] = min(bx[4], lx); bx[5] = max(bx[5], lx); bx[6] = min(bx[6], ly); bx[7] = max(bx[7], ly);
+                        }
+                    }
+                } else {
+                    Xo[t] = nanv<R>();
+                    Yo[t] = nanv<R>();
+                    Po[t] = nanv<R>();
+                }
+            }
+            if constexpr (xi_planes<R>() == 6) {
+                const unsigned m = __ballot_sync(0xffffffffu, queue);
+                if (queue) qu[qn + __popc(m & ((1u << lane) - 1u))] = lx | (ly << 16);
+                qn += __popc(m);
+                __syncwarp();
+                if (qn >= 32) blur(32);
             }
         }
+        if (qn > 0) blur(qn);
     }
     for (int k = 0; k < 8; k++) warp_minmax(bx[k], (k & 1) == 0);
     if (lane == 0)
         for (int k = 0; k < 8; k += 2) { atomicMin(&bb[4 + k], bx[k]); atomicMax(&bb[5 + k], bx[k + 1]); }
-    // the solid's sums (its mean velocity sets the next frame's offset): in the
-    // arithmetic precision (the terms are; FP64 is a narrow pipe on this GPU)
-    double st[6];
-    if (a.stats) block_sum<R, 6>(stl, reinterpret_cast<R *>(red));
-    for (int k = 0; k < 6; k++) st[k] = (double)stl[k];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (a.stats) {
-            double *o = a.stats + 8 * s;
-            const double L = st[0];
-            o[0] = L; o[1] = oo.x + st[1] / L; o[2] = oo.y + st[2] / L; o[3] = st[3]; o[4] = st[4]; o[5] = st[5];
-            o[6] = 0; o[7] = 0;
+    solid_sync();
+    if constexpr (CL) {
+        // the first CTA gathers the boxes and sums of the others, which stay until it has
+        long long v0 = 0, v1 = 0;
+        if (rank == 0 && warp == 0) {
+            const int src = lane < nc ? lane : 0;
+            int v[12];
+            for (int k = 4; k < 12; k++) v[k] = (int)cluster_ld(&bb[k], src);
+            int nS = lane < nc ? (int)cluster_ld(&bb[12], src) : 0;
+            if (lane < nc) {
+                const unsigned *q = reinterpret_cast<const unsigned *>(vsum);
+                v0 = (long long)(((unsigned long long)cluster_ld(q + 1, src) << 32) | cluster_ld(q, src));
+                v1 = (long long)(((unsigned long long)cluster_ld(q + 3, src) << 32) | cluster_ld(q + 2, src));
+            }
+            for (int k = 4; k < 12; k++) warp_minmax(v[k], (k & 1) == 0);
+            nS = __reduce_add_sync(0xffffffffu, nS);
+            for (int d = 16; d > 0; d >>= 1) {
+                v0 += __shfl_down_sync(0xffffffffu, v0, d);
+                v1 += __shfl_down_sync(0xffffffffu, v1, d);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                for (int k = 4; k < 12; k++) bb[k] = v[k];
+                bb[12] = nS;
+                vsum[0] = (unsigned long long)v0;
+                vsum[1] = (unsigned long long)v1;
+            }
         }
+        cluster_sync();
+        if (rank != 0) return;
+    }
+    // The frames, by one thread of the last warp; the registry, by the first ones.
+    if (tid == (int)blockDim.x - 32) {
         int2 nx = oo;
         // mean velocity of the solid at time n (zero at initialisation) moves d
         double ux = 0.0, uy = 0.0;
-        if (a.stats && st[3] > 0.0) { ux = st[4] / st[3]; uy = st[5] / st[3]; }
+        if (!a.init && bb[12] > 0) {
+            const double q = 1.0 / ((double)VEL_SCALE * (double)bb[12]);
+            ux = (double)(long long)vsum[0] * q;
+            uy = (double)(long long)vsum[1] * q;
+        }
         Frame fb = fo;
         if (bb[4] > bb[5]) {
             atomicOr(a.err, ERR_TILE_OVERFLOW);
@@ -1408,9 +1882,9 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
             fb.bx0 = (short)bb[4]; fb.bx1 = (short)bb[5]; fb.by0 = (short)bb[6]; fb.by1 = (short)bb[7];
             // centre the next frame on the solid (not on its band, which walls clip): the
             // frame then follows the solid's translation and eta stays small
-            if (bb[0] <= bb[1]) {
-                nx.x = oo.x + (bb[0] + bb[1]) / 2 - T / 2;
-                nx.y = oo.y + (bb[2] + bb[3]) / 2 - T / 2;
+            if (any) {
+                nx.x = oo.x + (sx0 + sx1) / 2 - T / 2;
+                nx.y = oo.y + (sy0 + sy1) / 2 - T / 2;
             }
         }
         a.frame_out[s] = fb;
@@ -1431,7 +1905,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
             for (int ax = 0; ax < nrx; ax++) {
                 const int tx0 = rx0[ax], ty0 = ry0[ay];
                 const int ntxr = rx1[ax] - tx0 + 1, nall = ntxr * (ry1[ay] - ty0 + 1);
-                for (int k = threadIdx.x; k < nall; k += blockDim.x) {
+                for (int k = tid; k < nall; k += blockDim.x) {
                     const int tile = (ty0 + k / ntxr) * sp.ntx + tx0 + k % ntxr;
                     const int slot = atomicAdd(&a.reg_count[tile], 1);
                     if (slot < sp.kmax) a.reg_solids[tile * KMAX + slot] = s;
@@ -1444,16 +1918,18 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
 
 template <class R, class S>
 __global__ void __launch_bounds__(RMT_THREADS, sizeof(R) == 4 ? RMT_MIN_BLOCKS : 2) rmt_solid_kernel(SimParams sp, RmtArgs<R, S> a) {
-    rmt_solid<R, S>(sp, a, a.order ? a.order[blockIdx.x] : (int)blockIdx.x);
+    rmt_solid<R, S, false>(sp, a, a.order ? a.order[blockIdx.x] : (int)blockIdx.x, 0, 1);
 }
 
-// The same with 1024-thread CTAs, for simulations with fewer solids than SMs:
-// each solid's layer chain then runs on four times the threads.  Same register
-// budget as the 256-thread kernel (64), hence the same instructions per node.
-constexpr int RMT_THREADS_BIG = 1024;
+// The same with each solid spread over a cluster of CTAs (grid: solids x cluster
+// size), for simulations with at most half as many solids as SMs.  512 threads (128 registers, no
+// spills): 256 are as fast on small disks and up to a third slower on large ones.
+constexpr int RMT_WIDE_THREADS = 512;
+constexpr int RMT_THREADS_BIG = 1024;  // lbrmt_set_rmt_threads' name for this form
 template <class R, class S>
-__global__ void __launch_bounds__(RMT_THREADS_BIG, 1) rmt_solid_kernel_big(SimParams sp, RmtArgs<R, S> a) {
-    rmt_solid<R, S>(sp, a, a.order ? a.order[blockIdx.x] : (int)blockIdx.x);
+__global__ void __launch_bounds__(RMT_WIDE_THREADS, 1) rmt_solid_kernel_wide(SimParams sp, RmtArgs<R, S> a) {
+    const int nc = cluster_size(), k = blockIdx.x / nc;
+    rmt_solid<R, S, true>(sp, a, a.order ? a.order[k] : k, cluster_rank(), nc);
 }
 
 // ===========================================================================
@@ -2072,8 +2548,6 @@ __device__ __forceinline__ void classify_region(const SimParams &sp, int r, cons
 // two shared-memory stages, completing on an mbarrier, so the copies of the
 // next tile overlap the collision of the current one.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
