@@ -924,22 +924,6 @@ __device__ inline double shape_sdf_mixed(int shape, double a, double b, double q
     return (y0 / e0) * (y0 / e0) + (y1 / e1) * (y1 / e1) < 1.0 ? -d : d;
 }
 
-// The same with the root polished in double wherever the distance is below
-// eps + shell (the blur zone and a shell around it): there the result is
-// exact to ~1e-13, for the level set's low part.
-__device__ inline double shape_sdf_polished(int shape, double a, double b, double qx, double qy, double eps,
-                                            double shell) {
-    if (shape == 2) return shape_sdf(shape, a, b, qx, qy);
-    double y0 = fabs(qx), y1 = fabs(qy), e0 = a, e1 = b;
-    if (e0 < e1) {
-        double t = e0; e0 = e1; e1 = t;
-        t = y0; y0 = y1; y1 = t;
-    }
-    // polish below eps + shell: the shell argument covers [0, eps + shell] around zero
-    const double d = ellipse_distance_q1_mixed(e0, e1, y0, y1, 0.0, eps + shell);
-    return (y0 / e0) * (y0 / e0) + (y1 / e1) * (y1 / e1) < 1.0 ? -d : d;
-}
-
 // Level set phi_0 of a disk at a tile node: with p = l + off (exact) and eta,
 // phi = |p + eta| - R = (|p|^2 - R^2 + 2 p.eta + |eta|^2) / (|p + eta| + R),
 // where |p|^2 - R^2 is formed with error-free products and a two-sum, so
@@ -970,19 +954,11 @@ __device__ __forceinline__ float two_sum_f(float a, float b, float &e) {
     return s;
 }
 
-// phi_0 of a tile node as a float pair ph + pl (error ~1e-14): for a disk,
+// phi_0 of a disk's tile node as a float pair ph + pl (error ~1e-14):
 // phi = (|p|^2 - R^2) / (|p| + R) with p = (l + off) + eta (hi + lo), in
-// float-float arithmetic; other shapes take the signed distance in double.
+// float-float arithmetic.
 __device__ __forceinline__ void phi_node_ff(float ex, float ey, float exl, float eyl, int lx, int ly, const Frame &fr,
                                             const Rsq<float> &q, float Rlo, float &ph, float &pl) {
-    if (q.shape != 0) {
-        const double X = ((double)lx + (double)fr.offx) + ((double)ex + (double)exl);
-        const double Y = ((double)ly + (double)fr.offy) + ((double)ey + (double)eyl);
-        const double d = shape_sdf(q.shape, q.a, q.b, X, Y);
-        ph = (float)d;
-        pl = (float)(d - (double)ph);
-        return;
-    }
     float e;
     const float pxh = two_sum_f(__fadd_rn((float)lx, fr.offx), ex, e), pxl = e + exl;
     const float pyh = two_sum_f(__fadd_rn((float)ly, fr.offy), ey, e), pyl = e + eyl;
@@ -1004,6 +980,132 @@ __device__ __forceinline__ void phi_node_ff(float ex, float ey, float exl, float
     const float q2 = res / dh;
     ph = q1 + q2;
     pl = q2 - (ph - q1);
+}
+
+// Float pairs with every operation written out (no contraction by the
+// compiler), so that each kernel forms the same bits.
+struct ff {
+    float h, l;
+};
+__device__ __forceinline__ ff ff_fast(float a, float b) {  // |a| >= |b|, or a == 0
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ ff ff_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ ff operator+(ff a, ff b) {
+    const ff s = ff_sum(a.h, b.h);
+    return ff_fast(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ ff operator-(ff a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ ff operator*(ff a, ff b) {
+    const float p = __fmul_rn(a.h, b.h);
+    return ff_fast(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ ff operator/(ff a, ff b) {
+    const float q = __fdiv_rn(a.h, b.h);
+    const float r = __fmaf_rn(-q, b.h, a.h);  // exact
+    return ff_fast(q, __fdiv_rn(__fmaf_rn(-q, b.l, __fadd_rn(r, a.l)), b.h));
+}
+__device__ __forceinline__ ff ff_sqrt(ff a) {
+    const float r = __fsqrt_rn(a.h);
+    return r > 0.0f ? ff_fast(r, __fdiv_rn(__fadd_rn(__fmaf_rn(-r, r, a.h), a.l), __fadd_rn(r, r))) : ff{0.0f, 0.0f};
+}
+__device__ __forceinline__ ff ff_abs(ff a) { return a.h < 0.0f || (a.h == 0.0f && a.l < 0.0f) ? -a : a; }
+__device__ __forceinline__ ff ff_of(double v) {
+    const float h = (float)v;
+    return {h, (float)(v - (double)h)};
+}
+
+// A non-disk solid's level set in FP32 arithmetic.  Rectangle: half-sides e0
+// (x) and e1 (y).  Ellipse: semi-axes e0 >= e1 (swapped: e0 along y), r1 = (e0 /
+// e1)^2 - 1, k0 = e0 / e1^2, k1 = 1 / e1, so that n0 = k0 |q0| and z1 = k1 |q1|.  One
+// thread per solid fills it in double.
+struct ShapeF {
+    int shape, swapped;
+    double a, b;
+    ff e0, e1, r1, k0, k1;
+};
+__device__ __forceinline__ void shape_consts(const SolidDesc &sd, ShapeF &c) {
+    c.shape = sd.shape; c.a = sd.a; c.b = sd.b;
+    c.swapped = sd.shape == 1 && sd.a < sd.b;
+    const double e0 = c.swapped ? sd.b : sd.a, e1 = c.swapped ? sd.a : sd.b, k1 = 1.0 / e1;
+    c.e0 = ff_of(e0); c.e1 = ff_of(e1); c.k1 = ff_of(k1);
+    c.k0 = ff_of(e0 / (e1 * e1));
+    c.r1 = ff_of((e0 - e1) * (e0 + e1) / (e1 * e1));
+}
+
+// The root w of (n0 / (w + r1))^2 + (z1 / w)^2 = 1 (Eberly's characterisation
+// of the closest point, w = 1 + t / e1^2), n0, z1 > 0, to FP32 rounding.  With G the
+// left side, the steps are Newton's on 1 - 1 / sqrt(G) (the form that Hebden and
+// More-Sorensen use for the secular equation, nearly linear in w): from the left
+// end of the bracket they rise to the root in three or four, where Newton's on G
+// itself took up to a dozen.
+__device__ __forceinline__ float ellipse_root(float n0, float z1, float r1) {
+    float w = fmaxf(z1, __fsub_rn(n0, r1));
+    for (int it = 0; it < 12; it++) {
+        const float ia = __fdividef(1.0f, __fadd_rn(w, r1)), ib = __fdividef(1.0f, w);
+        const float ra = __fmul_rn(n0, ia), rb = __fmul_rn(z1, ib), a2 = __fmul_rn(ra, ra), b2 = __fmul_rn(rb, rb);
+        const float G = __fadd_rn(a2, b2), D = __fmaf_rn(a2, ia, __fmul_rn(b2, ib));
+        const float dw = __fdividef(__fmul_rn(G, __fsub_rn(__fsqrt_rn(G), 1.0f)), D);
+        if (!(dw > __fmul_rn(2e-7f, w))) break;
+        w = __fadd_rn(w, dw);
+    }
+    return w;
+}
+
+// phi_0 at q = (X, Y) relative to the centre, to about 1e-6 (beyond the shell
+// around the blur zone, where only its sign and size count).
+__device__ __forceinline__ float shape_phi_f(const ShapeF &c, float X, float Y) {
+    if (c.shape == 2) {
+        const float dx = __fsub_rn(fabsf(X), c.e0.h), dy = __fsub_rn(fabsf(Y), c.e1.h);
+        const float ox = fmaxf(dx, 0.0f), oy = fmaxf(dy, 0.0f);
+        return __fadd_rn(__fsqrt_rn(__fmaf_rn(ox, ox, __fmul_rn(oy, oy))), fminf(fmaxf(dx, dy), 0.0f));
+    }
+    const float y0 = fabsf(c.swapped ? Y : X), y1 = fabsf(c.swapped ? X : Y);
+    const float n0 = __fmul_rn(c.k0.h, y0), z1 = __fmul_rn(c.k1.h, y1);
+    if (!(n0 > 1e-6f && z1 > 1e-6f))  // on an axis: the closed forms
+        return (float)shape_sdf(c.shape, c.a, c.b, (double)X, (double)Y);
+    const float w = ellipse_root(n0, z1, c.r1.h);
+    const float A = __fdividef(y0, __fadd_rn(w, c.r1.h)), B = __fdividef(y1, w);
+    return __fmul_rn(__fsub_rn(w, 1.0f), __fsqrt_rn(__fmaf_rn(A, A, __fmul_rn(B, B))));
+}
+
+// phi_0 as a float pair (error ~1e-13).  Ellipse: the FP32 root polished by two
+// Newton steps with the residual in float pairs, and from the closest point e_i^2
+// q_i / (t + e_i^2) the distance (w - 1) |(q0 / (w + r1), q1 / w)|, negative inside: no
+// difference of near numbers is left.  (The same in double took 287 K of a
+// solid's 370 K cycles on the 506-ellipse mixing, GB300's FP64 running at 1/64 of
+// its FP32 rate: K2 240 -> 66 us.)  On an axis, or should the steps not have converged, in double.
+__device__ __forceinline__ ff shape_phi_ff(const ShapeF &c, ff X, ff Y) {
+    const ff one = {1.0f, 0.0f};
+    if (c.shape == 2) {
+        const ff dx = ff_abs(X) + -c.e0, dy = ff_abs(Y) + -c.e1;
+        const bool px = dx.h > 0.0f, py = dy.h > 0.0f;
+        if (px && py) return ff_sqrt(dx * dx + dy * dy);
+        return dx.h > dy.h || (dx.h == dy.h && dx.l > dy.l) ? dx : dy;
+    }
+    const ff y0 = ff_abs(c.swapped ? Y : X), y1 = ff_abs(c.swapped ? X : Y);
+    const ff n0 = c.k0 * y0, z1 = c.k1 * y1;
+    if (n0.h > 1e-6f && z1.h > 1e-6f) {
+        ff w = {ellipse_root(n0.h, z1.h, c.r1.h), 0.0f};
+        float left = 1.0f;
+        for (int it = 0; it < 2; it++) {
+            const ff pa = w + c.r1, ra = n0 / pa, rb = z1 / w, a2 = ra * ra, b2 = rb * rb;
+            const ff f = (a2 + -one) + b2;
+            const float D = __fadd_rn(__fdividef(a2.h, pa.h), __fdividef(b2.h, w.h));
+            const float dw = __fdividef(__fmul_rn(0.5f, f.h), D);
+            w = w + ff{dw, 0.0f};
+            left = __fdividef(fabsf(dw), w.h);
+        }
+        if (left < 1e-6f) {  // the last step was below FP32's rounding: its square is what is left
+            const ff A = y0 / (w + c.r1), B = y1 / w;
+            return (w + -one) * ff_sqrt(A * A + B * B);
+        }
+    }
+    return ff_of(shape_sdf(c.shape, c.a, c.b, (double)X.h + (double)X.l, (double)Y.h + (double)Y.l));
 }
 
 // lambda = 1 - H_eps(phi) for phi = ph + pl as a float pair lh + ll, from the
@@ -1402,6 +1504,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     __shared__ int sbb[4];     // box of S over the cluster
     __shared__ int lut[32];
     __shared__ R wd[25];
+    __shared__ ShapeF shp;     // a non-disk solid's constants (FP32 arithmetic)
     __shared__ unsigned long long vsum[2];
     __syncthreads();  // the shared state of a previous solid is no longer read
     const SolidDesc &sd = a.solids[s];
@@ -1440,6 +1543,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
         const int dx = (tid - 32) % 5 - 2, dy = (tid - 32) / 5 - 2;
         wd[tid - 32] = pow2neg<R>(abs(dx) + abs(dy)) * rinv_tab<R>(dx, dy);
     }
+    if (xi_planes<R>() == 6 && sd.shape != 0 && tid == (int)blockDim.x - 1) shape_consts(sd, shp);
     for (int k = tid; k < (RMT_MASKS * mw + m0w) / 4; k += blockDim.x) reinterpret_cast<int4 *>(masks)[k] = make_int4(0, 0, 0, 0);
     int acc[3] = {0, 0, 0};
     int sb[4] = {1 << 29, -(1 << 29), 1 << 29, -(1 << 29)};
@@ -1766,11 +1870,11 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
                     if (rq.shape == 0) {
                         phi_node_ff(ex, ey, exl, eyl, lx, ly, fo, rq, sd.Rlo_f, phi, pl);
                     } else {
-                        const double X = ((double)lx + (double)fo.offx) + ((double)ex + (double)exl);
-                        const double Y = ((double)ly + (double)fo.offy) + ((double)ey + (double)eyl);
-                        const double dd = shape_sdf_polished(rq.shape, rq.a, rq.b, X, Y, sp.eps, PHI_D_SHELL);
-                        phi = R(dd);
-                        pl = R(dd - (double)phi);
+                        const ff X = ff_sum(__fadd_rn((float)lx, fo.offx), ex) + ff{exl, 0.0f};  // l + off is exact
+                        const ff Y = ff_sum(__fadd_rn((float)ly, fo.offy), ey) + ff{eyl, 0.0f};
+                        const ff d = shape_phi_ff(shp, X, Y);
+                        phi = d.h;
+                        pl = d.l;
                     }
                     Xo[5 * TT + t] = pl;  // read only where |phi| < eps + PHI_D_SHELL
                 }
@@ -1796,7 +1900,15 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
                         Xo[t] = ex;
                         Yo[t] = ey;
                     }
-                    const R phi = phi_eta(ex, ey, lx, ly, fo, rq);
+                    R phi;
+                    if constexpr (xi_planes<R>() == 6) {
+                        if (rq.shape == 0) phi = phi_eta(ex, ey, lx, ly, fo, rq);
+                        else
+                            phi = shape_phi_f(shp, __fadd_rn(__fadd_rn((float)lx, fo.offx), ex),
+                                              __fadd_rn(__fadd_rn((float)ly, fo.offy), ey));
+                    } else {
+                        phi = phi_eta(ex, ey, lx, ly, fo, rq);
+                    }
                     if constexpr (xi_planes<R>() == 6) {
                         // the next step advects only nodes within a layer of this step's
                         // solid (interfaces move less than one node per step): their

@@ -3,7 +3,7 @@ CTAs per solid, strips of rows) on the sizes where they can go wrong.
 
 Both forms form every sum in the same order, so their fields agree bit for bit:
 solids of a node or two (windows grown beyond 5x5, strips of two rows), solids at walls
-(clipped bands) and across periodic edges, many layers, and a disk whose layers
+(clipped bands) and across periodic edges, other shapes, many layers, and a disk whose layers
 hold more nodes than the narrow form's list.  Tiny
 disks are also held to the oracle, whose fits know neither form.
 """
@@ -42,6 +42,7 @@ CASES = {
     "tiny": lambda: _box(96, 80, 0, 0, [_disk(30.3, 40.2, 1.0), _disk(70.6, 20.1, 1.4), _disk(60.2, 61.7, 2.3)]),
     "at_walls": lambda: _box(90, 100, 1, 1, [_disk(7.2, 8.1, 5.0), _disk(82.5, 92.4, 5.5), _disk(45.0, 6.3, 4.0)]),
     "across_edges": lambda: _box(131, 118, 0, 0, [_disk(0.4, 117.3, 14.0), _disk(66.0, 58.5, 20.0)]),
+    "shapes": lambda: scenarios.shapes_small(1),
     "twenty_layers": lambda: _box(120, 130, 0, 1, [_disk(60.2, 65.3, 9.0)], n_layers=20),
     "wide_margin": lambda: _box(200, 190, 0, 1, [_disk(100.2, 95.3, 8.0)], deform_margin=4.0),
     "long_layers": lambda: _box(430, 440, 1, 1, [_disk(214.3, 220.4, 170.0)], deform_margin=0.05),
