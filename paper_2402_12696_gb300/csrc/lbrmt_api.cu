@@ -170,7 +170,7 @@ extern "C" lbrmt_status lbrmt_create(const lbrmt_config *cfg, void *cuda_stream,
     if (c.force_kind == LBRMT_FORCE_FIELD) ok = ok && (d.bfield = dalloc(s, 2 * P * rs));
     ok = ok && (d.mass_partials = (double *)dalloc(s, nparts * 8));
     ok = ok && (d.err = (unsigned *)dalloc(s, 16));
-    ok = ok && (d.lamtab = (LamEntry *)dalloc(s, (size_t)(2 * sp.lam_k0 + 1) * sizeof(LamEntry)));
+    ok = ok && (d.lamtab = dalloc(s, (size_t)(2 * sp.lam_k0 + 1) * (rs == 4 ? sizeof(LamEntry) : sizeof(LamEntryD))));
     ok = ok && (s->scratch = (double *)dalloc(s, 128));  // one solid's statistics or the total mass
     // side stream (lowest priority) and fork / join events of the overlapped step
     if (ok) {
@@ -211,6 +211,7 @@ extern "C" lbrmt_status lbrmt_create(const lbrmt_config *cfg, void *cuda_stream,
     if (e == cudaSuccess) {
         const int n = 2 * sp.lam_k0 + 1;
         std::vector<LamEntry> tab(n);
+        std::vector<LamEntryD> tabd(n);
         const double eps = c.eps, pi = M_PI;
         for (int k = 0; k < n; k++) {
             const double t = (double)(k - sp.lam_k0) * (double)sp.lam_h / eps;
@@ -225,12 +226,14 @@ extern "C" lbrmt_status lbrmt_create(const lbrmt_config *cfg, void *cuda_stream,
                 fact *= m;
                 lk[m] = -std::pow(pi, m - 1) / (2.0 * std::pow(eps, m)) * dsin[m] / fact;
             }
+            for (int m = 0; m < 6; m++) tabd[k].l[m] = lk[m];
             LamEntry &q = tab[k];
             q.l0h = (float)lam; q.l0l = (float)(lam - (double)q.l0h);
             q.l1h = (float)l1; q.l1l = (float)(l1 - (double)q.l1h);
             q.l2 = (float)lk[2]; q.l3 = (float)lk[3]; q.l4 = (float)lk[4]; q.l5 = (float)lk[5];
         }
-        e = cudaMemcpy(d.lamtab, tab.data(), n * sizeof(LamEntry), cudaMemcpyHostToDevice);
+        e = rs == 4 ? cudaMemcpy(d.lamtab, tab.data(), n * sizeof(LamEntry), cudaMemcpyHostToDevice)
+                    : cudaMemcpy(d.lamtab, tabd.data(), n * sizeof(LamEntryD), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) {
         if (rs == 4) {

@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(K3_THREADS, sizeof(R) == 4 ? 4 : 1) force_batc
     __syncthreads();
     const int total = pre[nsim];
     int cur = -1;
+    ForceMap fm;
     for (int it = blockIdx.x; it < total; it += gridDim.x) {
         int lo = 0, hi = nsim;  // largest lo with pre[lo] <= it
         while (hi - lo > 1) {
@@ -79,8 +80,9 @@ __global__ void __launch_bounds__(K3_THREADS, sizeof(R) == 4 ? 4 : 1) force_batc
             }
             __syncthreads();
             cur = lo;
+            fm = force_map(sp);
         }
-        force_tile<R>(sp, fa, fa.reg_active[it - pre[lo]], fs, reinterpret_cast<R *>(smem));
+        force_tile<R>(sp, fa, fm, fa.reg_active[it - pre[lo]], fs, reinterpret_cast<R *>(smem));
     }
 }
 

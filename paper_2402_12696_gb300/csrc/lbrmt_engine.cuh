@@ -14,10 +14,9 @@ namespace lbrmt {
 struct LaunchInfo {
     int tmax;            // largest solid tile side
     int force_blocks;    // persistent grid of K3
-    int force_blocks_ov; // the same in the overlapped step (fewer CTAs per SM)
+    int force_blocks_ov; // the same in the overlapped step
     int rmt_smem;        // dynamic shared memory of K2
     int rmt_carve;       // K2's preferred shared-memory carveout (percent), or -1
-    int force_carve_ov;  // the overlapped K3's preferred carveout (percent), or -1
     int force_smem;      // dynamic shared memory of K3
     int rmt_req = 0;      // requested K2 CTA width (0: chosen by configure)
     int rmt_threads = 256; // the form as lbrmt_rmt_threads tells it: 256, or 1024 (FP32 arithmetic only)
@@ -92,12 +91,6 @@ inline cudaError_t launch_carve(void (*kernel)(P...), dim3 grid, dim3 block, siz
 // Shared-memory carveout steps of this GPU family (KB): the SM's 256 KB of
 // L1/shared storage not carved out for shared memory is L1 cache.
 constexpr int CARVE_STEPS_KB[] = {8, 16, 32, 64, 100, 132, 164, 196, 228};
-// The smallest step that holds need bytes (-1: none up to per_sm).
-inline int carve_step(int need, int per_sm) {
-    for (int kb : CARVE_STEPS_KB)
-        if (kb * 1024 >= need) return kb * 1024 <= per_sm ? kb * 1024 : -1;
-    return -1;
-}
 // A step as a launch's carveout preference: percent of the largest carveout,
 // rounded down, so that the driver, which rounds up to its steps, lands on it.
 inline int carve_percent(int step, int per_sm) { return step > 0 ? (int)(100.0 * step / per_sm) : -1; }
@@ -354,31 +347,15 @@ struct Engine {
         li->rmt_nc = 0;
         if (w == RMT_THREADS_BIG || (sizeof(R) == 8 && few && li->rmt_req == 0)) e = configure_wide(sp, tmax, nsm0, li);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(force_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 force_smem_max() * (int)sizeof(R));
-        if (e != cudaSuccess) return e;
         int dev = 0, nsm = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, force_kernel<R>, K3_THREADS, li->force_smem);
-        if (e != cudaSuccess) return e;
-        li->force_blocks = nsm * (per > 0 ? per : 1);
-        // In the overlapped step K3 runs beside the free regions' K1: three of its
-        // CTAs per SM (of four that fit) leave the registers of two K1 CTAs, and
-        // the step is shorter although K3 alone takes longer.
-        li->force_blocks_ov = nsm * std::min(std::max(per, 1), 3);
-        // With fewer CTAs per SM than fit, the overlapped K3 asks for the
-        // carveout step that holds those only: more L1 beside them.
-        li->force_carve_ov = -1;
-        if (per > 3) {
-            int per_sm, resv;
-            smem_limits(&per_sm, &resv);
-            cudaFuncAttributes fa;
-            if (per_sm > 0 && cudaFuncGetAttributes(&fa, force_kernel<R>) == cudaSuccess)
-                li->force_carve_ov =
-                    carve_percent(carve_step(3 * (li->force_smem + (int)fa.sharedSizeBytes + resv), per_sm), per_sm);
-            else
-                cudaGetLastError();
+        for (int ov = 0; ov < 2; ov++) {
+            auto kernel = ov ? force_kernel<R, 48> : force_kernel<R, 56>;
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, force_smem_max() * (int)sizeof(R));
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, K3_THREADS, li->force_smem);
+            if (e != cudaSuccess) return e;
+            (ov ? li->force_blocks_ov : li->force_blocks) = nsm * std::max(per, 1);
         }
         configure_tma(sp, d, li, nsm);
         return cudaSuccess;
@@ -541,7 +518,7 @@ struct Engine {
     static cudaError_t init(const SimParams &sp, const DevState &d, const LaunchInfo &li, cudaStream_t st) {
         if (sp.nsolids > 0) {
             launch_rmt(sp, li, rmt_args(d, 0, 1), st);
-            force_kernel<R><<<li.force_blocks, K3_THREADS, li.force_smem, st>>>(sp, force_args(d, 0, 1));
+            force_kernel<R, 56><<<li.force_blocks, K3_THREADS, li.force_smem, st>>>(sp, force_args(d, 0, 1));
         }
         dim3 grid(sp.ntx, sp.nty), blk(TILE_N);
         init_f_kernel<R, S><<<grid, blk, 0, st>>>(sp, (S *)d.f[0], (S *)d.carry);
@@ -580,8 +557,8 @@ struct Engine {
         }
         if (ev) cudaEventRecord(ev[1], st);
         if (sp.nsolids > 0)
-            launch_carve(force_kernel<R>, dim3(overlap ? li.force_blocks_ov : li.force_blocks), dim3(K3_THREADS),
-                         li.force_smem, st, prio, overlap ? li.force_carve_ov : -1, sp, force_args(d, q, p));
+            launch_prio(overlap ? force_kernel<R, 48> : force_kernel<R, 56>, dim3(overlap ? li.force_blocks_ov : li.force_blocks),
+                        dim3(K3_THREADS), li.force_smem, st, prio, sp, force_args(d, q, p));
         if (ev) cudaEventRecord(ev[2], st);
         if (li.tma && li.use_tma)
             lb_tma_kernel<R, S><<<li.lb_blocks, TILE_N, li.lb_smem, st>>>(sp, la, li.tm_f[p], li.tm_c, sp.ntx * sp.nty);

@@ -136,6 +136,10 @@ struct LamEntry {
     float l0h, l0l, l1h, l1l, l2, l3, l4, l5;
 };
 constexpr int LAM_TAB_MAX = 513;  // entries (2 lam_k0 + 1)
+// The same for FP64 arithmetic (24 KB): lambda and five Taylor coefficients in double.
+struct LamEntryD {
+    double l[6];
+};
 
 // K1 walks regions LB_REGION_W nodes wide (rk registry tiles when tile_x is
 // narrower): the push stores of a warp then cover long rows, which keeps the
@@ -202,7 +206,7 @@ struct DevState {
     int *reg_nactive[2];
     void *pool[2];         // per tile: POOL_STRIDE values (layout above)
     void *bfield;          // force_kind 3: body force field, x plane then y plane (nx*ny each)
-    LamEntry *lamtab;      // solid-fraction table (FP32 arithmetic)
+    void *lamtab;          // solid-fraction table (LamEntry in FP32 arithmetic, LamEntryD in FP64)
     int *order;            // solids by decreasing tile side (launch order of the solid kernel)
     unsigned char *busy[2]; // per K1 region, by step parity: 1 if it may hold solid forcing this step
     void *fbody;           // per row: body-force x component
@@ -802,6 +806,14 @@ __device__ __forceinline__ bool fit_window(const RefVals<R, CL> &V, const int *l
     }
     return good;
 }
+
+// v / 3 to a rounding of the result: 1/3 as a float pair in FP32.
+template <class R> __device__ __forceinline__ R third(R v);
+template <> __device__ __forceinline__ float third<float>(float v) {
+    constexpr float hi = 1.0f / 3.0f, lo = (float)(1.0 / 3.0 - (double)hi);
+    return __fmaf_rn(v, hi, __fmul_rn(v, lo));
+}
+template <> __device__ __forceinline__ double third<double>(double v) { return v * (1.0 / 3.0); }
 
 // R^2 as an unevaluated sum hi + lo in precision R (from the host-side split).
 template <class R>
@@ -2054,9 +2066,29 @@ struct ForceArgs {
     const int *reg_count, *reg_solids, *reg_active, *reg_nactive;
     R *pool;
     const SolidDesc *solids;
-    const LamEntry *lamtab;
+    const void *lamtab;
     unsigned *err;
 };
+
+// lambda = 1 - H_eps(phi) to a rounding of the arithmetic, from the table: six
+// fused products where the formula takes a sine and three divisions (in FP64 about
+// 75 operations of a pipe that runs at 1/64 of FP32's rate).
+__device__ __forceinline__ float lambda_tab(const SimParams &sp, const void *tab, float ph, float eps) {
+    if (ph <= -eps) return 1.0f;
+    if (ph >= eps) return 0.0f;
+    const int k = (int)rintf(__fmul_rn(ph, sp.lam_inv_h));
+    const LamEntry *t = static_cast<const LamEntry *>(tab) + (k + sp.lam_k0);
+    const float d = __fmaf_rn(-(float)k, sp.lam_h, ph);  // exact
+    return __fmaf_rn(d, __fmaf_rn(d, __fmaf_rn(d, __fmaf_rn(d, __fmaf_rn(d, t->l5, t->l4), t->l3), t->l2), t->l1h), t->l0h);
+}
+__device__ __forceinline__ double lambda_tab(const SimParams &sp, const void *tab, double ph, double eps) {
+    if (ph <= -eps) return 1.0;
+    if (ph >= eps) return 0.0;
+    const int k = (int)rintf(__fmul_rn((float)ph, sp.lam_inv_h));
+    const double *l = (static_cast<const LamEntryD *>(tab) + (k + sp.lam_k0))->l;
+    const double d = __fma_rn(-whole<double>(k), (double)sp.lam_h, ph);
+    return __fma_rn(d, __fma_rn(d, __fma_rn(d, __fma_rn(d, __fma_rn(d, l[5], l[4]), l[3]), l[2]), l[1]), l[0]);
+}
 
 // Half-edge Jacobian of Eq. 3_3_refmap_jacobian from a 2x3 stencil: a = the
 // node on the low side of the edge, b = the high side, k = 0,1,2 across.
@@ -2064,7 +2096,7 @@ template <class R>
 __device__ __forceinline__ void edge_grad(const R a0, const R a1, const R a2, const R b0, const R b1, const R b2,
                                           R &dn, R &dt) {
     dn = b1 - a1;
-    dt = (b2 + a2 - b0 - a0) / R(4);
+    dt = (b2 + a2 - b0 - a0) * R(0.25);
 }
 
 // Neo-Hookean plane-strain deviatoric stress, Eq. 3_3_solid_stress, for the
@@ -2083,18 +2115,20 @@ __device__ __forceinline__ bool stress_from_grad(R Axx, R Axy, R Ayx, R Ayy, R G
     const R Exx = R(2) * Dxx + (Dxx * Dxx + Dxy * Dxy);
     const R Exy = (Dxy + Dyx) + (Dxx * Dyx + Dxy * Dyy);
     const R Eyy = R(2) * Dyy + (Dyx * Dyx + Dyy * Dyy);
-    txx = G * (R(2) * Exx - Eyy) / R(3);
+    const R G3 = third<R>(G);
+    txx = G3 * (R(2) * Exx - Eyy);
     txy = G * Exy;
-    tyy = G * (R(2) * Eyy - Exx) / R(3);
+    tyy = G3 * (R(2) * Eyy - Exx);
     return true;
 }
 
 // Per-tile constants of the registered solids (static shared memory of K3).
 // Threads per CTA of K3: the 2 tx ty + tx + ty half-edges of a 16x16 tile
 // (544) take two rounds of 288 threads where 256 threads need three.  Four
-// such CTAs fit an SM (48 registers); the overlapped step launches three per
-// SM so that the free regions' K1 runs beside them.  The node phase uses the
-// first TILE_N threads.
+// such CTAs fit an SM.  The node phase uses the first TILE_N threads.
+// Bound by its instructions and barriers: 4096^2 with 1024 disks 129 -> 95 us, 1501 x
+// 1203 with 110 28 -> 23, 506 ellipses 33 -> 28; FP64, bound by its pipe, 1024^2 with 64
+// disks 178 -> 99, the 64^2 cavity 36 -> 23.
 constexpr int K3_THREADS = TILE_N + 32;
 
 template <class R>
@@ -2104,8 +2138,9 @@ struct ForceShared {
     Frame sfr[KMAX];
     R sG[KMAX], sD[KMAX], sA[KMAX];
     float sDh[KMAX], sDl[KMAX];  // rho_s - rho_f as a float pair (the FP32 node terms' Delta rho)
-    Rsq<R> srq[KMAX];
+    Rsq<R> srq[KMAX];            // (the reverse kernel's)
     int sT[KMAX];
+    int bx[KMAX], by[KMAX];      // patch node (0, 0) in the solid's frame (periodic: wrapped)
     long long soff[KMAX];
 };
 
@@ -2121,233 +2156,276 @@ __host__ __device__ __forceinline__ int force_smem_max() {
     return m;
 }
 
+// What a thread of K3 works on in every tile of a shape, found once per CTA: its
+// two patch nodes (column 8 bits, row 6) and its half-edges (patch index of the
+// stencil's first node, 10 bits; x-edges before y-edges), all ones: none.  A tile's
+// code then divides by nothing (half of K3's 1 K instructions per warp and tile were index
+// arithmetic, the formula of lambda, and divisions by 3 and 4).
+constexpr int K3_ROUNDS = 3;  // of K3_THREADS threads: 642 edges and 520 patch nodes at most (128 x 2)
+constexpr unsigned K3_NO_NODE = 0x3fffu, K3_NO_EDGE = 0x3ffu;
+struct ForceMap {
+    unsigned nodes, edges;
+    __device__ __forceinline__ unsigned node(int k) const { return (nodes >> (14 * k)) & K3_NO_NODE; }
+    __device__ __forceinline__ unsigned edge(int k) const { return (edges >> (10 * k)) & K3_NO_EDGE; }
+};
+__device__ __forceinline__ ForceMap force_map(const SimParams &sp) {
+    ForceMap m = {0u, 0u};
+    const int TX = sp.tx, PX = TX + 2, PN = force_patch_n(TX, sp.ty), NXE = (TX + 1) * sp.ty, NE = NXE + TX * (sp.ty + 1);
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const int p = threadIdx.x + k * K3_THREADS;
+        m.nodes |= (p < PN ? (unsigned)((p % PX) | ((p / PX) << 8)) : K3_NO_NODE) << (14 * k);
+    }
+#pragma unroll
+    for (int k = 0; k < K3_ROUNDS; k++) {
+        const int e = threadIdx.x + k * K3_THREADS, f = e - NXE;
+        // x-edge between columns ex - 1 and ex (tile coordinates); y-edge between rows ey - 1 and ey
+        const int p = e < NXE ? (e / (TX + 1)) * PX + e % (TX + 1) : (f >> sp.lx) * PX + (f & (TX - 1));
+        m.edges |= (e < NE ? (unsigned)p : K3_NO_EDGE) << (10 * k);
+    }
+    return m;
+}
+
 // The registered solids of a tile and their descriptors into fs, read by one
 // whole warp (lane k: registry slot k) in parallel; slot = rank of the id (ids
 // are distinct): a fixed summation order.
 template <class R>
 __device__ __forceinline__ void force_solids(const SimParams &sp, const ForceArgs<R> &a, const int tile,
                                              ForceShared<R> &fs, const int k) {
+    const int slot = a.reg_solids[tile * KMAX + (k & (KMAX - 1))];  // read beside the count
     const int n = min(a.reg_count[tile], sp.kmax);
-    const int id = k < n ? a.reg_solids[tile * KMAX + k] : 0x7fffffff;
+    const int id = k < n ? slot : 0x7fffffff;
     int rank = 0;
 #pragma unroll
     for (int m = 0; m < KMAX; m++) rank += __shfl_sync(0xffffffffu, id, m) < id ? 1 : 0;
     if (k < n) {
         const SolidDesc &sd = a.solids[id];
+        const Frame fr = a.frame[id];
         fs.ids[rank] = id;
-        fs.sfr[rank] = a.frame[id];
+        fs.sfr[rank] = fr;
         fs.sG[rank] = pick<R>(sd.G, sd.G_f);
         fs.sD[rank] = pick<R>(sd.drho, sd.drho_f);
         fs.sA[rank] = pick<R>(sd.accel, sd.accel_f);
         fs.sDh[rank] = sd.drho_f;
         fs.sDl[rank] = sd.drho_lo_f;
-        fs.srq[rank] = Rsq<R>(sd);
         fs.sT[rank] = sd.T;
         fs.soff[rank] = sd.off;
+        const int ty = tile / sp.ntx, tx = tile - ty * sp.ntx;
+        const int bx = tx * sp.tx - 1 - fr.ox, by = ty * sp.ty - 1 - fr.oy;
+        fs.bx[rank] = sp.wall_x ? bx : wrapi(bx, sp.nx);
+        fs.by[rank] = sp.wall_y ? by : wrapi(by, sp.ny);
     }
     if (k == 0) fs.nk = n;
+}
+
+// Tile-local coordinates of patch column / row c of a solid (periodic: wrapped).
+__device__ __forceinline__ int patch_local(int b, int c, int wall, int n) {
+    int l = b + c;
+    if (!wall)
+        while (l >= n) l -= n;
+    return l;
 }
 
 // One registered tile of K3.  LOADED: fs already holds the tile's solids (read
 // during the previous tile); else the first warp reads them.  next >= 0: the
 // warp beyond the tile's TILE_N node threads reads the solids of tile `next`
-// into fs_next during the node phase, where it has no node (blockDim.x >=
-// TILE_N + 32).
+// into fs_next during the node phase, where it has no node (blockDim.x ==
+// K3_THREADS).
 template <class R, bool LOADED = false>
-__device__ void force_tile(const SimParams &sp, const ForceArgs<R> &a, const int tile, ForceShared<R> &fs, R *dyn,
-                           const int next = -1, ForceShared<R> *fs_next = nullptr) {
+__device__ void force_tile(const SimParams &sp, const ForceArgs<R> &a, const ForceMap &fm, const int tile,
+                           ForceShared<R> &fs, R *dyn, const int next = -1, ForceShared<R> *fs_next = nullptr) {
     const int TX = sp.tx, PX = TX + 2, PN = force_patch_n(TX, sp.ty);
-    const int NXE = (TX + 1) * sp.ty, NYE = TX * (sp.ty + 1);
+    const int NXE = (TX + 1) * sp.ty;
     R *sX = dyn;                       // [KMAX][PN]
     R *sY = sX + KMAX * PN;
     R *sP = sY + KMAX * PN;
     R *eT = sP + KMAX * PN;            // [(NXE + NYE) * 3] edge stresses
-    int *ids = fs.ids;
-    Frame *sfr = fs.sfr;
-    R *sG = fs.sG, *sD = fs.sD, *sA = fs.sA;
-    Rsq<R> *srq = fs.srq;
-    int *sT = fs.sT;
-    long long *soff = fs.soff;
     const R eps = pick<R>(sp.eps, sp.eps_f), eta = pick<R>(sp.eta, sp.eta_f);
-    {
-        const int tx = tile % sp.ntx, ty = tile / sp.ntx;
-        const int i0 = tx * TX, j0 = ty * sp.ty;
-        if (!LOADED) {
-            if (threadIdx.x < 32) force_solids<R>(sp, a, tile, fs, threadIdx.x);
-            __syncthreads();
-        }
-        const int n = fs.nk;
-        // Stage each solid's xi (and phi) on the tile plus a one-node halo.
-        for (int ks = 0; ks < n; ks++) {
-            const Frame fr = sfr[ks];
-            const int T = sT[ks];
-            const R *Xs = a.xi + soff[ks];
-            // local coordinates of patch node (0, 0) in the solid's frame (periodic: wrapped once here)
-            const int bx0 = sp.wall_x ? i0 - 1 - fr.ox : wrapi(i0 - 1 - fr.ox, sp.nx);
-            const int by0 = sp.wall_y ? j0 - 1 - fr.oy : wrapi(j0 - 1 - fr.oy, sp.ny);
-            BoxWalk wk(PX);
-            for (int p = threadIdx.x; p < PN; p += blockDim.x, wk.next()) {
-                int lx = bx0 + wk.c, ly = by0 + wk.r;
-                if (!sp.wall_x) while (lx >= sp.nx) lx -= sp.nx;
-                if (!sp.wall_y) while (ly >= sp.ny) ly -= sp.ny;
-                R X = nanv<R>(), Y = nanv<R>(), P = nanv<R>();
-                if (in_box(fr, lx, ly)) {
-                    // the three loads at once (the phi plane's address is valid in
-                    // the box); phi counts only where eta does
-                    X = Xs[ly * T + lx];
-                    Y = Xs[T * T + ly * T + lx];
-                    P = Xs[2 * T * T + ly * T + lx];
-                }
-                if (!(X == X)) P = nanv<R>();
-                sX[ks * PN + p] = X; sY[ks * PN + p] = Y; sP[ks * PN + p] = P;
-            }
-        }
+    if (!LOADED) {
+        if (threadIdx.x < 32) force_solids<R>(sp, a, tile, fs, threadIdx.x);
         __syncthreads();
-        // Half-edge stresses: blended solid stress (Eq. 3_6_global_stress) plus contact.
-        for (int e = threadIdx.x; e < NXE + NYE; e += blockDim.x) {
-            int pa[3], pb[3];  // patch indices of the 2x3 stencil (a low side, b high side)
-            const bool xedge = e < NXE;
-            if (xedge) {
-                const int ex = e % (TX + 1), ey = e / (TX + 1);  // edge between col ex-1 and ex (tile coords)
-                for (int k = 0; k < 3; k++) { pa[k] = (ey + k) * PX + ex; pb[k] = (ey + k) * PX + ex + 1; }
-            } else {
-                const int f = e - NXE;
-                const int ex = f % TX, ey = f / TX;               // edge between row ey-1 and ey
-                for (int k = 0; k < 3; k++) { pa[k] = ey * PX + ex + k; pb[k] = (ey + 1) * PX + ex + k; }
+    }
+    const int n = fs.nk;
+    // Stage each solid's xi (and phi) on the tile plus a one-node halo.
+    for (int ks = 0; ks < n; ks++) {
+        const Frame &fr = fs.sfr[ks];
+        const int T = fs.sT[ks], bx = fs.bx[ks], by = fs.by[ks];
+        const R *Xs = a.xi + fs.soff[ks];
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const int c = (int)fm.node(k);
+            if (c == (int)K3_NO_NODE) continue;
+            const int lx = patch_local(bx, c & 255, sp.wall_x, sp.nx);
+            const int ly = patch_local(by, c >> 8, sp.wall_y, sp.ny);
+            R X = nanv<R>(), Y = nanv<R>(), P = nanv<R>();
+            if (in_box(fr, lx, ly)) {
+                // the three loads at once (the phi plane's address is valid in
+                // the box); phi counts only where eta does
+                const R *q = Xs + ly * T + lx;
+                X = q[0];
+                Y = q[T * T];
+                P = q[2 * T * T];
             }
-            R Sxx = 0, Sxy = 0, Syy = 0, L = 0, Cxx = 0, Cxy = 0, Cyy = 0;
-            bool okv[KMAX];
-            R phh[KMAX];
+            if (!(X == X)) P = nanv<R>();
+            const int p = ks * PN + (int)threadIdx.x + k * K3_THREADS;
+            sX[p] = X; sY[p] = Y; sP[p] = P;
+        }
+    }
+    __syncthreads();
+    // Half-edge stresses: blended solid stress (Eq. 3_6_global_stress) plus contact.
+#pragma unroll
+    for (int q = 0; q < K3_ROUNDS; q++) {
+        const int e = threadIdx.x + q * K3_THREADS, p0 = (int)fm.edge(q);
+        if (p0 == (int)K3_NO_EDGE) continue;
+        // the 2x3 stencil: a on the low side at p0 + k al, b on the high side at p0 + ac + k al
+        const bool xedge = e < NXE;
+        const int al = xedge ? PX : 1, ac = xedge ? 1 : PX;
+        R Sxx = 0, Sxy = 0, Syy = 0, L = 0;
+        int near = 0;  // solids whose edge value of phi is below eps
+        for (int ks = 0; ks < n; ks++) {
+            const R *P = sP + ks * PN + p0;
+            const R ph = R(0.5) * (P[al] + P[ac + al]);
+            // beyond the blur zone the solid's stress has weight lambda = 0 in
+            // Eq. 3_6_global_stress: it is not formed (nor its Jacobian checked)
+            if (!(ph < eps)) continue;  // or a node is missing
+            const R *X = sX + ks * PN + p0, *Y = sY + ks * PN + p0;
+            R dXn, dXt, dYn, dYt, txx, txy, tyy;
+            edge_grad<R>(X[0], X[al], X[2 * al], X[ac], X[ac + al], X[ac + 2 * al], dXn, dXt);
+            if (!(dXt == dXt)) continue;  // a node of the stencil is missing
+            near++;
+            edge_grad<R>(Y[0], Y[al], Y[2 * al], Y[ac], Y[ac + al], Y[ac + 2 * al], dYn, dYt);
+            const R lam = lambda_tab(sp, a.lamtab, ph, eps);
+            const R G = fs.sG[ks];
+            // J = d xi / dx = I + d eta / dx (the stored eta excludes the node position)
+            const bool good = stress_from_grad<R>(xedge ? dXn : dXt, xedge ? dXt : dXn, xedge ? dYn : dYt,
+                                                  xedge ? dYt : dYn, G, txx, txy, tyy);
+            if (!good) { atomicOr(a.err, ERR_SINGULAR); continue; }
+            Sxx = fma_rn<R>(lam, txx, Sxx); Sxy = fma_rn<R>(lam, txy, Sxy); Syy = fma_rn<R>(lam, tyy, Syy); L += lam;
+        }
+        if (L > R(1)) { Sxx /= L; Sxy /= L; Syy /= L; }
+        if (near > 1) {  // contact between every pair of them
+            auto edge_phi = [&](int ks, R &ph) {
+                const R *P = sP + ks * PN + p0;
+                ph = R(0.5) * (P[al] + P[ac + al]);
+                const R all = P[0] + P[2 * al] + P[ac] + P[ac + 2 * al];
+                return ph < eps && all == all;
+            };
+            R Cxx = 0, Cxy = 0, Cyy = 0;
             for (int ks = 0; ks < n; ks++) {
-                const R *X = sX + ks * PN, *Y = sY + ks * PN, *P = sP + ks * PN;
-                bool ok = true;
-                for (int k = 0; k < 3; k++) ok = ok && (P[pa[k]] == P[pa[k]]) && (P[pb[k]] == P[pb[k]]);
-                okv[ks] = ok;
-                if (!ok) continue;
-                const R ph = R(0.5) * (P[pa[1]] + P[pb[1]]);
-                phh[ks] = ph;
-                // beyond the blur zone the solid's stress has weight lambda = 0 in
-                // Eq. 3_6_global_stress: it is not formed (nor its Jacobian checked)
-                if (!(ph < eps)) continue;
-                const R lam = R(1) - heaviside<R>(ph, eps);
-                R dXn, dXt, dYn, dYt, txx, txy, tyy;
-                edge_grad<R>(X[pa[0]], X[pa[1]], X[pa[2]], X[pb[0]], X[pb[1]], X[pb[2]], dXn, dXt);
-                edge_grad<R>(Y[pa[0]], Y[pa[1]], Y[pa[2]], Y[pb[0]], Y[pb[1]], Y[pb[2]], dYn, dYt);
-                const R G = sG[ks];
-                // J = d xi / dx = I + d eta / dx (the stored eta excludes the node position)
-                const bool good = xedge ? stress_from_grad<R>(dXn, dXt, dYn, dYt, G, txx, txy, tyy)
-                                        : stress_from_grad<R>(dXt, dXn, dYt, dYn, G, txx, txy, tyy);
-                if (!good) { atomicOr(a.err, ERR_SINGULAR); continue; }
-                Sxx += lam * txx; Sxy += lam * txy; Syy += lam * tyy; L += lam;
-            }
-            for (int ks = 0; ks < n; ks++) {
-                if (!okv[ks] || !(phh[ks] < eps)) continue;
+                R phs, pht;
+                if (!edge_phi(ks, phs)) continue;
                 for (int kt = ks + 1; kt < n; kt++) {
-                    if (!okv[kt] || !(phh[kt] < eps)) continue;
-                    const R fs = R(0.5) * (R(1) - phh[ks] / eps), ft = R(0.5) * (R(1) - phh[kt] / eps);
-                    const R fm = fs < ft ? fs : ft;
-                    const R *Ps = sP + ks * PN, *Pt = sP + kt * PN;
+                    if (!edge_phi(kt, pht)) continue;
+                    const R f_s = R(0.5) * (R(1) - phs / eps), f_t = R(0.5) * (R(1) - pht / eps);
+                    const R fmn = f_s < f_t ? f_s : f_t;
+                    const R *Ps = sP + ks * PN + p0, *Pt = sP + kt * PN + p0;
                     R gn, gt;
-                    edge_grad<R>(Ps[pa[0]] - Pt[pa[0]], Ps[pa[1]] - Pt[pa[1]], Ps[pa[2]] - Pt[pa[2]],
-                                 Ps[pb[0]] - Pt[pb[0]], Ps[pb[1]] - Pt[pb[1]], Ps[pb[2]] - Pt[pb[2]], gn, gt);
+                    edge_grad<R>(Ps[0] - Pt[0], Ps[al] - Pt[al], Ps[2 * al] - Pt[2 * al], Ps[ac] - Pt[ac],
+                                 Ps[ac + al] - Pt[ac + al], Ps[ac + 2 * al] - Pt[ac + 2 * al], gn, gt);
                     const R gxx = xedge ? gn : gt, gyy = xedge ? gt : gn;
                     const R nrm = rsqrt_<R>(gxx * gxx + gyy * gyy);
                     if (nrm == R(0)) continue;
                     const R nx_ = gxx / nrm, ny_ = gyy / nrm;
-                    const R kk = -eta * fm * (sG[ks] + sG[kt]);
+                    const R kk = -eta * fmn * (fs.sG[ks] + fs.sG[kt]);
                     Cxx += kk * (nx_ * nx_ - R(0.5)); Cxy += kk * (nx_ * ny_); Cyy += kk * (ny_ * ny_ - R(0.5));
                 }
             }
-            if (L > R(1)) { Sxx /= L; Sxy /= L; Syy /= L; }
-            eT[3 * e + 0] = Sxx + Cxx; eT[3 * e + 1] = Sxy + Cxy; eT[3 * e + 2] = Syy + Cyy;
+            Sxx += Cxx; Sxy += Cxy; Syy += Cyy;
         }
-        __syncthreads();
-        // Node: divergence (Eq. 3_3_div_solid_stress), solid fraction, drho, solid acceleration.
-        // Meanwhile the warp past the node threads reads the next tile's solids.
-        if (next >= 0 && threadIdx.x >= TILE_N && threadIdx.x < TILE_N + 32)
-            force_solids<R>(sp, a, next, *fs_next, threadIdx.x - TILE_N);
-        {
-            const int cx = threadIdx.x & (TX - 1), cy = threadIdx.x >> sp.lx;
-            const int i = i0 + cx, j = j0 + cy;
-            if (threadIdx.x < TILE_N && i < sp.nx && j < sp.ny) {
-                const R *tl = eT + 3 * (cy * (TX + 1) + cx), *tr = eT + 3 * (cy * (TX + 1) + cx + 1);
-                const R *tb = eT + 3 * (NXE + cy * TX + cx), *tt = eT + 3 * (NXE + (cy + 1) * TX + cx);
-                const R fsx = (tr[0] - tl[0]) + (tt[1] - tb[1]);
-                const R fsy = (tr[1] - tl[1]) + (tt[2] - tb[2]);
-                const int p = (cy + 1) * PX + cx + 1;
-                R L = 0, Ay = 0, Dh = 0, Dl = 0;
-                if constexpr (sizeof(R) == 4) {
-                    // Delta rho = sum lambda (rho_s - rho_f) is an O(1) number whose
-                    // rounding would drive the pressure: lambda comes as a float pair
-                    // from the level set's pair (the relabel's low part) in and near
-                    // the blur zone, exactly 0 or 1 elsewhere; float-float sums
-                    float Lh = 0.0f, Ll = 0.0f;
-                    for (int ks = 0; ks < n; ks++) {
-                        const R ph = sP[ks * PN + p];
-                        if (!(ph == ph)) continue;
-                        float lh = 0.0f, ll = 0.0f;
-                        // phi's low part exists where |phi| < eps + PHI_D_SHELL (the relabel's
-                        // test, on its FP32 phi); within half that shell it is read
-                        if (ph <= -eps - R(0.5f * PHI_D_SHELL)) lh = 1.0f;
-                        else if (ph < eps + R(0.5f * PHI_D_SHELL)) {
-                            const Frame &fr = sfr[ks];
-                            const int lx = sp.wall_x ? i - fr.ox : wrapi(i - fr.ox, sp.nx);
-                            const int ly = sp.wall_y ? j - fr.oy : wrapi(j - fr.oy, sp.ny);
-                            const int T = sT[ks];
-                            lambda_ff(sp, a.lamtab, ph, a.xi[soff[ks] + 5 * T * T + ly * T + lx], lh, ll);
-                        }
-                        if (lh == 0.0f) continue;
-                        L += lh;
-                        Ay += lh * sA[ks];
-                        ff_add(Lh, Ll, lh, ll);
-                        ff_add_prod(Dh, Dl, lh, ll, fs.sDh[ks], fs.sDl[ks]);
-                    }
-                    if (Lh + Ll > 1.0f) ff_div(Dh, Dl, Lh, Ll);
-                } else {
-                    double Ld = 0.0, Dd = 0.0;
-                    for (int ks = 0; ks < n; ks++) {
-                        const R ph = sP[ks * PN + p];
-                        if (!(ph == ph)) continue;
-                        const R lam = R(1) - heaviside<R>(ph, eps);
-                        L += lam;
-                        Ay += lam * sA[ks];
-                        Ld += lam;
-                        Dd += lam * sD[ks];
-                    }
-                    if (Ld > 1.0) Dd /= Ld;
-                    Dh = R(Dd);
-                }
-                if (L > R(1)) Ay /= L;
-                R *po = a.pool + (long long)tile * POOL_STRIDE + threadIdx.x;
-                po[POOL_FX] = fsx;
-                if (sp.force_mode == 1) {
-                    po[POOL_FY] = fsy;
-                    po[POOL_AY] = Ay;
-                } else {
-                    po[POOL_FY] = fsy + Ay;
-                }
-                R *pd = a.pool + (long long)tile * POOL_STRIDE + POOL_DRHO + 2 * threadIdx.x;
-                pd[0] = Dh;
-                pd[1] = Dl;
-            }
-        }
-        __syncthreads();
+        eT[3 * e + 0] = Sxx; eT[3 * e + 1] = Sxy; eT[3 * e + 2] = Syy;
     }
+    __syncthreads();
+    // Node: divergence (Eq. 3_3_div_solid_stress), solid fraction, drho, solid acceleration.
+    // Meanwhile the warp past the node threads reads the next tile's solids.
+    if (next >= 0 && threadIdx.x >= TILE_N && threadIdx.x < TILE_N + 32)
+        force_solids<R>(sp, a, next, *fs_next, threadIdx.x - TILE_N);
+    {
+        const int cx = threadIdx.x & (TX - 1), cy = threadIdx.x >> sp.lx;
+        const int ty = tile / sp.ntx, tx = tile - ty * sp.ntx;
+        const int i = tx * TX + cx, j = ty * sp.ty + cy;
+        if (threadIdx.x < TILE_N && i < sp.nx && j < sp.ny) {
+            const R *tl = eT + 3 * (cy * (TX + 1) + cx), *tr = eT + 3 * (cy * (TX + 1) + cx + 1);
+            const R *tb = eT + 3 * (NXE + cy * TX + cx), *tt = eT + 3 * (NXE + (cy + 1) * TX + cx);
+            const R fsx = (tr[0] - tl[0]) + (tt[1] - tb[1]);
+            const R fsy = (tr[1] - tl[1]) + (tt[2] - tb[2]);
+            const int p = (cy + 1) * PX + cx + 1;
+            R L = 0, Ay = 0, Dh = 0, Dl = 0;
+            if constexpr (sizeof(R) == 4) {
+                // Delta rho = sum lambda (rho_s - rho_f) is an O(1) number whose
+                // rounding would drive the pressure: lambda comes as a float pair
+                // from the level set's pair (the relabel's low part) in and near
+                // the blur zone, exactly 0 or 1 elsewhere; float-float sums
+                float Lh = 0.0f, Ll = 0.0f;
+                for (int ks = 0; ks < n; ks++) {
+                    const R ph = sP[ks * PN + p];
+                    if (!(ph == ph)) continue;
+                    float lh = 0.0f, ll = 0.0f;
+                    // phi's low part exists where |phi| < eps + PHI_D_SHELL (the relabel's
+                    // test, on its FP32 phi); within half that shell it is read
+                    if (ph <= -eps - R(0.5f * PHI_D_SHELL)) lh = 1.0f;
+                    else if (ph < eps + R(0.5f * PHI_D_SHELL)) {
+                        const int lx = patch_local(fs.bx[ks], cx + 1, sp.wall_x, sp.nx);
+                        const int ly = patch_local(fs.by[ks], cy + 1, sp.wall_y, sp.ny);
+                        const int T = fs.sT[ks];
+                        lambda_ff(sp, static_cast<const LamEntry *>(a.lamtab), ph, a.xi[fs.soff[ks] + 5 * T * T + ly * T + lx],
+                                  lh, ll);
+                    }
+                    if (lh == 0.0f) continue;
+                    L += lh;
+                    Ay += lh * fs.sA[ks];
+                    ff_add(Lh, Ll, lh, ll);
+                    ff_add_prod(Dh, Dl, lh, ll, fs.sDh[ks], fs.sDl[ks]);
+                }
+                if (Lh + Ll > 1.0f) ff_div(Dh, Dl, Lh, Ll);
+            } else {
+                double Ld = 0.0, Dd = 0.0;
+                for (int ks = 0; ks < n; ks++) {
+                    const R ph = sP[ks * PN + p];
+                    if (!(ph < eps)) continue;
+                    const R lam = lambda_tab(sp, a.lamtab, ph, eps);
+                    L += lam;
+                    Ay += lam * fs.sA[ks];
+                    Ld += lam;
+                    Dd += lam * fs.sD[ks];
+                }
+                if (Ld > 1.0) Dd /= Ld;
+                Dh = R(Dd);
+            }
+            if (L > R(1)) Ay /= L;
+            R *po = a.pool + (long long)tile * POOL_STRIDE + threadIdx.x;
+            po[POOL_FX] = fsx;
+            if (sp.force_mode == 1) {
+                po[POOL_FY] = fsy;
+                po[POOL_AY] = Ay;
+            } else {
+                po[POOL_FY] = fsy + Ay;
+            }
+            R *pd = a.pool + (long long)tile * POOL_STRIDE + POOL_DRHO + 2 * threadIdx.x;
+            pd[0] = Dh;
+            pd[1] = Dl;
+        }
+    }
+    __syncthreads();
 }
 
-template <class R>
-__global__ void __launch_bounds__(K3_THREADS) __maxnreg__(sizeof(R) == 4 ? 48 : 224) force_kernel(SimParams sp, ForceArgs<R> a) {
+// REGS (FP32): 56 registers hold the tile's code without spills, four CTAs on an
+// SM; in the overlapped step 48 leave room for a CTA of the free regions' K1 beside the
+// four, which there is worth more (4096^2 suspension: K3 alone 95 against 102 us, the
+// step 474-478 against 465).
+template <class R, int REGS>
+__global__ void __launch_bounds__(K3_THREADS) __maxnreg__(sizeof(R) == 4 ? REGS : 224) force_kernel(SimParams sp, ForceArgs<R> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ ForceShared<R> fs[2];  // this tile's solids, and the next tile's (read during this one)
-    const int nact = *a.reg_nactive;
     int it = blockIdx.x;
+    int tile = it < sp.ntx * sp.nty ? a.reg_active[it] : 0;  // read beside the count
+    const int nact = *a.reg_nactive;
     if (it >= nact) return;  // uniform over the CTA
-    int tile = a.reg_active[it];
+    const ForceMap fm = force_map(sp);
     if (threadIdx.x < 32) force_solids<R>(sp, a, tile, fs[0], threadIdx.x);
     __syncthreads();
     for (int b = 0; it < nact; it += gridDim.x, b ^= 1) {
         const int next = it + (int)gridDim.x < nact ? a.reg_active[it + gridDim.x] : -1;
-        force_tile<R, true>(sp, a, tile, fs[b], reinterpret_cast<R *>(smem), next, &fs[b ^ 1]);
+        force_tile<R, true>(sp, a, fm, tile, fs[b], reinterpret_cast<R *>(smem), next, &fs[b ^ 1]);
         tile = next;
     }
 }
@@ -2374,14 +2452,6 @@ struct LbArgs {
     const R *pool_prev;        // force pool of the previous step (its Delta rho is the rest base)
     unsigned *err;
 };
-
-// v / 3 to a rounding of the result: 1/3 as a float pair in FP32.
-template <class R> __device__ __forceinline__ R third(R v);
-template <> __device__ __forceinline__ float third<float>(float v) {
-    constexpr float hi = 1.0f / 3.0f, lo = (float)(1.0 / 3.0 - (double)hi);
-    return __fmaf_rn(v, hi, __fmul_rn(v, lo));
-}
-template <> __device__ __forceinline__ double third<double>(double v) { return v * (1.0 / 3.0); }
 
 // The arithmetic of one node of K1 once its inputs are loaded: moments, SFC
 // equilibrium, Guo forcing and BGK collision.  f: the stored populations (f[0]
