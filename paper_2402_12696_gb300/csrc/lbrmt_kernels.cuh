@@ -39,11 +39,13 @@ constexpr int RMT_THREADS = 256;
 constexpr int TILE_SIDE_MAX = 448;          // largest solid tile side
 // Shared memory of K2: the solid's sets as one bit per tile node (row masks
 // below), then lists (ints: pass 0's nodes per warp, each layer's targets), and
-// in its wide form the reference map of the CTA's strip of rows.
+// in its wide form the plans of two layers' fits and the reference map of the
+// CTA's strip of rows.
 constexpr int RMT_MASKS = 5;                // S, layers <= 2, and three in rotation
+constexpr int RMT_MASKS_WIDE = 6;           // and four: the wide form dilates two layers ahead
 constexpr int RMT_LIST_BYTES = 6144;        // list space of a 256-thread CTA
 constexpr int RMT_LIST_MIN_BYTES = 4096;    // least (128 nodes per warp) list space for which K2 takes a smaller carveout
-constexpr int RMT_WIDE_LIST_BYTES = 16384;  // list space of a CTA that has its SM to itself
+constexpr int RMT_WIDE_LIST_BYTES = 12288;  // list space of the wide form: three layers' targets
 constexpr int RMT_SMEM_CAP = 227 * 1024;    // largest dynamic shared memory of a CTA
 __host__ __device__ constexpr int mask_row_words(int T) { return ((T + 34) >> 5) + 1; }
 // Rows of a set: the tile's, or of a strip of a cluster of nc CTAs with the
@@ -56,8 +58,12 @@ __host__ __device__ constexpr int rmt_mask_bytes(int T, int nc, int NL) { return
 // The wide form's set of pass 0 (the CTA's rows of the input box) and its map (two halo rows on either side).
 __host__ __device__ constexpr int strip_mask_words(int T, int nc) { return (((T + nc - 1) / nc + 1) * mask_row_words(T) + 3) & ~3; }
 __host__ __device__ constexpr int strip_values(int T, int nc) { return ((T + nc - 1) / nc + 5) * T; }
+// Targets of a layer in one CTA whose fits are planned ahead (more: planned in place).
+__host__ __device__ constexpr int plan_cap(int real) { return real == 4 ? 256 : 128; }
+__host__ __device__ constexpr int plan_bytes(int real) { return real == 4 ? 48 : 80; }  // sizeof(FitRec)
 __host__ __device__ constexpr int rmt_wide_smem(int T, int nc, int NL, int real) {
-    return rmt_mask_bytes(T, nc, NL) + 4 * strip_mask_words(T, nc) + RMT_WIDE_LIST_BYTES + 2 * real * strip_values(T, nc);
+    return RMT_MASKS_WIDE * 4 * mask_words(T, nc, NL) + 4 * strip_mask_words(T, nc) + RMT_WIDE_LIST_BYTES +
+           2 * plan_cap(real) * plan_bytes(real) + 2 * real * strip_values(T, nc);
 }
 constexpr int RMT_SMEM_MAX = rmt_mask_bytes(TILE_SIDE_MAX, 1, 20) + RMT_LIST_BYTES;
 // Shared memory of the reverse sweep's K2: byte labels and layer lists.
@@ -426,6 +432,8 @@ __device__ __forceinline__ int cluster_size() { unsigned r; asm("mov.u32 %0, %%c
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ unsigned cluster_addr(const void *p, int rank) {
     unsigned a;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
@@ -689,74 +697,60 @@ template <> struct FitCoef<double> {
     }
 };
 
-// The fitted value at one target (Sec. 3.2, steps (i)-(iii)) by a group of LPT
-// lanes, the rows of its 5x5 window dealt out over them; XY: twice that,
-// one half for each coordinate (FP64).  value = ref + sum_k w_k (c13 dx + c23 dy
-// + c33) (X_k - ref) / det with the cofactors of M's last row, over the valid
-// nodes (bits m).  The fit is of differences from the value at the target's
-// 4-neighbour in the layer before (a valid node by construction), which keeps
-// the sums small.  Without directional weights (use_n: layers 1 and 2, weights
-// 2^-(|dx|+|dy|) max(0, d.n) / |d|, (gx, gy) along n; a common factor of the weights
-// drops out, so n is not normalised; wd: 2^-(|dx|+|dy|) / |d|) the cofactors come from the validity bits
-// alone, exactly.  A layer takes as long as this chain, so its loads do not wait
-// for one another: every node of a row is loaded, one that does not count from
-// the reference's address (its difference is then zero).
-// False if the window does not define the plane.  The group's lanes call together.
-template <class R, bool CL, int LPT, bool XY>
-__device__ __forceinline__ bool fit_window(const RefVals<R, CL> &V, const int *lut, const R *wd, unsigned m, int x, int y,
-                                           bool use_n, R gx, R gy, R &ox, R &oy) {
-    const int q = threadIdx.x & (LPT - 1), c = XY ? (threadIdx.x / LPT) & 1 : 0;
-    constexpr int G = XY ? 2 * LPT : LPT;
-    const unsigned gm = (0xffffffffu >> (32 - G)) << (threadIdx.x & 31 & ~(G - 1));
-    const int t = V.at(x, y);
-    const int kref = (m >> 11) & 1u ? t - 1 : ((m >> 13) & 1u ? t + 1 : ((m >> 7) & 1u ? t - V.stride : t + V.stride));
-    constexpr int NR = (4 + LPT) / LPT;  // rows per lane
-    R xref, yref, ax[NR], ay[NR], det;
-    if constexpr (XY) xref = V.get(kref, c);
-    else V.get2(kref, xref, yref);
-    bool good;
-    auto add = [&](int i, bool on, int k, R g) {
-        if constexpr (XY) {
-            ax[i] = fma_rn<R>(g, V.get(on ? k : kref, c) - xref, ax[i]);
-        } else {
-            R vx, vy;
-            V.get2_if(on, k, kref, xref, yref, vx, vy);
-            ax[i] = fma_rn<R>(g, vx - xref, ax[i]);
-            ay[i] = fma_rn<R>(g, vy - yref, ay[i]);
-        }
-    };
+// A fit up to the values (Sec. 3.2, steps (i)-(iii)): the extrapolated value is
+//   ref + sum_k w_k (c13 dx + c23 dy + c33) (X_k - ref) / det
+// over the nodes that count, with the cofactors of the last row of the normal
+// matrix M = sum_k w_k (dx, dy, 1) (dx, dy, 1)^T, a function of the sets and of phi^n alone.  The
+// fit is of differences from the value at the target's 4-neighbour in the layer
+// before (a valid node by construction), which keeps the sums small.
+//   Layers beyond the second: w = 2^-(|dx| + |dy|); M follows from the window's 25 validity
+//   bits in whole numbers, so do det and the cofactors (i13, i23, i33).
+//   Layers 1 and 2, where a normal (gx, gy) of phi^n is to be had: w times max(0,
+//   d.n) / |d|, d = target - node (a common factor of the weights drops out, so n is
+//   not normalised).
+template <class R>
+struct FitPlan {
+    R c13, c23, c33;  // directional
+    R gx, gy, rdet;   // rdet: 1 / det
     int i13, i23, i33;
-#pragma unroll
-    for (int i = 0; i < NR; i++) ax[i] = ay[i] = R(0);
+    unsigned bits;    // the nodes that count (25), FIT_DIR, FIT_NONE; and the valid ones' reference
+};
+template <class R>
+struct alignas(16) FitRec {
+    FitPlan<R> f;
+    int e;  // the target: x | y << 16
+};
+static_assert(sizeof(FitRec<float>) == plan_bytes(4) && sizeof(FitRec<double>) == plan_bytes(8), "plan_bytes");
+constexpr unsigned FIT_DIR = 1u << 25, FIT_NONE = 1u << 26;  // directional weights; the window defines no plane
+constexpr int FIT_REF = 27;                                  // reference node: 0 left, 1 right, 2 up, 3 down
+
+// By a group of LPT lanes, the window's rows dealt out over them (every lane
+// gets the whole plan).  m: the valid nodes of the window.
+template <class R, int LPT>
+__device__ __forceinline__ void fit_plan(const int *lut, const R *wd, unsigned m, bool use_n, R gx, R gy, unsigned gm,
+                                         FitPlan<R> &f) {
+    const int q = threadIdx.x & (LPT - 1);
+    const unsigned ref = (m >> 11) & 1u ? 0u : ((m >> 13) & 1u ? 1u : ((m >> 7) & 1u ? 2u : 3u));
+    R det;
     if (!use_n) {
-        const int idet = window_moments(lut, m, i13, i23, i33);
-        good = idet != 0;
+        const int idet = window_moments(lut, m, f.i13, f.i23, f.i33);
         det = whole<R>(idet);
-        const FitCoef<R> fc(i13, i23, i33);
-#pragma unroll
-        for (int i = 0; i < NR; i++) {
-            const int d = i * LPT + q, dy = d - 2;  // d >= 5: no row
-            const unsigned r = d < 5 ? (m >> (5 * d)) & 31u : 0u;
-            if (!CL && r == 0u) continue;
-            const int k = t + dy * V.stride;
-            const auto row = fc.row(dy), col = fc.col(dy);
-#pragma unroll
-            for (int dx = -2; dx <= 2; dx++) add(i, (r >> (dx + 2)) & 1u, k + dx, FitCoef<R>::at(row, col, dx));
-        }
+        f.bits = m | (idet != 0 ? 0u : FIT_NONE);
     } else {
+        constexpr int NR = (4 + LPT) / LPT;  // rows per lane
         const float gxf = (float)gx, gyf = (float)gy, lim = (float)COS_TIE * sqrtf(gxf * gxf + gyf * gyf);
         R s0[NR], s1[NR], s2[NR];
         unsigned pos = 0;
 #pragma unroll
         for (int i = 0; i < NR; i++) {
-            const int d = i * LPT + q, dy = d - 2;
+            const int d = i * LPT + q, dy = d - 2;  // d >= 5: no row
             const unsigned r = d < 5 ? (m >> (5 * d)) & 31u : 0u;
             const R *w = wd + 5 * (d < 5 ? d : 0);
             const R dygy = R(dy) * gy;
             s0[i] = s1[i] = s2[i] = R(0);
 #pragma unroll
             for (int dx = -2; dx <= 2; dx++) {
-                // d.n times |d| |n|, d = target - node; a cosine up to COS_TIE counts as zero
+                // d.n times |d| |n|; a cosine up to COS_TIE counts as zero
                 const R dn = -fma_rn<R>(R(dx), gx, dygy);
                 const bool p = ((r >> (dx + 2)) & 1u) && above(dn, lim * sqrtf((float)(dx * dx) + (float)(dy * dy)));
                 const R wt = p ? dn * w[dx + 2] : R(0);
@@ -772,39 +766,84 @@ __device__ __forceinline__ bool fit_window(const RefVals<R, CL> &V, const int *l
             const R dy = R(i * LPT + q - 2);
             y1[i] = dy * s1[i]; y0[i] = dy * s0[i]; y2[i] = dy * y0[i];
         }
-        const R a = row_sum<LPT>(gm, s2), b = row_sum<LPT>(gm, y1), cc = row_sum<LPT>(gm, s1);
-        const R d_ = row_sum<LPT>(gm, y2), e = row_sum<LPT>(gm, y0), fw = row_sum<LPT>(gm, s0);
+        const R a = row_sum<LPT>(gm, s2), b = row_sum<LPT>(gm, y1), c = row_sum<LPT>(gm, s1);
+        const R d = row_sum<LPT>(gm, y2), e = row_sum<LPT>(gm, y0), fw = row_sum<LPT>(gm, s0);
 #pragma unroll
-        for (int d = 1; d < LPT; d <<= 1) pos |= __shfl_xor_sync(gm, pos, d);
-        const R c13 = fma_rn<R>(b, e, -mul_rn<R>(cc, d_)), c23 = fma_rn<R>(b, cc, -mul_rn<R>(a, e)),
-                c33 = fma_rn<R>(a, d_, -mul_rn<R>(b, b));
-        det = fma_rn<R>(cc, c13, fma_rn<R>(e, c23, mul_rn<R>(fw, c33)));
-        good = window_moments(lut, pos, i13, i23, i33) != 0 && det != R(0);
+        for (int k = 1; k < LPT; k <<= 1) pos |= __shfl_xor_sync(gm, pos, k);
+        f.c13 = fma_rn<R>(b, e, -mul_rn<R>(c, d));
+        f.c23 = fma_rn<R>(b, c, -mul_rn<R>(a, e));
+        f.c33 = fma_rn<R>(a, d, -mul_rn<R>(b, b));
+        f.gx = gx;
+        f.gy = gy;
+        det = fma_rn<R>(c, f.c13, fma_rn<R>(e, f.c23, mul_rn<R>(fw, f.c33)));
+        int i13, i23, i33;
+        f.bits = pos | FIT_DIR | (window_moments(lut, pos, i13, i23, i33) != 0 && det != R(0) ? 0u : FIT_NONE);
+    }
+    f.rdet = R(1) / det;
+    f.bits |= ref << FIT_REF;
+}
+
+// The values of a plan at the target (x, y), by LPT lanes, or (XY) twice that, one
+// half for each coordinate (FP64).  wd: 2^-(|dx|+|dy|) / |d|.  Every node of a row is
+// loaded (a node that does not count gives the reference's value: a zero
+// difference), so that no load waits for another.
+template <class R, bool CL, int LPT, bool XY>
+__device__ __forceinline__ void fit_values(const RefVals<R, CL> &V, const R *wd, const FitPlan<R> &f, int x, int y,
+                                           unsigned gm, R &ox, R &oy) {
+    constexpr int NR = (4 + LPT) / LPT;  // rows per lane
+    const int q = threadIdx.x & (LPT - 1), c = XY ? (threadIdx.x / LPT) & 1 : 0;
+    const int t = V.at(x, y), rf = f.bits >> FIT_REF, step = rf < 2 ? 1 : V.stride, kref = (rf == 0 || rf == 2) ? t - step : t + step;
+    R xref, yref, ax[NR], ay[NR];
+    if constexpr (XY) xref = V.get(kref, c);
+    else V.get2(kref, xref, yref);
+    auto add = [&](int i, bool on, int k, R g) {
+        if constexpr (XY) {
+            ax[i] = fma_rn<R>(g, V.get(on ? k : kref, c) - xref, ax[i]);
+        } else {
+            R vx, vy;
+            V.get2_if(on, k, kref, xref, yref, vx, vy);
+            ax[i] = fma_rn<R>(g, vx - xref, ax[i]);
+            ay[i] = fma_rn<R>(g, vy - yref, ay[i]);
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < NR; i++) ax[i] = ay[i] = R(0);
+    if (!(f.bits & FIT_DIR)) {
+        const FitCoef<R> fc(f.i13, f.i23, f.i33);
+#pragma unroll
+        for (int i = 0; i < NR; i++) {
+            const int d = i * LPT + q, dy = d - 2;  // d >= 5: no row
+            const unsigned r = d < 5 ? (f.bits >> (5 * d)) & 31u : 0u;
+            if (!CL && r == 0u) continue;
+            const int k = t + dy * V.stride;
+            const auto row = fc.row(dy), col = fc.col(dy);
+#pragma unroll
+            for (int dx = -2; dx <= 2; dx++) add(i, (r >> (dx + 2)) & 1u, k + dx, FitCoef<R>::at(row, col, dx));
+        }
+    } else {
 #pragma unroll
         for (int i = 0; i < NR; i++) {
             const int d = i * LPT + q, dy = d - 2;
-            const unsigned r = d < 5 ? (pos >> (5 * d)) & 31u : 0u;
+            const unsigned r = d < 5 ? (f.bits >> (5 * d)) & 31u : 0u;
             if (!CL && r == 0u) continue;
             const int k = t + dy * V.stride;
             const R *w = wd + 5 * (d < 5 ? d : 0);
-            const R base = fma_rn<R>(R(dy), c23, c33), dygy = R(dy) * gy;
+            const R base = fma_rn<R>(R(dy), f.c23, f.c33), dygy = R(dy) * f.gy;
 #pragma unroll
             for (int dx = -2; dx <= 2; dx++)
                 add(i, (r >> (dx + 2)) & 1u, k + dx,
-                    mul_rn<R>(mul_rn<R>(-fma_rn<R>(R(dx), gx, dygy), w[dx + 2]), fma_rn<R>(R(dx), c13, base)));
+                    mul_rn<R>(mul_rn<R>(-fma_rn<R>(R(dx), f.gx, dygy), w[dx + 2]), fma_rn<R>(R(dx), f.c13, base)));
         }
     }
     const R sx = row_sum<LPT>(gm, ax);
     if constexpr (XY) {
-        const R v = xref + sx / det, w = __shfl_xor_sync(gm, v, LPT);
+        const R v = fma_rn<R>(sx, f.rdet, xref), w = __shfl_xor_sync(gm, v, LPT);
         ox = c ? w : v;
         oy = c ? v : w;
     } else {
-        const R sy = row_sum<LPT>(gm, ay);
-        ox = xref + sx / det;
-        oy = yref + sy / det;
+        ox = fma_rn<R>(sx, f.rdet, xref);
+        oy = fma_rn<R>(row_sum<LPT>(gm, ay), f.rdet, yref);
     }
-    return good;
 }
 
 // v / 3 to a rounding of the result: 1/3 as a float pair in FP32.
@@ -1523,12 +1562,16 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     const int NL = sp.n_layers;
     const int T = sd.T, TT = T * T, rw = mask_row_words(T), mw = mask_words(T, nc, NL);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    constexpr int NM = CL ? RMT_MASKS_WIDE : RMT_MASKS, NLIST = CL ? 3 : 2;
     unsigned *masks = reinterpret_cast<unsigned *>(smem);
     const int m0w = CL ? strip_mask_words(T, nc) : 0;
-    int *lists = reinterpret_cast<int *>(masks + RMT_MASKS * mw + m0w);
+    int *lists = reinterpret_cast<int *>(masks + NM * mw + m0w);
     unsigned dsm;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
-    const int list_ints = CL ? RMT_WIDE_LIST_BYTES / 4 : ((int)dsm >> 2) - RMT_MASKS * mw, layer_cap = list_ints >> 1;
+    const int list_ints = CL ? RMT_WIDE_LIST_BYTES / 4 : ((int)dsm >> 2) - NM * mw, layer_cap = list_ints / NLIST;
+    auto list_of = [&](int l) { return lists + (CL ? l % 3 : (l & 1)) * layer_cap; };
+    FitRec<R> *plans = reinterpret_cast<FitRec<R> *>(lists + list_ints);  // CL
+    constexpr int PCAP = plan_cap((int)sizeof(R));
     auto solid_sync = [&]() {
         if constexpr (CL) cluster_sync();
         else __syncthreads();
@@ -1556,7 +1599,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
         wd[tid - 32] = pow2neg<R>(abs(dx) + abs(dy)) * rinv_tab<R>(dx, dy);
     }
     if (xi_planes<R>() == 6 && sd.shape != 0 && tid == (int)blockDim.x - 1) shape_consts(sd, shp);
-    for (int k = tid; k < (RMT_MASKS * mw + m0w) / 4; k += blockDim.x) reinterpret_cast<int4 *>(masks)[k] = make_int4(0, 0, 0, 0);
+    for (int k = tid; k < (NM * mw + m0w) / 4; k += blockDim.x) reinterpret_cast<int4 *>(masks)[k] = make_int4(0, 0, 0, 0);
     int acc[3] = {0, 0, 0};
     int sb[4] = {1 << 29, -(1 << 29), 1 << 29, -(1 << 29)};
     __syncthreads();
@@ -1569,7 +1612,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     const int jr0 = jb0 + (CL ? ih * rank / nc : 0), jr1 = jb0 + (CL ? ih * (rank + 1) / nc : ih);
     const int bn = bw * (jr1 - jr0);
     // the set S as this pass finds it: rows of the output tile (CL: the strip's alone)
-    const RowMask mP = {CL ? masks + RMT_MASKS * mw : masks, rw, CL ? jr0 - shy : -2};
+    const RowMask mP = {CL ? masks + NM * mw : masks, rw, CL ? jr0 - shy : -2};
     if (a.init) {
         const Rsq<R> rq(sd);
         BoxWalk wk(bw);
@@ -1673,16 +1716,16 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     const int x0 = max(sx0 - NL, cx0), x1 = min(sx1 + NL, cx1), y0 = max(sy0 - NL, cy0), y1 = min(sy1 + NL, cy1);
     const Strips st = {y0, any ? y1 : y0 - 1, 31 - __clz(nc), NL};  // nc: a power of two
     const int yr0 = st.first(rank), yr1 = st.first(rank + 1);
-    // nodes within l steps of S: S itself, layers <= 2 kept for the relabel, three buffers in turn
+    // nodes within l steps of S: S itself, layers <= 2 kept for the relabel, the others in turn
     const int my0 = CL ? st.set_first(rank) : -2;
     auto set_of = [&](int l) {
-        const RowMask m = {masks + (l == 0 ? 0 : l == 1 ? 2 : l == 2 ? 1 : 2 + (l - 2) % 3) * mw, rw, my0};
+        const RowMask m = {masks + (l == 0 ? 0 : l == 1 ? 2 : l == 2 ? 1 : 2 + (CL ? (l - 2) & 3 : (l - 2) % 3)) * mw, rw, my0};
         return m;
     };
     const RowMask mS = set_of(0);
     RefVals<R, CL> V;
     if constexpr (CL) {
-        V.tile = reinterpret_cast<typename Vec2<R>::type *>(lists + list_ints);
+        V.tile = reinterpret_cast<typename Vec2<R>::type *>(plans + 2 * PCAP);
         V.stride = any ? x1 - x0 + 1 : 1;
         V.o = (yr0 - 2) * V.stride + x0;
         // the rows of S that this CTA's sets start from, from the CTAs that found them
@@ -1715,7 +1758,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     const int dy0 = CL ? max(y0, yr0 - NL) : y0, dn = wn * ((CL ? min(y1, yr1 + NL - 1) : y1) - dy0 + 1);
     auto dilate = [&](int l) {
         const unsigned *const v = set_of(l - 1).p, *const o = set_of(l).p;
-        int *list = lists + (l & 1) * layer_cap;
+        int *list = list_of(l);
         for (int kw = blockDim.x - 32 - 32 * warp; kw < dn; kw += blockDim.x) {  // uniform over the warp
             const int k = kw + lane, row = wn > 1 ? (int)__umulhi((unsigned)k, wdiv) : k;
             const int w = wa + k - row * wn, y = dy0 + row;
@@ -1730,17 +1773,8 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
                 const_cast<unsigned *>(o)[at] = d;
                 ring = y >= yr0 && y < yr1 ? d & ~c : 0u;
             }
-            if (__ballot_sync(0xffffffffu, ring != 0u) == 0u) continue;
-            const int cnt = __popc(ring);
-            int pre = cnt;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, pre, d);
-                if (lane >= d) pre += t;
-            }
-            int at = 0;
-            if (lane == 31) at = atomicAdd(&lcnt[l], pre);
-            at = __shfl_sync(0xffffffffu, at, 31) + pre - cnt;
+            if (!ring) continue;
+            int at = atomicAdd(&lcnt[l], __popc(ring));
             const int e0 = (32 * w - 32) | (y << 16);
             while (ring) {
                 const int b = __ffs(ring) - 1;
@@ -1755,16 +1789,15 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
         if constexpr (CL) {
             V.tile[V.at(lx, ly)].x = vx;
             V.tile[V.at(lx, ly)].y = vy;
-            for (int k = rank - 1; k >= 0 && ly < st.first(k + 1) + 2; k--) {
+            auto push = [&](int k) {
                 R *p = reinterpret_cast<R *>(V.tile + (ly - st.first(k) + 2) * V.stride + lx - x0);
                 cluster_st(p, k, vx);
                 cluster_st(p + 1, k, vy);
-            }
-            for (int k = rank + 1; k < nc && ly >= st.first(k) - 2; k++) {
-                R *p = reinterpret_cast<R *>(V.tile + (ly - st.first(k) + 2) * V.stride + lx - x0);
-                cluster_st(p, k, vx);
-                cluster_st(p + 1, k, vy);
-            }
+            };
+            if (ly < yr0 + 2)
+                for (int k = rank - 1; k >= 0 && ly < st.first(k + 1) + 2; k--) push(k);
+            if (ly >= yr1 - 2)
+                for (int k = rank + 1; k < nc && ly >= st.first(k) - 2; k++) push(k);
         } else {
             Xo[ly * T + lx] = vx;
             Yo[ly * T + lx] = vy;
@@ -1784,76 +1817,143 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
         gy = pn - ps;
         return gx * gx + gy * gy > R(0);
     };
-    // The n listed targets of layer l, LPT (XY: twice that) lanes to each.
-    auto fit_layer = [&](auto lpt, auto xy, int l, const int *list, int n) {
-        constexpr int LPT = decltype(lpt)::value;
-        constexpr bool XY = decltype(xy)::value;
-        constexpr int G = XY ? 2 * LPT : LPT;
+    auto finish = [&](int l, int e, const FitPlan<R> &f, R ox, R oy) {
+        const int lx = e & 0xffff, ly = e >> 16;
+        if ((f.bits & FIT_NONE) && !fit_grown<R, CL>(V, set_of(l - 1), st, x0, T, lx, ly, sp.rmax, (f.bits & FIT_DIR) != 0u,
+                                                     f.gx, f.gy, ox, oy))
+            atomicOr(a.err, ERR_EXTRAP);
+        put(lx, ly, ox, oy);
+    };
+    // Layer l planned and fitted in place, a lane to a target: the narrow form (with
+    // several CTAs per SM, lanes that repeat work cost more than they save), and a
+    // layer too long for the wide form's plans.  A list that does not hold the
+    // layer is filled again for as many rows at a time as it holds in any case.
+    auto fit_in_place = [&](int l, bool refill) {
         const RowMask v = set_of(l - 1);
-        for (int k0 = 32 * warp / G; k0 < n; k0 += blockDim.x / G) {  // uniform over the warp
-            const int k = k0 + lane / G;
-            const bool on = k < n;
-            const int e = list[on ? k : n - 1], lx = e & 0xffff, ly = e >> 16;
-            R gx, gy, ox, oy;
-            const bool use_n = normal(l, lx, ly, gx, gy);
-            const bool good = fit_window<R, CL, LPT, XY>(V, lut, wd, v.window5(lx, ly), lx, ly, use_n, gx, gy, ox, oy);
-            if (!on || lane % G != 0) continue;
-            if (!good && !fit_grown<R, CL>(V, v, st, x0, T, lx, ly, sp.rmax, use_n, gx, gy, ox, oy)) atomicOr(a.err, ERR_EXTRAP);
-            put(lx, ly, ox, oy);
+        int *list = list_of(l), n = lcnt[l];
+        const int rows = layer_cap / T;
+        for (int c = yr0; c < yr1; c += rows) {
+            if (refill) {
+                const unsigned *const o = set_of(l).p;
+                __syncthreads();
+                if (tid == 0) lcnt[0] = 0;
+                __syncthreads();
+                for (int k = tid; k < wn * min(rows, yr1 - c); k += blockDim.x) {
+                    const int ly = c + k / wn, w = wa + k % wn, q = (ly - my0) * rw + w;
+                    for (unsigned ring = o[q] & ~v.p[q]; ring; ring &= ring - 1u)
+                        list[atomicAdd(&lcnt[0], 1)] = (32 * w + __ffs(ring) - 33) | (ly << 16);
+                }
+                __syncthreads();
+                n = lcnt[0];
+            }
+            for (int k = tid; k < n; k += blockDim.x) {
+                const int e = list[k], lx = e & 0xffff, ly = e >> 16;
+                R gx, gy, ox, oy;
+                FitPlan<R> f;
+                const bool use_n = normal(l, lx, ly, gx, gy);
+                fit_plan<R, 1>(lut, wd, v.window5(lx, ly), use_n, gx, gy, 0u, f);
+                fit_values<R, CL, 1, false>(V, wd, f, lx, ly, 0u, ox, oy);
+                finish(l, e, f, ox, oy);
+            }
+            if (!refill) break;
         }
     };
-    if (any) {
+    // The wide form's plans of layer l, LPT lanes to a target, by the warps from w0 on.
+    auto plan_layer = [&](auto lpt, int l, int w0) {
+        constexpr int LPT = decltype(lpt)::value;
+        const RowMask v = set_of(l - 1);
+        const int *list = list_of(l), n = lcnt[l], wk = warp >= w0 ? warp - w0 : warp - w0 + nw;
+        FitRec<R> *p = plans + (l & 1) * PCAP;
+        const unsigned gm = (0xffffffffu >> (32 - LPT)) << (lane & ~(LPT - 1));
+        for (int k = (32 * wk + lane) / LPT; k < n; k += (int)blockDim.x / LPT) {
+            const int e = list[k], lx = e & 0xffff, ly = e >> 16;
+            R gx, gy;
+            FitPlan<R> f;
+            const bool use_n = normal(l, lx, ly, gx, gy);
+            fit_plan<R, LPT>(lut, wd, v.window5(lx, ly), use_n, gx, gy, gm, f);
+            if (lane % LPT == 0) {
+                p[k].f = f;
+                p[k].e = e;
+            }
+        }
+    };
+    // The fits of a planned layer, LPT (XY: twice that) lanes to a target.
+    auto fit_planned = [&](auto lpt, int l) {
+        constexpr int LPT = decltype(lpt)::value;
+        constexpr bool XY = sizeof(R) == 8;
+        constexpr int G = XY ? 2 * LPT : LPT;
+        const int n = lcnt[l];
+        const FitRec<R> *p = plans + (l & 1) * PCAP;
+        const unsigned gm = (0xffffffffu >> (32 - G)) << (lane & ~(G - 1));
+        for (int k = tid / G; k < n; k += blockDim.x / G) {
+            const FitPlan<R> f = p[k].f;
+            const int e = p[k].e;
+            R ox, oy;
+            fit_values<R, CL, LPT, XY>(V, wd, f, e & 0xffff, e >> 16, gm, ox, oy);
+            if (lane % G == 0) finish(l, e, f, ox, oy);
+        }
+    };
+    if (any && a.init) {  // xi = x on the band at initialisation
+        const R e0x = R(frame_d(fo, sd.xc, true)), e0y = R(frame_d(fo, sd.yc, false));
+        for (int l = 1; l <= NL; l++) {
+            dilate(l);
+            __syncthreads();
+            const unsigned *const v = set_of(l - 1).p, *const o = set_of(l).p;
+            for (int k = tid; k < wn * (yr1 - yr0); k += blockDim.x) {
+                const int ly = yr0 + k / wn, w = wa + k % wn, q = (ly - my0) * rw + w;
+                for (unsigned ring = o[q] & ~v[q]; ring; ring &= ring - 1u) put(32 * w + __ffs(ring) - 33, ly, e0x, e0y);
+            }
+        }
+        solid_sync();
+    } else if (any && !CL) {
         dilate(1);
         __syncthreads();
         for (int l = 1; l <= NL; l++) {
             if (l < NL) dilate(l + 1);
-            int n = lcnt[l], *list = lists + (l & 1) * layer_cap;
-            if (a.init) {  // xi = x on the band at initialisation
-                const unsigned *const v = set_of(l - 1).p, *const o = set_of(l).p;
-                const R e0x = R(frame_d(fo, sd.xc, true)), e0y = R(frame_d(fo, sd.yc, false));
-                for (int k = tid; k < wn * (yr1 - yr0); k += blockDim.x) {
-                    const int ly = yr0 + k / wn, w = wa + k % wn, q = (ly - my0) * rw + w;
-                    for (unsigned ring = o[q] & ~v[q]; ring; ring &= ring - 1u) put(32 * w + __ffs(ring) - 33, ly, e0x, e0y);
-                }
-                solid_sync();
-                continue;
+            fit_in_place(l, lcnt[l] > layer_cap);
+            __syncthreads();  // the next layer reads this one's values, and its list is complete
+        }
+    } else if (any) {
+        // One CTA per SM, and a layer as long as one target's chain: so everything
+        // that does not need the layer before -- the sets, the normals, the cofactors and
+        // the reciprocal of the determinant -- is done one and two layers ahead by the warps
+        // that have no target, between the arrival at the cluster's barrier and the
+        // wait (475 cycles).  What is left is a window of products and the sum over its rows,
+        // dealt out to 2, 4 or 8 lanes while the targets leave lanes idle -- in
+        // FP64, whose pipe takes a warp instruction per scheduler in 64 cycles, up to
+        // one warp for each of the four, and a lane per coordinate.
+        auto plan = [&](int l, int w0) {
+            const int n = lcnt[l], room = sizeof(R) == 8 ? 128 : (int)blockDim.x / 2;
+            if (n > PCAP) return;
+            if (l > 2) plan_layer(std::integral_constant<int, 1>(), l, w0);
+            else if (8 * n <= room) plan_layer(std::integral_constant<int, 8>(), l, w0);
+            else if (4 * n <= room) plan_layer(std::integral_constant<int, 4>(), l, w0);
+            else plan_layer(std::integral_constant<int, 1>(), l, w0);
+        };
+        dilate(1);
+        __syncthreads();
+        if (NL > 1) dilate(2);
+        plan(1, 0);
+        __syncthreads();
+        if (NL > 2) dilate(3);
+        if (NL > 1) plan(2, nw / 2);
+        __syncthreads();
+        for (int l = 1; l <= NL; l++) {
+            const int n = lcnt[l], room = sizeof(R) == 8 ? 64 : (int)blockDim.x;
+            int used = 1;  // lanes to a target
+            if (n > PCAP) fit_in_place(l, true);
+            else if (8 * n <= room) { used = 8; fit_planned(std::integral_constant<int, 8>(), l); }
+            else if (4 * n <= room) { used = 4; fit_planned(std::integral_constant<int, 4>(), l); }
+            else if (2 * n <= room) { used = 2; fit_planned(std::integral_constant<int, 2>(), l); }
+            else fit_planned(std::integral_constant<int, 1>(), l);
+            cluster_arrive();
+            if (l >= 2 && l < NL) {
+                const int w0 = (n * used * (sizeof(R) == 8 ? 2 : 1) + 31) >> 5;
+                plan(l + 1, w0 < nw ? w0 : 0);
+                if (l + 2 <= NL) dilate(l + 2);
             }
-            // a list that does not hold the layer is filled again for as many rows at a
-            // time as it holds in any case (their nodes come in any order)
-            const bool over = n > layer_cap;
-            const int rows = layer_cap / T;
-            for (int c = yr0; c < yr1; c += rows) {
-                if (over) {
-                    const unsigned *const v = set_of(l - 1).p, *const o = set_of(l).p;
-                    __syncthreads();
-                    if (tid == 0) lcnt[0] = 0;
-                    __syncthreads();
-                    for (int k = tid; k < wn * min(rows, yr1 - c); k += blockDim.x) {
-                        const int ly = c + k / wn, w = wa + k % wn, q = (ly - my0) * rw + w;
-                        for (unsigned ring = o[q] & ~v[q]; ring; ring &= ring - 1u)
-                            list[atomicAdd(&lcnt[0], 1)] = (32 * w + __ffs(ring) - 33) | (ly << 16);
-                    }
-                    __syncthreads();
-                    n = lcnt[0];
-                }
-                // Lanes to a target: with one CTA per SM a layer takes as long as one fit, so
-                // the window's rows go to 2, 4 or 8 lanes while the targets leave lanes
-                // idle -- in FP64, whose pipe takes a warp instruction per scheduler in 64
-                // cycles, up to one warp for each of the four, and a lane per coordinate.
-                // With several CTAs per SM the extra instructions cost more than they save.
-                if constexpr (CL) {
-                    typedef std::integral_constant<bool, sizeof(R) == 8> xy_t;
-                    const int room = sizeof(R) == 8 ? 64 : (int)blockDim.x;
-                    if (8 * n <= room) fit_layer(std::integral_constant<int, 8>(), xy_t(), l, list, n);
-                    else if (4 * n <= room) fit_layer(std::integral_constant<int, 4>(), xy_t(), l, list, n);
-                    else if (2 * n <= room) fit_layer(std::integral_constant<int, 2>(), xy_t(), l, list, n);
-                    else fit_layer(std::integral_constant<int, 1>(), xy_t(), l, list, n);
-                } else {
-                    fit_layer(std::integral_constant<int, 1>(), std::false_type(), l, list, n);
-                }
-                if (!over) break;
-            }
-            solid_sync();  // the next layer reads this one's values, and its list is complete
+            cluster_wait();   // the next layer reads this one's values,
+            __syncthreads();  // and what this CTA's warps have planned and listed
         }
     }
 
