@@ -317,8 +317,9 @@ int lbrmt_uses_tma(const lbrmt_sim *sim);
  * highest priority; the step ends when both are done (the caller's stream then
  * waits for the internal one).  The results are the same bit for bit.  A solid
  * found in a region that a step treated as free raises LBRMT_ERR_NUMERIC at the
- * next error check.  Not used with tensor-memory loads (lbrmt_set_use_tma) or
- * without solids; lbrmt_step_timed always takes the sequential schedule.
+ * next error check.  With tensor-memory loads (lbrmt_set_use_tma) used from 4 M
+ * nodes on in FP32 arithmetic (the busy regions are then staged, the free ones
+ * read directly); not used without solids; lbrmt_step_timed always takes the sequential schedule.
  * lbrmt_uses_overlap tells whether steps overlap (after initialisation). */
 lbrmt_status lbrmt_set_overlap(lbrmt_sim *sim, int enable);
 int lbrmt_uses_overlap(const lbrmt_sim *sim);

@@ -23,6 +23,11 @@ struct LaunchInfo {
     int rmt_nc = 0;        // CTAs per solid (a cluster) of K2's wide form; 0: the narrow form
     bool tma = false;    // tensor maps of the populations and density plane are valid
     bool use_tma = true; // K1 with TMA staging (else the direct-load kernel)
+    // The staged K1 takes the busy regions' tiles of an overlapped step, the direct-load
+    // kernel the free regions.  From 4 M nodes on in FP32 arithmetic: the free K1 must
+    // outlast the extra launches (FP16 at 4096^2: 511 -> 474 us a step; sequential is
+    // faster at 512^2, 49 against 53 us, and in FP64 at 1024^2, 437 against 448).
+    bool staged_overlap = false;
     int lb_blocks = 0, lb_smem = 0;
     CUtensorMap tm_f[2], tm_c;
     // Overlapped step: K1 of the regions without solid forcing runs on a side
@@ -38,7 +43,7 @@ struct LaunchInfo {
 
 // Does a step run the overlapped schedule (K1 split into busy and free regions)?
 inline bool step_overlaps(const SimParams &sp, const LaunchInfo &li) {
-    return li.split && li.side && sp.nsolids > 0 && !(li.tma && li.use_tma);
+    return li.split && li.side && sp.nsolids > 0 && (!(li.tma && li.use_tma) || li.staged_overlap);
 }
 
 // Kernel launches of one step (timed: the sequential schedule of lbrmt_step_timed).
@@ -224,14 +229,17 @@ struct Engine {
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
         if (!ok) return;
         li->lb_smem = 2 * 10 * TILE_N * (int)ss + 128;  // + alignment of the stages
-        if (cudaFuncSetAttribute(lb_tma_kernel<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, li->lb_smem) !=
-            cudaSuccess)
+        if (cudaFuncSetAttribute(lb_tma_kernel<R, S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, li->lb_smem) !=
+                cudaSuccess ||
+            cudaFuncSetAttribute(lb_tma_kernel<R, S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, li->lb_smem) !=
+                cudaSuccess)
             return;
         int per = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, lb_tma_kernel<R, S>, TILE_N, li->lb_smem) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, lb_tma_kernel<R, S, false>, TILE_N, li->lb_smem) != cudaSuccess ||
             per < 1)
             return;
         li->lb_blocks = nsm * per;
+        li->staged_overlap = sizeof(R) == 4 && sp.P >= (1ll << 22);
         li->tma = true;
     }
 
@@ -560,9 +568,11 @@ struct Engine {
             launch_prio(overlap ? force_kernel<R, 48> : force_kernel<R, 56>, dim3(overlap ? li.force_blocks_ov : li.force_blocks),
                         dim3(K3_THREADS), li.force_smem, st, prio, sp, force_args(d, q, p));
         if (ev) cudaEventRecord(ev[2], st);
-        if (li.tma && li.use_tma)
-            lb_tma_kernel<R, S><<<li.lb_blocks, TILE_N, li.lb_smem, st>>>(sp, la, li.tm_f[p], li.tm_c, sp.ntx * sp.nty);
-        else if (overlap) {
+        if (li.tma && li.use_tma) {
+            if (overlap && !(chain & CHAIN_FIRST)) cudaStreamWaitEvent(st, li.done[q], 0);  // free K1 of step n - 1
+            launch_prio(overlap ? lb_tma_kernel<R, S, true> : lb_tma_kernel<R, S, false>, dim3(li.lb_blocks), blk, li.lb_smem, st,
+                        prio, sp, la, li.tm_f[p], li.tm_c, sp.ntx * sp.nty, (const unsigned char *)d.busy[p]);
+        } else if (overlap) {
             if (!(chain & CHAIN_FIRST)) cudaStreamWaitEvent(st, li.done[q], 0);  // free K1 of step n - 1
             launch_prio(lb_step_kernel<R, S, 1>, grid, blk, 0, st, prio, sp, la, (const unsigned char *)d.busy[p]);
         } else

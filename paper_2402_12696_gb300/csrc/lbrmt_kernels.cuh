@@ -1542,11 +1542,11 @@ template <class R> __device__ __forceinline__ R frame_shift(int sh, float off_ou
 // sets 4 K, layers 1-2 23 K, layers 3-11 48 K, relabel 31 K, frame and registry 6 K
 // (54, 24, 20, 53, 32, 12 K with byte labels, an L1 distance transform and a
 // branch per window node, and 7 K instead of 4 K before pass 0, most of it FP64
-// in every thread).  Per launch: 4096^2 with 1024 disks 198 -> 164 us; 1501 x 1203 with 110 88 -> 75;
-// 96 cavities in one batch 213 -> 175.  In a cluster of 16 CTAs: one disk of radius
-// 128 1529 -> 66 us (its layers no longer fitted the list and scanned the tile), of
-// 64 192 -> 51, of 16 57 -> 40 (cluster of 8), 24 of 10-20 58 -> 42; in FP64, whose pipe takes a warp
-// instruction per scheduler in 64 cycles, 64 disks 352 -> 156, one 204 -> 73.
+// in every thread).  Per launch: 4096^2 with 1024 disks 198 -> 163 us; 1501 x 1203 with
+// 110 88 -> 73; 96 cavities in one batch 213 -> 166.  In a cluster of 16 CTAs: one disk of
+// radius 128 1529 -> 62 us (its layers no longer fitted the list and scanned the tile), of
+// 64 192 -> 46, of 16 57 -> 35 (cluster of 8), 24 of 10-20 58 -> 38; in FP64, whose pipe
+// takes a warp instruction per scheduler in 64 cycles, 64 disks 352 -> 144, one 204 -> 62.
 template <class R, class S, bool CL>
 __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int s, const int rank, const int nc) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -2710,7 +2710,7 @@ __device__ __forceinline__ R lb_node(const SimParams &sp, const LbArgs<R, S> &a,
 // tile's planes are in shared memory).
 template <class R, class S, bool STAGED>
 __device__ __forceinline__ void lb_tile(const SimParams &sp, const LbArgs<R, S> &a, const int bx, const int by,
-                                        const S *stage) {
+                                        const S *stage, const bool clr_active) {
     const int lt = threadIdx.x;
     const int i = bx * sp.tx + (lt & (sp.tx - 1)), j = by * sp.ty + (lt >> sp.lx);
     const int tile = by * sp.ntx + bx;
@@ -2719,7 +2719,7 @@ __device__ __forceinline__ void lb_tile(const SimParams &sp, const LbArgs<R, S> 
     __syncthreads();
     if (lt == 0) {
         a.clr_count[tile] = 0;
-        if (tile == 0) *a.clr_nactive = 0;
+        if (tile == 0 && clr_active) *a.clr_nactive = 0;
     }
 }
 
@@ -2860,10 +2860,12 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned parity)
     }
 }
 
-template <class R, class S>
+// BUSY: only the tiles of the overlapped step's busy regions.
+template <class R, class S, bool BUSY>
 __global__ void __launch_bounds__(TILE_N, LB_MIN_BLOCKS<R, S>) lb_tma_kernel(SimParams sp, LbArgs<R, S> a,
                                                         const __grid_constant__ CUtensorMap tm_f,
-                                                        const __grid_constant__ CUtensorMap tm_c, int ntiles) {
+                                                        const __grid_constant__ CUtensorMap tm_c, int ntiles,
+                                                        const unsigned char *busy) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bar[2];
     __shared__ int ok;
@@ -2890,12 +2892,18 @@ __global__ void __launch_bounds__(TILE_N, LB_MIN_BLOCKS<R, S>) lb_tma_kernel(Sim
         tma_load_3d(dst, &tm_f, bx * sp.tx, by * sp.ty, 0, b);
         tma_load_3d(dst + 9u * TILE_N * (unsigned)sizeof(S), &tm_c, bx * sp.tx, by * sp.ty, 0, b);
     };
-    int tile = blockIdx.x;
+    // the CTA's tiles: every gridDim.x-th, BUSY: of those the busy regions' ones
+    auto next_tile = [&](int t) {
+        if constexpr (BUSY)
+            while (t < ntiles && !busy[(t / sp.ntx) * sp.nrx + ((t % sp.ntx) >> sp.lk)]) t += gridDim.x;
+        return t;
+    };
+    int tile = next_tile(blockIdx.x), tile1 = next_tile(tile + gridDim.x);
     if (lt == 0) {
         if (tile < ntiles) issue(tile, 0);
-        if (tile + (int)gridDim.x < ntiles) issue(tile + gridDim.x, 1);
+        if (tile1 < ntiles) issue(tile1, 1);
     }
-    for (int it = 0; tile < ntiles; tile += gridDim.x, it++) {
+    for (int it = 0; tile < ntiles; it++) {
         const int st = it & 1;
         if (lt == 0) ok = mbar_wait_bounded(smem_u32(&bar[st]), (it >> 1) & 1) ? 1 : 0;
         __syncthreads();
@@ -2903,13 +2911,15 @@ __global__ void __launch_bounds__(TILE_N, LB_MIN_BLOCKS<R, S>) lb_tma_kernel(Sim
             if (lt == 0) {
                 atomicOr(a.err, ERR_TIMEOUT);
                 // let the other stage's copy (if one was issued) land before leaving
-                if (tile + (int)gridDim.x < ntiles) mbar_wait_bounded(smem_u32(&bar[st ^ 1]), ((it + 1) >> 1) & 1);
+                if (tile1 < ntiles) mbar_wait_bounded(smem_u32(&bar[st ^ 1]), ((it + 1) >> 1) & 1);
             }
             return;
         }
-        lb_tile<R, S, true>(sp, a, tile % sp.ntx, tile / sp.ntx, stage0 + st * stage_elems);
+        lb_tile<R, S, true>(sp, a, tile % sp.ntx, tile / sp.ntx, stage0 + st * stage_elems, !BUSY);
         // every thread has read stage st (lb_tile ends with a barrier): refill it
-        if (lt == 0 && tile + 2 * (int)gridDim.x < ntiles) issue(tile + 2 * gridDim.x, st);
+        tile = tile1;
+        tile1 = next_tile(tile1 + gridDim.x);
+        if (lt == 0 && tile1 < ntiles) issue(tile1, st);
     }
 }
 
