@@ -597,14 +597,31 @@ struct Engine {
         return cudaGetLastError();
     }
 
+    // CTAs per solid of the statistics: up to 8 (a portable cluster), two CTAs on each of the 152 SMs
+    static int stats_ctas(int nsolids) {
+        int nc = 8;
+        while (nc > 1 && nsolids * nc > 304) nc /= 2;
+        return nc;
+    }
+
     static cudaError_t stats(const SimParams &sp, const DevState &d, int cur, double *out, cudaStream_t st) {
         if (sp.nsolids == 0) return cudaSuccess;
-        solid_stats_kernel<R, S><<<sp.nsolids, STATS_THREADS, 0, st>>>(sp, (const S *)d.f[cur], (const S *)d.carry,
-                                                             (const R *)d.fbody, (const R *)d.bfield,
-                                                             d.reg_count[1 - cur], d.reg_solids[1 - cur],
-                                                             (const R *)d.pool[1 - cur], (const R *)d.xi[cur],
-                                                             d.frame[cur], d.solids, d.order, out);
-        return cudaGetLastError();
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        const int nc = stats_ctas(sp.nsolids);
+        cfg.gridDim = dim3(sp.nsolids * nc);
+        cfg.blockDim = dim3(STATS_THREADS);
+        cfg.stream = st;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = nc;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, solid_stats_kernel<R, S>, sp, (const S *)d.f[cur], (const S *)d.carry,
+                                  (const R *)d.fbody, (const R *)d.bfield, (const int *)d.reg_count[1 - cur],
+                                  (const int *)d.reg_solids[1 - cur], (const R *)d.pool[1 - cur],
+                                  (const R *)d.xi[cur], (const Frame *)d.frame[cur], (const SolidDesc *)d.solids,
+                                  (const int *)d.order, out);
     }
 
     static cudaError_t mass(const SimParams &sp, const DevState &d, int cur, cudaStream_t st) {

@@ -444,6 +444,11 @@ __device__ __forceinline__ unsigned cluster_ld(const void *p, int rank) {
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(p, rank)) : "memory");
     return v;
 }
+__device__ __forceinline__ double cluster_ld(const double *p, int rank) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(cluster_addr(p, rank)) : "memory");
+    return v;
+}
 __device__ __forceinline__ void cluster_ld2(const float2 *p, int rank, float &x, float &y) {
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(cluster_addr(p, rank)) : "memory");
 }
@@ -3299,13 +3304,13 @@ __device__ __forceinline__ void contact_tile_sum(const SimParams &sp, const R *x
 // hold another solid t, the divergence (Eq. 3_3_div_solid_stress) of the pair's
 // contact stress at every domain node nearer to s than to t (phi_s < phi_t,
 // half where equal; a node outside t's band is nearer to s), summed over the
-// pairs in FP64 by the CTA's threads.
+// pairs in FP64 by the CTA's threads; CTA rank of nc takes every nc-th such tile.
 constexpr int CONTACT_CAP = 128;  // tiles a solid shares with another, listed in shared memory
 
 template <class R>
 __device__ __noinline__ void contact_force_sum(const SimParams &sp, const int *reg, const int *reg_solids, const R *xi,
                                   const Frame *frames, const SolidDesc *solids, int s, const Frame &fr, double (&fc)[2],
-                                  int *ctile /* shared, CONTACT_CAP */, int *nct /* shared */) {
+                                  int *ctile /* shared, CONTACT_CAP */, int *nct /* shared */, int rank, int nc) {
     const SolidDesc sd = solids[s];
     const R eps = pick<R>(sp.eps, sp.eps_f), eta = pick<R>(sp.eta, sp.eta_f);
     if (fr.bx0 > fr.bx1) return;  // uniform over the CTA
@@ -3337,6 +3342,7 @@ __device__ __noinline__ void contact_force_sum(const SimParams &sp, const int *r
     __syncthreads();
     const int ncand = *nct;
     if (ncand > CONTACT_CAP) {  // more than the list holds: every tile of the box in turn, in the same order
+        int turn = 0;
         for (int ay = 0; ay < nry; ay++)
             for (int by = ry0[ay]; by <= ry1[ay]; by++)
                 for (int ax = 0; ax < nrx; ax++)
@@ -3346,8 +3352,8 @@ __device__ __noinline__ void contact_force_sum(const SimParams &sp, const int *r
                         if (n < 2) continue;
                         bool mine = false;
                         for (int m = 0; m < n; m++) mine = mine || reg_solids[tile * KMAX + m] == s;
-                        if (mine) contact_tile_sum<R>(sp, xi, frames, solids, reg, reg_solids, s, sd, fr, eps, eta,
-                                                      tile, fc);
+                        if (mine && turn++ % nc == rank)
+                            contact_tile_sum<R>(sp, xi, frames, solids, reg, reg_solids, s, sd, fr, eps, eta, tile, fc);
                     }
         return;
     }
@@ -3359,9 +3365,43 @@ __device__ __noinline__ void contact_force_sum(const SimParams &sp, const int *r
             ctile[b + 1] = v;
         }
     __syncthreads();
-    for (int c = 0; c < ncand; c++) contact_tile_sum<R>(sp, xi, frames, solids, reg, reg_solids, s, sd, fr, eps, eta,
-                                                        ctile[c], fc);
+    for (int c = rank; c < ncand; c += nc)
+        contact_tile_sum<R>(sp, xi, frames, solids, reg, reg_solids, s, sd, fr, eps, eta, ctile[c], fc);
 }
+
+// The ten columns of a warp's lanes summed: each step halves both the lanes that hold
+// a column and the columns that a lane holds (12 additions a lane; 50 column by column,
+// and an FP64 one occupies its scheduler for 64 cycles).  Lane l returns the sum of
+// column 5 b4 + 3 b3 + 2 b2 + b1 (b: the bits of l) where `column` is not negative.
+__device__ __forceinline__ double warp_columns(double (&v)[STATS_COLS], int &column) {
+    static_assert(STATS_COLS == 10, "the halving below is written for ten columns");
+    const int lane = threadIdx.x & 31;
+    constexpr int N[5] = {10, 5, 3, 2, 1};
+#pragma unroll
+    for (int st = 0; st < 5; st++) {
+        const int m = 16 >> st, h = (N[st] + 1) / 2;
+        const bool hi = (lane & m) != 0;
+#pragma unroll
+        for (int k = 0; k < h; k++) {
+            if (N[st] == 1) {
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
+            } else {
+                const double a = v[k], b = k + h < N[st] ? v[k + h] : 0.0;
+                v[k] = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, m);
+            }
+        }
+    }
+    const int b3 = (lane >> 3) & 1, r = 2 * ((lane >> 2) & 1) + ((lane >> 1) & 1);
+    column = (lane & 1) || r >= (b3 ? 2 : 3) ? -1 : 5 * (lane >> 4) + 3 * b3 + r;
+    return v[0];
+}
+
+// Statistics of one solid: a CTA, or a cluster of CTAs that share its box's nodes and
+// contact tiles (partial sums per warp, then CTA, then cluster, each in order).
+// Bound by the latency of the gathers of a node and, in FP64, by its pipe: the cluster
+// is as large as keeps every CTA resident (stats_ctas).  Per launch, one CTA and the cluster:
+// one disk of radius 128 207 -> 37 us, of 13 in FP64 43 -> 18.5, 24 of 10-20 31 -> 18.5;
+// 506 ellipses (one CTA either way) 58 -> 42 by the shorter reduction (warp_columns).
 
 template <class R, class S>
 __global__ void __launch_bounds__(STATS_THREADS, sizeof(R) == 4 ? 3 : 2) solid_stats_kernel(SimParams sp, const S *f, const S *carry,
@@ -3369,11 +3409,12 @@ __global__ void __launch_bounds__(STATS_THREADS, sizeof(R) == 4 ? 3 : 2) solid_s
                                                                     const R *xi, const Frame *frames,
                                                                     const SolidDesc *solids, const int *order,
                                                                     double *out) {
-    __shared__ double red[32 * STATS_COLS];
+    __shared__ double red[STATS_THREADS / 32 * STATS_COLS], tot[STATS_COLS];  // sums of the warps, of the CTA
     __shared__ unsigned long long dmax;
     __shared__ int queue[STATS_THREADS / 32][64];  // per warp: < 32 waiting + one round of 32
     __shared__ int ctile[CONTACT_CAP], nct;         // tiles shared with another solid (contact sum)
-    const int s = order ? order[blockIdx.x] : (int)blockIdx.x;  // largest tiles first, as K2
+    const int rank = cluster_rank(), nc = cluster_size(), si = (int)blockIdx.x / nc;
+    const int s = order ? order[si] : si;  // largest tiles first, as K2
     const SolidDesc sd = solids[s];
     const Frame fr = frames[s];
     const int2 o = make_int2(fr.ox, fr.oy), ow = make_int2(wrapi(fr.ox, sp.nx), wrapi(fr.oy, sp.ny));
@@ -3402,10 +3443,10 @@ __global__ void __launch_bounds__(STATS_THREADS, sizeof(R) == 4 ? 3 : 2) solid_s
     // four rounds of the walk per pass: their loads are issued together.  Each
     // lane steps its box position (c, r) by the warps' stride, without divisions.
     constexpr int WU = 4;
-    const int step = nw * 32;
+    const int step = nc * nw * 32, first = (rank * nw + warp) * 32;
     int c = 0, r = 0, dc = 0, dr = 0;
-    if (w > 0) { c = (warp * 32 + lane) % w; r = (warp * 32 + lane) / w; dc = step % w; dr = step / w; }
-    for (int base = warp * 32; base < n; base += WU * step) {
+    if (w > 0) { c = (first + lane) % w; r = (first + lane) / w; dc = step % w; dr = step / w; }
+    for (int base = first; base < n; base += WU * step) {
         int ee[WU];
         bool keep[WU];
         R xv[WU], pv[WU];
@@ -3447,28 +3488,42 @@ __global__ void __launch_bounds__(STATS_THREADS, sizeof(R) == 4 ? 3 : 2) solid_s
     v[8] = v[9] = 0.0;
     {
         double fc[2] = {0.0, 0.0};
-        contact_force_sum<R>(sp, reg, reg_solids, xi, frames, solids, s, fr, fc, ctile, &nct);
+        contact_force_sum<R>(sp, reg, reg_solids, xi, frames, solids, s, fr, fc, ctile, &nct, rank, nc);
         v[8] = fc[0];
         v[9] = fc[1];
     }
-#pragma unroll
-    for (int k = 0; k < STATS_COLS; k++)
-        for (int d = 16; d > 0; d >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], d);
-    if (lane == 0)
-        for (int k = 0; k < STATS_COLS; k++) red[warp * STATS_COLS + k] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double st[STATS_COLS];
-        for (int k = 0; k < STATS_COLS; k++) {
-            st[k] = 0.0;
-            for (int ww = 0; ww < nw; ww++) st[k] += red[ww * STATS_COLS + k];
-        }
-        double *q = out + STATS_COLS * s;
-        q[0] = st[0]; q[1] = o.x + st[1] / st[0]; q[2] = o.y + st[2] / st[0]; q[3] = st[3]; q[4] = st[4]; q[5] = st[5];
-        q[6] = __longlong_as_double((long long)dmax);
-        q[7] = st[7] > 0.0 ? st[6] / st[7] : 0.0;
-        q[8] = st[8]; q[9] = st[9];
+    {
+        int col;
+        const double x = warp_columns(v, col);
+        if (col >= 0) red[warp * STATS_COLS + col] = x;
     }
+    __syncthreads();
+    if (threadIdx.x < STATS_COLS) {
+        double st = 0.0;
+        for (int ww = 0; ww < nw; ww++) st += red[ww * STATS_COLS + threadIdx.x];
+        tot[threadIdx.x] = st;
+    }
+    if (nc > 1) cluster_sync();
+    if (rank == 0 && warp == 0) {
+        double st = 0.0;
+        __syncwarp();
+        if (lane < STATS_COLS) st = tot[lane];
+        unsigned long long dm = dmax;
+        for (int k = 1; k < nc; k++) {
+            if (lane < STATS_COLS) st += cluster_ld(&tot[lane], k);
+            const unsigned long long d = (unsigned long long)__double_as_longlong(
+                cluster_ld(reinterpret_cast<const double *>(&dmax), k));
+            dm = d > dm ? d : dm;
+        }
+        // area, centroid (2), mass, momentum (2), max and mean |det F - 1|, contact force (2)
+        const double area = __shfl_sync(0xffffffffu, st, 0), dsum = __shfl_sync(0xffffffffu, st, 6);
+        double x = st;
+        if (lane == 1 || lane == 2) x = (lane == 1 ? o.x : o.y) + st / area;
+        if (lane == 6) x = __longlong_as_double((long long)dm);
+        if (lane == 7) x = st > 0.0 ? dsum / st : 0.0;
+        if (lane < STATS_COLS) out[STATS_COLS * s + lane] = x;
+    }
+    if (nc > 1) cluster_sync();  // the partial sums are read
 }
 
 // Fixed-order FP64 sum of the per-block mass partials (single CTA).
