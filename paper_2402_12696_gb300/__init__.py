@@ -561,7 +561,7 @@ class Simulation:
     def field(self, name, solid=0):
         """Device tensor (float64, [ny, nx]) of one field."""
         torch = self.torch
-        with torch.cuda.device(self.device), torch.cuda.stream(self.stream):
+        with torch.cuda.stream(self.stream):  # and its device
             out = torch.empty(self.ny * self.nx, dtype=torch.float64, device=self.device)
             fid = FIELDS[name] if isinstance(name, str) else int(name)
             lbrmt_read_fields(self.h, 0, fid, solid, out.data_ptr())

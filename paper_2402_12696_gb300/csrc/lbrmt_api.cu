@@ -74,6 +74,19 @@ static void dfree_all(lbrmt_sim *s) {
         else cudaFree(p);
     }
     s->allocs.clear();
+    if (s->report) cudaFreeHost(s->report);
+    s->report = nullptr;
+}
+
+// The page-locked report for nsolids solids (replaces a smaller one).
+static bool alloc_report(lbrmt_sim *s, int nsolids) {
+    if (s->report) cudaFreeHost(s->report);
+    s->report = nullptr;
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, 16 + (size_t)nsolids * STATS_COLS * 8, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess)
+        return false;
+    s->report = (unsigned *)p;
+    return true;
 }
 
 extern "C" void lbrmt_default_config(lbrmt_config *c) {
@@ -171,6 +184,7 @@ extern "C" lbrmt_status lbrmt_create(const lbrmt_config *cfg, void *cuda_stream,
     ok = ok && (d.mass_partials = (double *)dalloc(s, nparts * 8));
     ok = ok && (d.err = (unsigned *)dalloc(s, 16));
     ok = ok && (d.lamtab = dalloc(s, (size_t)(2 * sp.lam_k0 + 1) * (rs == 4 ? sizeof(LamEntry) : sizeof(LamEntryD))));
+    ok = ok && alloc_report(s, 0);
     ok = ok && (s->scratch = (double *)dalloc(s, 128));  // one solid's statistics or the total mass
     // side stream (lowest priority) and fork / join events of the overlapped step
     if (ok) {
@@ -281,13 +295,12 @@ extern "C" lbrmt_status lbrmt_add_solid(lbrmt_sim *s, int shape, double cx, doub
     return lbrmt_add_solid_shape(s, LBRMT_SHAPE_DISK, cx, cy, radius, radius, rho_s, G, id_out);
 }
 
-static lbrmt_status check_flags(lbrmt_sim *s) {
-    unsigned h[4] = {0, 0, 0, 0};
-    cudaError_t e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return cuda_fail(s, e, "stream");
-    e = cudaMemcpy(h, s->d.err, 16, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(s, e, "error flags");
-    const unsigned f = h[0];
+cudaError_t lbrmt_internal_queue_flags(lbrmt_sim *s) {
+    return cudaMemcpyAsync(s->report, s->d.err, 16, cudaMemcpyDeviceToHost, s->stream);
+}
+
+lbrmt_status lbrmt_internal_flag_status(lbrmt_sim *s) {
+    const unsigned f = *(volatile unsigned *)s->report;
     if (!f) return LBRMT_OK;
     if (f & ERR_NAN) return fail(s, LBRMT_ERR_NUMERIC, "non-finite density or velocity");
     if (f & ERR_SLOT_OVERFLOW) return fail(s, LBRMT_ERR_OVERFLOW, "more solids on a tile than max_solids_per_tile");
@@ -301,6 +314,14 @@ static lbrmt_status check_flags(lbrmt_sim *s) {
     if (f & ERR_FREE_REGION)
         return fail(s, LBRMT_ERR_NUMERIC, "an interface moved more than one node in a step (a region stepped as solid-free held a solid)");
     return fail(s, LBRMT_ERR_NUMERIC, "device error flag");
+}
+
+static lbrmt_status check_flags(lbrmt_sim *s) {
+    cudaError_t e = lbrmt_internal_queue_flags(s);
+    if (e != cudaSuccess) return cuda_fail(s, e, "error flags");
+    e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return cuda_fail(s, e, "stream");
+    return lbrmt_internal_flag_status(s);
 }
 
 lbrmt_status lbrmt_internal_check_flags(lbrmt_sim *s) { return check_flags(s); }
@@ -455,6 +476,7 @@ extern "C" lbrmt_status lbrmt_init(lbrmt_sim *s) {
         s->scratch = sc;
     }
     if (!ok) return fail(s, LBRMT_ERR_CUDA, "out of device memory for the solid tiles");
+    if (S > 0 && !alloc_report(s, S)) return fail(s, LBRMT_ERR_CUDA, "out of page-locked memory for the statistics");
     return run_init(s);
 }
 
@@ -761,11 +783,13 @@ extern "C" lbrmt_status lbrmt_solid_stats(lbrmt_sim *s, int sim_index, double *h
     }
     const int S = (int)s->solids.size();
     if (S == 0) return LBRMT_OK;
-    cudaError_t e = s->eng->stats(s->sp, s->d, (int)(s->steps & 1), s->scratch, s->stream);
+    double *out = (double *)(s->report + 4);
+    cudaError_t e = s->eng->stats(s->sp, s->d, (int)(s->steps & 1), out, s->report, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "stats kernel");
-    e = cudaMemcpyAsync(host_out, s->scratch, (size_t)S * STATS_COLS * 8, cudaMemcpyDeviceToHost, s->stream);
-    if (e != cudaSuccess) return cuda_fail(s, e, "copy stats");
-    return check_flags(s);
+    e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return cuda_fail(s, e, "stream");
+    std::memcpy(host_out, out, (size_t)S * STATS_COLS * 8);
+    return lbrmt_internal_flag_status(s);
 }
 
 extern "C" lbrmt_status lbrmt_solid_stats_async(lbrmt_sim *s, int sim_index, double *host_out) {
@@ -774,11 +798,11 @@ extern "C" lbrmt_status lbrmt_solid_stats_async(lbrmt_sim *s, int sim_index, dou
     const int S = (int)s->solids.size();
     if (S == 0) return LBRMT_OK;
     if (double *dv = (double *)mapped_view(host_out)) {  // page-locked: the kernel writes it
-        cudaError_t e = s->eng->stats(s->sp, s->d, (int)(s->steps & 1), dv, s->stream);
+        cudaError_t e = s->eng->stats(s->sp, s->d, (int)(s->steps & 1), dv, nullptr, s->stream);
         if (e != cudaSuccess) return cuda_fail(s, e, "stats kernel");
         return LBRMT_OK;
     }
-    cudaError_t e = s->eng->stats(s->sp, s->d, (int)(s->steps & 1), s->scratch, s->stream);
+    cudaError_t e = s->eng->stats(s->sp, s->d, (int)(s->steps & 1), s->scratch, nullptr, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "stats kernel");
     e = cudaMemcpyAsync(host_out, s->scratch, (size_t)S * STATS_COLS * 8, cudaMemcpyDeviceToHost, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "copy stats");

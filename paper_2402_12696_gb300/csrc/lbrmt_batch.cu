@@ -202,10 +202,12 @@ static lbrmt_status capture(lbrmt_batch *b, int nsteps, cudaGraphExec_t *out) {
 }
 
 static lbrmt_status check_members(lbrmt_batch *b) {
-    cudaError_t e = cudaStreamSynchronize(b->stream);
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < (int)b->m.size() && e == cudaSuccess; k++) e = lbrmt_internal_queue_flags(b->m[k].sim);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "stream");
     for (int k = 0; k < (int)b->m.size(); k++) {
-        lbrmt_status st = lbrmt_internal_check_flags(b->m[k].sim);
+        lbrmt_status st = lbrmt_internal_flag_status(b->m[k].sim);
         if (st != LBRMT_OK) return member_fail(b, k, st);
     }
     return LBRMT_OK;

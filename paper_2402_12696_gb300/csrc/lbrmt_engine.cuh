@@ -161,7 +161,8 @@ struct EngineOps {
                         cudaEvent_t *ev, void *tape, int chain);
     cudaError_t (*field)(const SimParams &, const DevState &, int cur, int lastreg, int kind, int solid,
                          double *out, cudaStream_t);
-    cudaError_t (*stats)(const SimParams &, const DevState &, int cur, double *out, cudaStream_t);
+    // flags_out: where the error flags go besides (null: nowhere)
+    cudaError_t (*stats)(const SimParams &, const DevState &, int cur, double *out, unsigned *flags_out, cudaStream_t);
     // per-tile FP64 sums of rho - rho_f of the current populations into d.mass_partials (ntx nty values)
     cudaError_t (*mass)(const SimParams &, const DevState &, int cur, cudaStream_t);
     cudaError_t (*set_pop)(const SimParams &, const DevState &, int cur, const double *src, cudaStream_t);
@@ -604,7 +605,8 @@ struct Engine {
         return nc;
     }
 
-    static cudaError_t stats(const SimParams &sp, const DevState &d, int cur, double *out, cudaStream_t st) {
+    static cudaError_t stats(const SimParams &sp, const DevState &d, int cur, double *out, unsigned *flags_out,
+                             cudaStream_t st) {
         if (sp.nsolids == 0) return cudaSuccess;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
@@ -621,7 +623,7 @@ struct Engine {
                                   (const R *)d.fbody, (const R *)d.bfield, (const int *)d.reg_count[1 - cur],
                                   (const int *)d.reg_solids[1 - cur], (const R *)d.pool[1 - cur],
                                   (const R *)d.xi[cur], (const Frame *)d.frame[cur], (const SolidDesc *)d.solids,
-                                  (const int *)d.order, out);
+                                  (const int *)d.order, out, (const unsigned *)d.err, flags_out);
     }
 
     static cudaError_t mass(const SimParams &sp, const DevState &d, int cur, cudaStream_t st) {

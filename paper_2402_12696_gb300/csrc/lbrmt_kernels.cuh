@@ -3408,7 +3408,9 @@ __global__ void __launch_bounds__(STATS_THREADS, sizeof(R) == 4 ? 3 : 2) solid_s
                                                                     const R *fbody, const R *bfield, const int *reg, const int *reg_solids, const R *pool,
                                                                     const R *xi, const Frame *frames,
                                                                     const SolidDesc *solids, const int *order,
-                                                                    double *out) {
+                                                                    double *out, const unsigned *err,
+                                                                    unsigned *flags_out) {
+    if (flags_out && blockIdx.x == 0 && threadIdx.x == 0) *flags_out = *err;
     __shared__ double red[STATS_THREADS / 32 * STATS_COLS], tot[STATS_COLS];  // sums of the warps, of the CTA
     __shared__ unsigned long long dmax;
     __shared__ int queue[STATS_THREADS / 32][64];  // per warp: < 32 waiting + one round of 32
