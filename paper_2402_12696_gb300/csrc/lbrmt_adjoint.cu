@@ -40,6 +40,8 @@ struct AdjointStore {
     void *fb[2] = {nullptr, nullptr}, *cb[2] = {nullptr, nullptr};
     void *Fb = nullptr, *Db = nullptr, *xib[2] = {nullptr, nullptr};
     double *Gb = nullptr, *dLdc = nullptr;
+    signed char *labels = nullptr;                // per tile node, of the reverse K2
+    int *lists = nullptr;
 };
 
 void lbrmt_internal_adjoint_free(lbrmt_sim *s) {
@@ -179,8 +181,11 @@ static lbrmt_status backward_impl(lbrmt_sim *s, const double *dLdc, double *dLdG
         A.Db = lbrmt_internal_alloc(s, P * sizeof(R));
         A.Gb = (double *)lbrmt_internal_alloc(s, (size_t)std::max(S, 1) * 2 * 8);
         A.dLdc = (double *)lbrmt_internal_alloc(s, (size_t)std::max(S, 1) * 2 * 8);
-        if (!A.fb[0] || !A.fb[1] || !A.cb[0] || !A.cb[1] || !A.xib[0] || !A.xib[1] || !A.Fb || !A.Db || !A.Gb || !A.dLdc)
-            return lbrmt_internal_fail(s, LBRMT_ERR_CUDA, "out of device memory for the adjoint");
+        const size_t nodes = (size_t)(s->xi_total / xi_planes<R>()) + 8;
+        A.labels = (signed char *)lbrmt_internal_alloc(s, nodes);
+        A.lists = (int *)lbrmt_internal_alloc(s, nodes * sizeof(int));
+        if (!A.labels || !A.lists || !A.fb[0] || !A.fb[1] || !A.cb[0] || !A.cb[1] || !A.xib[0] || !A.xib[1] || !A.Fb || !A.Db || !A.Gb || !A.dLdc)
+            return A.Fb = nullptr, lbrmt_internal_fail(s, LBRMT_ERR_CUDA, "out of device memory for the adjoint");
     }
     double *Gb = A.Gb, *Rb = A.Gb + std::max(S, 1);
     R *xib[2] = {(R *)A.xib[0], (R *)A.xib[1]};
@@ -208,13 +213,28 @@ static lbrmt_status backward_impl(lbrmt_sim *s, const double *dLdc, double *dLdG
                             force_adj_smem_max() * (int)sizeof(R)));
     ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, force_adjoint_kernel<R>, TILE_N, fsm));
     const int fblocks = nsm * std::max(per, 1);
-    const int rsm = ((s->li.tmax * s->li.tmax + 15) & ~15) + 8 * LIST_CAP;  // labels and layer lists
-    ok(cudaFuncSetAttribute(rmt_adjoint_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_ADJ_SMEM_MAX));
-    // the forward's choice: 1024-thread CTAs for FP32 arithmetic and few solids
-    constexpr bool can_big = sizeof(R) == 4;
-    const bool big = can_big && s->li.rmt_threads == RMT_THREADS_BIG;
-    if constexpr (can_big)
-        if (big) ok(cudaFuncSetAttribute(rmt_adjoint_kernel_big<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, RMT_ADJ_SMEM_MAX));
+    // K2 reverse: CTAs per solid as in the forward's wide form (one CTA to an SM at most, 8 tile
+    // rows to a CTA), or as many more as its strip needs to fit shared memory
+    const int rcap = RMT_SMEM_CAP - 2048;
+    ok(cudaFuncSetAttribute(rmt_adjoint_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, rcap));
+    ok(cudaFuncSetAttribute(rmt_adjoint_kernel<R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t rcfg = {};
+    cudaLaunchAttribute rat[1];
+    rcfg.blockDim = dim3(RMT_ADJ_THREADS);
+    rcfg.stream = st;
+    rcfg.attrs = rat;
+    rcfg.numAttrs = 1;
+    rat[0].id = cudaLaunchAttributeClusterDimension;
+    rat[0].val.clusterDim.y = rat[0].val.clusterDim.z = 1;
+    for (int nc = 16; nc >= 1 && S > 0; nc /= 2) {
+        if (nc > 1 && (S * nc > nsm || 8 * nc > s->li.tmax) && rmt_adj_smem(s->li.tmax, nc / 2, sp.n_layers) <= rcap) continue;
+        rat[0].val.clusterDim.x = nc;
+        rcfg.gridDim = dim3(S * nc);
+        rcfg.dynamicSmemBytes = rmt_adj_smem(s->li.tmax, nc, sp.n_layers);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, rmt_adjoint_kernel<R>, &rcfg) != cudaSuccess) cudaGetLastError();
+        if (nc == 1 || n > 0) break;
+    }
     const int lblocks = (int)std::min<long long>((P + 255) / 256, (long long)nsm * 8);
     if (e != cudaSuccess) return lbrmt_internal_fail(s, LBRMT_ERR_CUDA, std::string("adjoint setup: ") + cudaGetErrorString(e));
 
@@ -289,13 +309,9 @@ static lbrmt_status backward_impl(lbrmt_sim *s, const double *dLdc, double *dLdG
                 ra.fb = fb[p];
                 ra.cb = cb[p];
                 ra.solids = d.solids;
-                bool launched = false;
-                if constexpr (can_big)
-                    if (big) {
-                        rmt_adjoint_kernel_big<R><<<S, RMT_THREADS_BIG, rsm, st>>>(sp, ra);
-                        launched = true;
-                    }
-                if (!launched) rmt_adjoint_kernel<R><<<S, RMT_THREADS, rsm, st>>>(sp, ra);
+                ra.labels = A.labels;
+                ra.lists = A.lists;
+                ok(cudaLaunchKernelEx(&rcfg, rmt_adjoint_kernel<R>, sp, ra));
                 ok(cudaMemsetAsync(xib[q], 0, xib_bytes, st));
             }
             ok(cudaGetLastError());

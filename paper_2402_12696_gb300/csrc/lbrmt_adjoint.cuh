@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(TILE_N) force_adjoint_kernel(SimParams sp, For
 }
 
 // ---------------------------------------------------------------------------
-// K2 reverse: one solid per CTA.
+// K2 reverse: a cluster of CTAs per solid.
 // ---------------------------------------------------------------------------
 template <class R>
 struct RmtAdjArgs {
@@ -456,26 +456,10 @@ struct RmtAdjArgs {
     R *xib_in;                          // adjoint of xi^n, accumulated
     R *fb, *cb;                         // adjoint of f^n and of the half-force of step n, accumulated
     const SolidDesc *solids;
+    // workspace, per tile node: its layer (-1: none), and the strips' lists of targets
+    signed char *labels;
+    int *lists;
 };
-
-// Normal of phi^n at input-frame node (ix, iy) from central differences, as the forward.
-template <class R>
-__device__ __forceinline__ bool adj_normal(const R *Xi, const R *Yi, int T, int ix, int iy, const Frame &fi,
-                                           const Rsq<R> &rq, R &nhx, R &nhy, R &gxp, R &gyp, R &nn) {
-    if (!(ix > fi.bx0 && iy > fi.by0 && ix < fi.bx1 && iy < fi.by1)) return false;
-    const int k0 = iy * T + ix;
-    const R Xe = Xi[k0 + 1], Xw = Xi[k0 - 1], Xn = Xi[k0 + T], Xs = Xi[k0 - T];
-    if (!(Xe == Xe && Xw == Xw && Xn == Xn && Xs == Xs)) return false;
-    const R pe = phi_eta(Xe, Yi[k0 + 1], ix + 1, iy, fi, rq), pw = phi_eta(Xw, Yi[k0 - 1], ix - 1, iy, fi, rq);
-    const R pn = phi_eta(Xn, Yi[k0 + T], ix, iy + 1, fi, rq), ps = phi_eta(Xs, Yi[k0 - T], ix, iy - 1, fi, rq);
-    gxp = (pe - pw) / R(2);
-    gyp = (pn - ps) / R(2);
-    nn = rsqrt_<R>(gxp * gxp + gyp * gyp);
-    if (!(nn > R(0))) return false;
-    nhx = gxp / nn;
-    nhy = gyp / nn;
-    return true;
-}
 
 // Weight of valid node (dx, dy) relative to the target (0 if the node is not used).
 template <class R>
@@ -492,11 +476,11 @@ __device__ __forceinline__ R adj_weight(const signed char *lab, int k, int l, in
     return wt;
 }
 
-// Reverse of one extrapolated target (tx, ty) of layer l: pass its adjoint
-// (xb, yb) to the nodes of its fit and, for the directional weights, return
-// the adjoint of the unit normal.
+// Reverse of one extrapolated target (tx, ty) of layer l with any window: pass its
+// adjoint (xb, yb) to the nodes of its fit and, for the directional weights, return
+// the adjoint of the unit normal.  One thread; only for the rare windows beyond 5x5.
 template <class R>
-__device__ void extrapolate_adjoint(const SimParams &sp, const signed char *lab, const R *X, const R *Y, R *Xb,
+__device__ __noinline__ void extrapolate_adjoint(const SimParams &sp, const signed char *lab, const R *X, const R *Y, R *Xb,
                                     int T, int tx, int ty, int l, bool use_n, R nhx, R nhy, R xb, R yb, R &nbx,
                                     R &nby) {
     nbx = R(0);
@@ -585,153 +569,429 @@ __device__ void extrapolate_adjoint(const SimParams &sp, const signed char *lab,
         }
 }
 
+// A target's fit in reverse, as RMT_ADJ_LANES lanes hold it: everything that does not
+// depend on its adjoint.
+constexpr int RMT_ADJ_LANES = 8;
 template <class R>
-__device__ void rmt_adjoint_solid(const SimParams &sp, const RmtAdjArgs<R> &a);
+struct AdjPlan {
+    static constexpr int NW = (25 + RMT_ADJ_LANES - 1) / RMT_ADJ_LANES;
+    int e;       // lx | ly << 16; -1: no target
+    bool plane;  // false: a window beyond 5x5 (extrapolate_adjoint)
+    R al[NW];    // d value / d node for the lane's window nodes sub + j RMT_ADJ_LANES
+    // layers 1 and 2, lanes 0-3: the adjoint (px, py) . (xb, yb) of phi^n at the lane's neighbour, d phi / d eta there
+    R px, py, dx, dy;
+};
 
+// K2 reverse of solid s, its band spread over the nc CTAs of a cluster in strips of
+// rows.  The layers of the forward step are formed anew (S from phi^n as bit masks, of
+// the rows that the strip can be reached from) and listed.  Then, in reverse order, eight lanes to a target: its adjoint goes to the nodes of its fit by
+// atomics at L2, one cluster barrier per layer; last the advection of the strip's nodes of S.
+// Bound by that chain's latency: per layer a load, the atomics and the barrier (2 K cycles); the
+// next layer's fits are planned before the barrier's wait.
+// A disk of radius 39 on 256^2 (16 CTAs) takes, in cycles, S 5 K, the layers and lists 11 K,
+// layers 11-3 27 K, layers 2-1 14 K, the advection 7 K: 120 -> 34 us against one CTA of 1024 threads
+// with byte labels, a target per thread and a window walked three times.
 template <class R>
-__global__ void __launch_bounds__(RMT_THREADS) rmt_adjoint_kernel(SimParams sp, RmtAdjArgs<R> a) {
-    rmt_adjoint_solid<R>(sp, a);
-}
-
-// 1024-thread CTAs for FP32 simulations with few solids (as the forward kernel).
-template <class R>
-__global__ void __launch_bounds__(RMT_THREADS_BIG, 1) rmt_adjoint_kernel_big(SimParams sp, RmtAdjArgs<R> a) {
-    rmt_adjoint_solid<R>(sp, a);
-}
-
-template <class R>
-__device__ void rmt_adjoint_solid(const SimParams &sp, const RmtAdjArgs<R> &a) {
+__global__ void __launch_bounds__(RMT_ADJ_THREADS, 1) rmt_adjoint_kernel(SimParams sp, RmtAdjArgs<R> a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int bb[4];
-    __shared__ int lcnt[24], loff[24];
-    const int s = blockIdx.x;
-    const SolidDesc sd = a.solids[s];
-    const int T = sd.T, TT = T * T;
-    const int lane = threadIdx.x & 31;
-    signed char *lab = reinterpret_cast<signed char *>(smem);
+    __shared__ int loff[24];  // a layer's targets: list[loff[l] .. loff[l + 1])
+    __shared__ int fill[24];  // their number
+    __shared__ int lut[32];
+    __shared__ R rd[25], wd[25];  // 1 / |d| of the window's nodes, times 2^-(|dx|+|dy|)
+    const int nc = cluster_size(), rank = cluster_rank(), s = (int)blockIdx.x / nc;
+    const SolidDesc &sd = a.solids[s];
+    const int NL = sp.n_layers, T = sd.T, TT = T * T, rw = mask_row_words(T), mw = mask_words(T, nc, NL);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = RMT_ADJ_THREADS / 32;
     const Frame fo = a.frame_out[s], fi = a.frame_in[s];
     const int2 oo = make_int2(fo.ox, fo.oy);
     const int shx = fo.ox - fi.ox, shy = fo.oy - fi.oy;
-    const Rsq<R> rq(sd);
-    const R *Xi = a.xi_in + sd.off, *Yi = Xi + TT;
+    const R *Xi = a.xi_in + sd.off, *Yi = Xi + TT, *Pi = Yi + TT;
     const R *Xo = a.xi_out + sd.off, *Yo = Xo + TT;
     R *XbO = a.xib_out + sd.off;
     R *XbI = a.xib_in + sd.off;
-    const R eps = pick<R>(sp.eps, sp.eps_f);
-    const long long P = sp.P;
-    if (threadIdx.x < 4) bb[threadIdx.x] = (threadIdx.x & 1) ? -(1 << 29) : (1 << 29);
-    if (threadIdx.x < 24) lcnt[threadIdx.x] = 0;
-    for (int k = threadIdx.x; k < (TT + 15) >> 4; k += blockDim.x)
-        reinterpret_cast<int4 *>(lab)[k] = make_int4(-1, -1, -1, -1);
-    int sb[4] = {1 << 29, -(1 << 29), 1 << 29, -(1 << 29)};
+    const long long P = sp.P, node0 = sd.off / xi_planes<R>();
+    signed char *lab = a.labels + node0;
+    // the band's box and this CTA's rows of it (the forward recorded the box)
+    const int x0 = fo.bx0, x1 = fo.bx1, y0 = fo.by0, y1 = fo.by1;
+    if (x0 > x1 || y0 > y1) return;  // uniform over the cluster
+    const Strips st = {y0, y1, 31 - __clz(nc), NL};
+    const int yr0 = st.first(rank), yr1 = st.first(rank + 1);
+    const int my0 = st.set_first(rank);
+    const RowMask mS = {reinterpret_cast<unsigned *>(smem), rw, st.set_first(rank)};
+    // layers of the strip and two halo rows and columns (NL + 1: none): node (x, y) at slab[(y - yr0 + 2) ls + x - x0 + 2]
+    const int ls = x1 - x0 + 5, lh = yr1 - yr0 + 4;
+    int *const slist = reinterpret_cast<int *>(mS.p + mw);  // the layers' targets, where they fit
+    unsigned char *slab = reinterpret_cast<unsigned char *>(slist + RMT_ADJ_LIST), *srow = slab + ls * lh;
+    if (tid < 24) loff[tid] = 0;
+    if (tid < 24) fill[tid] = 0;
+    if (tid < 32) lut[tid] = row_moments(tid);
+    if (tid >= 32 && tid < 57) {
+        const int dx = (tid - 32) % 5 - 2, dy = (tid - 32) / 5 - 2;
+        rd[tid - 32] = rinv_tab<R>(dx, dy);
+        wd[tid - 32] = pow2neg<R>(abs(dx) + abs(dy)) * rinv_tab<R>(dx, dy);
+    }
+    for (int k = tid; k < mw / 4; k += RMT_ADJ_THREADS) reinterpret_cast<int4 *>(smem)[k] = make_int4(0, 0, 0, 0);
+    {  // labels for a fit beyond its 5x5 window (extrapolate_adjoint): this CTA's rows, free
+        const int c0 = rank == 0 ? 0 : yr0 * T, c1 = rank == nc - 1 ? TT : yr1 * T;  // T: a multiple of 8
+        for (int k = c0 + 8 * tid; k < c1; k += 8 * RMT_ADJ_THREADS) *reinterpret_cast<int2 *>(lab + k) = make_int2(-1, -1);
+    }
     __syncthreads();
-    // the advected set S^n and its stencil conditions, as the forward
-    {
-        const int bw = fi.bx1 - fi.bx0 + 1, bn = (fi.bx1 >= fi.bx0 && fi.by1 >= fi.by0) ? bw * (fi.by1 - fi.by0 + 1) : 0;
-        for (int kk = threadIdx.x; kk < bn; kk += blockDim.x) {
-            const int ix = fi.bx0 + kk % bw, iy = fi.by0 + kk / bw;
-            const int lx = ix - shx, ly = iy - shy, gx = oo.x + lx, gy = oo.y + ly;
-            const int k = iy * T + ix;
-            const R ex = Xi[k];
-            if (!(ex == ex)) continue;
-            const R phi = phi_eta(ex, Yi[k], ix, iy, fi, rq);
-            if (!(phi < eps) || !domain_cell(sp, gx, gy)) continue;
-            if (lx < 0 || ly < 0 || lx >= T || ly >= T) continue;
-            if (!(phi < -R(PHI_TIE))) continue;
-            const long long c = (long long)wrapi(gy, sp.ny) * sp.nx + wrapi(gx, sp.nx);
-            const R u = a.tape[P + c], v = a.tape[2 * P + c];
-            const int sx = (u >= R(0)) ? -1 : 1, sy = (v >= R(0)) ? -1 : 1;
-            const int x2 = ix + 2 * sx, y2 = iy + 2 * sy;
-            if (x2 < fi.bx0 || x2 > fi.bx1 || y2 < fi.by0 || y2 > fi.by1) continue;
-            lab[ly * T + lx] = 0;
-            sb[0] = min(sb[0], lx); sb[1] = max(sb[1], lx); sb[2] = min(sb[2], ly); sb[3] = max(sb[3], ly);
+    const int wa = (x0 + 32) >> 5, wn = ((x1 + 32) >> 5) - wa + 1;
+    const unsigned wdiv = wn > 1 ? 0xffffffffu / (unsigned)wn + 1u : 0u;  // k / wn = umulhi(k, wdiv) for k wn < 2^32
+    {  // S: a warp per mask word, of the rows that the strip and its halo can be reached from
+        const int r0 = max(yr0 - NL - 2, y0), n = (min(yr1 + NL + 1, y1) - r0 + 1) * wn;
+        // the input box, within the domain
+        const int ax = max(fi.bx0 - shx, sp.wall_x ? -oo.x : 0), ay = max(fi.by0 - shy, sp.wall_y ? -oo.y : 0);
+        const int ex = min(min(fi.bx1 - shx, T - 1), sp.wall_x ? sp.nx - 1 - oo.x : T - 1);
+        const int ey = min(min(fi.by1 - shy, T - 1), sp.wall_y ? sp.ny - 1 - oo.y : T - 1);
+        for (int k0 = warp; k0 < n; k0 += 4 * nw) {
+            R ph[4];
+            int at[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int k = k0 + q * nw, row = wn > 1 ? (int)__umulhi((unsigned)k, wdiv) : k, w = wa + k - row * wn;
+                const int ly = r0 + row, lx = 32 * w - 32 + lane;
+                at[q] = k < n ? (ly - mS.y0) * rw + w : -1;  // uniform over the warp
+                ph[q] = R(0);
+                if (k < n && lx >= max(ax, 0) && lx <= ex && ly >= ay && ly <= ey) ph[q] = Pi[(ly + shy) * T + lx + shx];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const unsigned m = __ballot_sync(0xffffffffu, ph[q] < -R(PHI_TIE));
+                if (lane == 0 && at[q] >= 0) mS.p[at[q]] = m;
+            }
         }
     }
-    for (int k = 0; k < 4; k++) warp_minmax(sb[k], (k & 1) == 0);
-    if (lane == 0) { atomicMin(&bb[0], sb[0]); atomicMax(&bb[1], sb[1]); atomicMin(&bb[2], sb[2]); atomicMax(&bb[3], sb[3]); }
     __syncthreads();
-    const int sx0 = bb[0], sx1 = bb[1], sy0 = bb[2], sy1 = bb[3];
-    if (sx0 > sx1) return;
-    const int NL = sp.n_layers;
-    // the layers, as the forward, listed so that a layer's targets fill whole warps
-    int *lists = reinterpret_cast<int *>(smem + ((TT + 15) & ~15));
-    label_layers_l1(sp, lab, T, sx0, sx1, sy0, sy1, oo, NL, lcnt);
-    __syncthreads();
-    const bool listed = list_layers(lab, T, max(sx0 - NL, 0), min(sx1 + NL, T - 1), max(sy0 - NL, 0),
-                                    min(sy1 + NL, T - 1), NL, lcnt, loff, lists, 2 * LIST_CAP);
-    // extrapolated layers in reverse order
-    for (int l = NL; l >= 1; l--) {
-        const int nitems = listed ? loff[l + 1] - loff[l] : TT;
-        for (int k = threadIdx.x; k < nitems; k += blockDim.x) {
-            int lx, ly;
-            if (listed) {
-                const int e = lists[loff[l] + k];
-                lx = e & 0xffff; ly = e >> 16;
-            } else {  // too many band nodes for the lists: scan the tile
-                lx = k % T; ly = k / T;
-                if (lab[k] != l) continue;
-            }
-            const int t = ly * T + lx;
-            const R xb = XbO[t], yb = XbO[TT + t];
-            if (xb == R(0) && yb == R(0)) continue;
-            bool use_n = false;
-            R nhx = 0, nhy = 0, gxp = 0, gyp = 0, nn = 0;
-            const int ix = lx + shx, iy = ly + shy;
-            if (l <= 2) use_n = adj_normal<R>(Xi, Yi, T, ix, iy, fi, rq, nhx, nhy, gxp, gyp, nn);
-            R nbx, nby;
-            extrapolate_adjoint<R>(sp, lab, Xo, Yo, XbO, T, lx, ly, l, use_n, nhx, nhy, xb, yb, nbx, nby);
-            if (use_n && (nbx != R(0) || nby != R(0))) {
-                // n = g / |g|, g = central differences of phi^n
-                const R ndot = nhx * nbx + nhy * nby;
-                const R gbx = (nbx - nhx * ndot) / nn, gby = (nby - nhy * ndot) / nn;
-                const int k0 = iy * T + ix;
-                const int kn[4] = {k0 + 1, k0 - 1, k0 + T, k0 - T};
-                const int nxo[4] = {1, -1, 0, 0}, nyo[4] = {0, 0, 1, -1};
-                const R pbv[4] = {gbx / R(2), -gbx / R(2), gby / R(2), -gby / R(2)};
-                for (int m = 0; m < 4; m++) {
-                    R dx_, dy_;
-                    dphi_deta<R>(Xi[kn[m]], Yi[kn[m]], ix + nxo[m], iy + nyo[m], fi, dx_, dy_);
-                    atomicAdd(&XbI[kn[m]], pbv[m] * dx_);
-                    atomicAdd(&XbI[TT + kn[m]], pbv[m] * dy_);
+    // The layer of each node of the strip and its halo, the number of 4-neighbour steps to S:
+    // the steps along its row to the nearest set bit (from a window of the row's mask, 2 NL
+    // + 1 bits), then the least over the rows around it, nearest first.
+    const int hr0 = yr0 - 2 - NL;
+    {
+        BoxWalk wl(ls);
+        for (int k = tid; k < ls * (lh + 2 * NL); k += RMT_ADJ_THREADS, wl.next()) {
+            const int x = x0 - 2 + wl.c, y = hr0 + wl.r;
+            int d = 64;
+            if (x >= x0 && x <= x1 && y >= y0 && y <= y1) {
+                const int sh = (x - NL + 64) & 31, wi = ((x - NL + 64) >> 5) - 1;  // bit 0 of the window: node x - NL
+                const unsigned *r = mS.p + (y - mS.y0) * rw + wi;
+                const unsigned a0 = r[0], a1 = wi + 1 < rw ? r[1] : 0u, lo = __funnelshift_r(a0, a1, sh);
+                if (NL <= 15) {
+                    d = min(__clz(__brev(lo >> NL)), __clz(lo << (31 - NL)));
+                } else {
+                    const unsigned hi = __funnelshift_r(a1, wi + 2 < rw ? r[2] : 0u, sh);
+                    const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+                    d = min(__clzll(__brevll(m >> NL)), __clzll(m << (63 - NL)));
                 }
             }
+            srow[k] = (unsigned char)d;
         }
-        __syncthreads();
     }
-    // advected nodes: eta^{n+1} = eta - (u - dd) - u d_x eta - v d_y eta (one-sided, upwind)
+    __syncthreads();
     {
-        const int w = sx1 - sx0 + 1, nb = w * (sy1 - sy0 + 1);
-        for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-            const int lx = sx0 + k % w, ly = sy0 + k / w, t = ly * T + lx;
-            if (lab[t] != 0) continue;
-            const R Xb = XbO[t], Yb = XbO[TT + t];
-            if (Xb == R(0) && Yb == R(0)) continue;
-            const int ix = lx + shx, iy = ly + shy, kk = iy * T + ix;
-            const int gx = oo.x + lx, gy = oo.y + ly;
-            const long long c = (long long)wrapi(gy, sp.ny) * sp.nx + wrapi(gx, sp.nx);
-            const R rho = a.tape[c], u = a.tape[P + c], v = a.tape[2 * P + c];
-            const int sx = (u >= R(0)) ? -1 : 1, sy = (v >= R(0)) ? -1 : 1;
-            const int k1 = kk + sx, k2 = kk + 2 * sx, k3 = kk + sy * T, k4 = kk + 2 * sy * T;
-            const R hx = R(-sx) * R(0.5), hy = R(-sy) * R(0.5);
-            const R ex = Xi[kk], ey = Yi[kk];
-            const R dXdx = hx * (R(3) * ex - R(4) * Xi[k1] + Xi[k2]), dYdx = hx * (R(3) * ey - R(4) * Yi[k1] + Yi[k2]);
-            const R dXdy = hy * (R(3) * ex - R(4) * Xi[k3] + Xi[k4]), dYdy = hy * (R(3) * ey - R(4) * Yi[k3] + Yi[k4]);
-            const R c0 = R(1) - R(3) * (u * hx + v * hy);
-            atomicAdd(&XbI[kk], Xb * c0); atomicAdd(&XbI[TT + kk], Yb * c0);
-            atomicAdd(&XbI[k1], Xb * R(4) * u * hx); atomicAdd(&XbI[TT + k1], Yb * R(4) * u * hx);
-            atomicAdd(&XbI[k2], -Xb * u * hx); atomicAdd(&XbI[TT + k2], -Yb * u * hx);
-            atomicAdd(&XbI[k3], Xb * R(4) * v * hy); atomicAdd(&XbI[TT + k3], Yb * R(4) * v * hy);
-            atomicAdd(&XbI[k4], -Xb * v * hy); atomicAdd(&XbI[TT + k4], -Yb * v * hy);
-            const R ub = -Xb * (R(1) + dXdx) - Yb * dYdx;
-            const R vb = -Xb * dXdy - Yb * (R(1) + dYdy);
-            // u = (sum c f + half-force) / rho
-            const R inv = R(1) / rho;
-#pragma unroll
-            for (int q = 0; q < 9; q++)
-                atomicAdd(&a.fb[q * P + c], ((R(cxq(q)) - u) * ub + (R(cyq(q)) - v) * vb) * inv);
-            atomicAdd(&a.cb[c], ub * inv);
-            atomicAdd(&a.cb[P + c], vb * inv);
+        BoxWalk wl(ls);
+        for (int k = tid; k < ls * lh; k += RMT_ADJ_THREADS, wl.next()) {
+            const int x = x0 - 2 + wl.c, y = yr0 - 2 + wl.r;
+            const unsigned char *r = srow + k + NL * ls;
+            int l = NL + 1;
+            if (x >= x0 && x <= x1 && y >= y0 && y <= y1) {
+                l = min(l, (int)r[0]);
+                for (int dy = 1; dy < l; dy++) l = min(l, dy + min((int)r[-dy * ls], (int)r[dy * ls]));
+            }
+            slab[k] = (unsigned char)l;
         }
+    }
+    __syncthreads();
+    // The lists, a layer per warp (counters in shared memory would take an atomic per node on
+    // as few addresses as there are layers).
+    const int ns = (yr1 - yr0) * ls;  // the strip's rows, with their free halo columns
+    const unsigned char *strip = slab + 2 * ls;
+    const unsigned lsdiv = 0xffffffffu / (unsigned)ls + 1u;  // k / ls = umulhi(k, lsdiv) for k ls < 2^32
+    for (int l = warp + 1; l <= NL; l += nw) {
+        int c = 0;
+        for (int k = lane; k < ns; k += 32) c += strip[k] == l ? 1 : 0;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) fill[l] = c;
+    }
+    __syncthreads();
+    if (warp == 0) {  // ends of the layers
+        int e = lane >= 1 && lane <= NL ? fill[lane] : 0;
+        for (int d = 1; d < 32; d *= 2) {
+            const int v = __shfl_up_sync(0xffffffffu, e, d);
+            if (lane >= d) e += v;
+        }
+        if (lane >= 1 && lane <= NL) loff[lane + 1] = e;
+    }
+    __syncthreads();
+    int *const list = loff[NL + 1] <= RMT_ADJ_LIST ? slist : a.lists + node0 + (long long)yr0 * T;
+    for (int l = warp; l <= NL; l += nw) {
+        int at = loff[max(l, 1)];
+        for (int k0 = 0; k0 < ns; k0 += 128) {
+            unsigned m[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int k = k0 + 32 * q + lane;
+                m[q] = __ballot_sync(0xffffffffu, k < ns && strip[min(k, ns - 1)] == l);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if ((m[q] >> lane) & 1u) {
+                    const int k = k0 + 32 * q + lane, r = (int)__umulhi((unsigned)k, lsdiv), x = x0 - 2 + k - r * ls, y = yr0 + r;
+                    lab[y * T + x] = (signed char)l;
+                    if (l > 0) list[at + __popc(m[q] & ((1u << lane) - 1u))] = x | (y << 16);
+                }
+                at += __popc(m[q]);
+            }
+        }
+    }
+    __syncthreads();
+    constexpr int L = RMT_ADJ_LANES, NW = AdjPlan<R>::NW, G = RMT_ADJ_THREADS / L;
+    const int sub = lane % L;
+    const unsigned gm = (0xffffffffu >> (32 - L)) << (lane & ~(L - 1));
+    auto sum = [&](R v) {
+#pragma unroll
+        for (int d = L / 2; d > 0; d >>= 1) v += __shfl_xor_sync(gm, v, d);
+        return v;
+    };
+    // layers 1 and 2: the normal of phi^n from central differences, as the forward
+    auto normal = [&](int l, int lx, int ly, R &nhx, R &nhy, R &nn) {
+        const int ix = lx + shx, iy = ly + shy, k0 = iy * T + ix;
+        nhx = nhy = nn = R(0);
+        if (l > 2 || !(ix > fi.bx0 && iy > fi.by0 && ix < fi.bx1 && iy < fi.by1)) return false;
+        const R Xe = Xi[k0 + 1], Xw = Xi[k0 - 1], Xn = Xi[k0 + T], Xs = Xi[k0 - T];
+        const R gx = (Pi[k0 + 1] - Pi[k0 - 1]) * R(0.5), gy = (Pi[k0 + T] - Pi[k0 - T]) * R(0.5);
+        nn = rsqrt_<R>(gx * gx + gy * gy);
+        nhx = gx / nn;
+        nhy = gy / nn;
+        return Xe == Xe && Xw == Xw && Xn == Xn && Xs == Xs && nn > R(0);
+    };
+    // the neighbour of lane sub (< 4) in the central differences
+    auto nbr = [&](int sb, int &ox, int &oy) {
+        ox = sb < 2 ? 1 - 2 * sb : 0;
+        oy = sb < 2 ? 0 : 5 - 2 * sb;
+    };
+    auto make = [&](int l, int k) {  // uniform over the lanes of a target
+        AdjPlan<R> p;
+        p.e = -1;
+        p.plane = true;
+        p.px = p.py = p.dx = p.dy = R(0);
+        if (k >= loff[l + 1]) return p;
+        p.e = list[k];
+        const int lx = p.e & 0xffff, ly = p.e >> 16, t = ly * T + lx;
+        unsigned own = 0;  // the fit's nodes among the lane's, of earlier layers
+#pragma unroll
+        for (int j = 0; j < NW; j++) {
+            const int w = sub + j * L;
+            if (w < 25 && slab[(ly - yr0 + w / 5) * ls + lx - x0 + w % 5] < l) own |= 1u << w;
+        }
+        const unsigned bits = __reduce_or_sync(gm, own);
+        R nhx, nhy, nn;
+        const bool use_n = normal(l, lx, ly, nhx, nhy, nn);
+        int c13, c23, c33;
+        if (!use_n) {
+            const int det = window_moments(lut, bits, c13, c23, c33);
+            p.plane = det != 0;
+            const R id = R(16) / whole<R>(det);  // the moments carry powers of 16: (c / 16^2) / (det / 16^3)
+            const R g0 = whole<R>(c13) * id, g1 = whole<R>(c23) * id, g2 = whole<R>(c33) * id;  // M^-1 e3
+#pragma unroll
+            for (int j = 0; j < NW; j++) {
+                const int w = sub + j * L, dx = w % 5 - 2, dy = w / 5 - 2;
+                p.al[j] = w < 25 && ((bits >> w) & 1u) ? pow2neg<R>(abs(dx) + abs(dy)) * (g0 * R(dx) + g1 * R(dy) + g2) : R(0);
+            }
+            return p;
+        }
+        // directional weights 2^-(|dx|+|dy|) dn; the inverse of M = [[a b c],[b d e],[c e f]]
+        R wt[NW], m[6] = {R(0), R(0), R(0), R(0), R(0), R(0)}, Xv[NW], Yv[NW];
+        unsigned mine = 0;
+        const R xref = Xo[t], yref = Yo[t];  // the fit's value at the target
+#pragma unroll
+        for (int j = 0; j < NW; j++) {
+            const int w = sub + j * L, q = t + (w / 5 - 2) * T + w % 5 - 2;
+            const bool on = w < 25 && ((bits >> w) & 1u);
+            Xv[j] = on ? Xo[q] : xref;
+            Yv[j] = on ? Yo[q] : yref;
+            const R x = R(w % 5 - 2), y = R(w / 5 - 2);
+            R v = R(0);
+            if (on) {
+                const R dn = (-x * nhx - y * nhy) * rd[w];
+                if (dn > R(COS_TIE)) v = dn * pow2neg<R>(abs(w % 5 - 2) + abs(w / 5 - 2));
+            }
+            if (v > R(0)) mine |= 1u << w;
+            wt[j] = v;
+            const R wx = v * x, wy = v * y;
+            m[0] += wx * x; m[1] += wx * y; m[2] += wx; m[3] += wy * y; m[4] += wy; m[5] += v;
+        }
+        const unsigned pos = __reduce_or_sync(gm, mine);  // nodes of positive weight
+        p.plane = window_moments(lut, pos, c13, c23, c33) != 0;
+#pragma unroll
+        for (int j = 0; j < 6; j++) m[j] = sum(m[j]);
+        const R C11 = m[3] * m[5] - m[4] * m[4], C12 = m[2] * m[4] - m[1] * m[5], C13 = m[1] * m[4] - m[2] * m[3];
+        const R C22 = m[0] * m[5] - m[2] * m[2], C23 = m[1] * m[2] - m[0] * m[4], C33 = m[0] * m[3] - m[1] * m[1];
+        const R det = m[0] * C11 + m[1] * C12 + m[2] * C13;
+        p.plane = p.plane && det != R(0);
+        const R id = R(1) / det, g0 = C13 * id, g1 = C23 * id, g2 = C33 * id;
+        // d value / d w_k = (M^-1 e3 . (dx, dy, 1)) residual_k
+        R b[6] = {R(0), R(0), R(0), R(0), R(0), R(0)}, nb[4] = {R(0), R(0), R(0), R(0)};
+#pragma unroll
+        for (int j = 0; j < NW; j++) {
+            const int w = sub + j * L;
+            const R x = R(w % 5 - 2), y = R(w / 5 - 2), wx = wt[j] * x, wy = wt[j] * y;
+            p.al[j] = wt[j] * (g0 * x + g1 * y + g2);
+            Xv[j] -= xref;
+            Yv[j] -= yref;
+            b[0] += wx * Xv[j]; b[1] += wy * Xv[j]; b[2] += wt[j] * Xv[j];
+            b[3] += wx * Yv[j]; b[4] += wy * Yv[j]; b[5] += wt[j] * Yv[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 6; j++) b[j] = sum(b[j]);
+        const R cX0 = (C11 * b[0] + C12 * b[1] + C13 * b[2]) * id, cX1 = (C12 * b[0] + C22 * b[1] + C23 * b[2]) * id;
+        const R cX2 = (C13 * b[0] + C23 * b[1] + C33 * b[2]) * id;
+        const R cY0 = (C11 * b[3] + C12 * b[4] + C13 * b[5]) * id, cY1 = (C12 * b[3] + C22 * b[4] + C23 * b[5]) * id;
+        const R cY2 = (C13 * b[3] + C23 * b[4] + C33 * b[5]) * id;
+#pragma unroll
+        for (int j = 0; j < NW; j++) {
+            const int w = sub + j * L;
+            if (!(wt[j] > R(0))) continue;
+            const R x = R(w % 5 - 2), y = R(w / 5 - 2), g = (g0 * x + g1 * y + g2) * wd[w];
+            const R rx = (Xv[j] - (cX0 * x + cX1 * y + cX2)) * g, ry = (Yv[j] - (cY0 * x + cY1 * y + cY2)) * g;
+            nb[0] -= x * rx; nb[1] -= y * rx; nb[2] -= x * ry; nb[3] -= y * ry;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) nb[j] = sum(nb[j]);
+        if (sub < 4) {
+            // n = g / |g|, g = central differences of phi^n
+            const R n1 = nhx * nb[0] + nhy * nb[1], n2 = nhx * nb[2] + nhy * nb[3];
+            const R h = (sub & 1) ? R(-0.5) / nn : R(0.5) / nn;
+            p.px = h * (sub < 2 ? nb[0] - nhx * n1 : nb[1] - nhy * n1);
+            p.py = h * (sub < 2 ? nb[2] - nhx * n2 : nb[3] - nhy * n2);
+            int ox, oy;
+            nbr(sub, ox, oy);
+            const int ix = lx + shx + ox, iy = ly + shy + oy, q = iy * T + ix;
+            dphi_deta<R>(Xi[q], Yi[q], ix, iy, fi, p.dx, p.dy);
+        }
+        return p;
+    };
+    auto apply = [&](int l, const AdjPlan<R> &p) {
+        if (p.e < 0) return;
+        const int lx = p.e & 0xffff, ly = p.e >> 16, t = ly * T + lx;
+        const R xb = __ldcg(XbO + t), yb = __ldcg(XbO + TT + t);
+        if (xb == R(0) && yb == R(0)) return;
+        if (!p.plane) {
+            if (sub) return;
+            R nhx, nhy, nn, nbx, nby;
+            const bool use_n = normal(l, lx, ly, nhx, nhy, nn);
+            extrapolate_adjoint<R>(sp, lab, Xo, Yo, XbO, T, lx, ly, l, use_n, nhx, nhy, xb, yb, nbx, nby);
+            if (!use_n || (nbx == R(0) && nby == R(0))) return;
+            const R nd = nhx * nbx + nhy * nby;
+            for (int m = 0; m < 4; m++) {
+                int ox, oy;
+                nbr(m, ox, oy);
+                const int ix = lx + shx + ox, iy = ly + shy + oy, q = iy * T + ix;
+                const R pb = (m < 2 ? nbx - nhx * nd : nby - nhy * nd) * ((m & 1) ? R(-0.5) : R(0.5)) / nn;
+                R dx, dy;
+                dphi_deta<R>(Xi[q], Yi[q], ix, iy, fi, dx, dy);
+                atomicAdd(&XbI[q], pb * dx);
+                atomicAdd(&XbI[TT + q], pb * dy);
+            }
+            return;
+        }
+#pragma unroll
+        for (int j = 0; j < NW; j++) {
+            const int w = sub + j * L, q = t + (w / 5 - 2) * T + w % 5 - 2;
+            if (p.al[j] == R(0)) continue;
+            atomicAdd(&XbO[q], p.al[j] * xb);
+            atomicAdd(&XbO[TT + q], p.al[j] * yb);
+        }
+        const R pb = p.px * xb + p.py * yb;
+        if (pb != R(0)) {
+            int ox, oy;
+            nbr(sub, ox, oy);
+            const int q = (ly + shy + oy) * T + lx + shx + ox;
+            atomicAdd(&XbI[q], pb * p.dx);
+            atomicAdd(&XbI[TT + q], pb * p.dy);
+        }
+    };
+    // An advected node: eta^{n+1} = eta - (u - dd) - u d_x eta - v d_y eta (one-sided, upwind).
+    struct Adv {
+        int t, kk;  // output and input tile node; t < 0: none
+        long long c;
+        R rho, u, v, dXdx, dYdx, dXdy, dYdy;
+    };
+    const int nadv = (x1 - x0 + 1) * (yr1 - yr0);
+    BoxWalk wk(x1 - x0 + 1);
+    auto adv_load = [&](int k) {  // wk stands at node k
+        Adv n;
+        const int lx = x0 + wk.c, ly = yr0 + wk.r;
+        n.t = -1;
+        if (k >= nadv || !mS.bit(lx, ly)) return n;
+        const int ix = lx + shx, iy = ly + shy, kk = iy * T + ix;
+        n.kk = kk;
+        n.c = (long long)wrapi(oo.y + ly, sp.ny) * sp.nx + wrapi(oo.x + lx, sp.nx);
+        n.rho = a.tape[n.c];
+        n.u = a.tape[P + n.c];
+        n.v = a.tape[2 * P + n.c];
+        const int sx = (n.u >= R(0)) ? -1 : 1, sy = (n.v >= R(0)) ? -1 : 1;
+        const int x2 = ix + 2 * sx, y2 = iy + 2 * sy;
+        if (x2 < fi.bx0 || x2 > fi.bx1 || y2 < fi.by0 || y2 > fi.by1) return n;  // the forward flagged it
+        n.t = ly * T + lx;
+        const int k1 = kk + sx, k2 = kk + 2 * sx, k3 = kk + sy * T, k4 = kk + 2 * sy * T;
+        const R hx = R(-sx) * R(0.5), hy = R(-sy) * R(0.5), ex = Xi[kk], ey = Yi[kk];
+        n.dXdx = hx * (R(3) * ex - R(4) * Xi[k1] + Xi[k2]);
+        n.dYdx = hx * (R(3) * ey - R(4) * Yi[k1] + Yi[k2]);
+        n.dXdy = hy * (R(3) * ex - R(4) * Xi[k3] + Xi[k4]);
+        n.dYdy = hy * (R(3) * ey - R(4) * Yi[k3] + Yi[k4]);
+        return n;
+    };
+    auto adv_apply = [&](const Adv &n) {
+        if (n.t < 0) return;
+        const R Xb = __ldcg(XbO + n.t), Yb = __ldcg(XbO + TT + n.t), u = n.u, v = n.v;
+        if (Xb == R(0) && Yb == R(0)) return;
+        const int sx = (u >= R(0)) ? -1 : 1, sy = (v >= R(0)) ? -1 : 1;
+        const int kk = n.kk, k1 = kk + sx, k2 = kk + 2 * sx, k3 = kk + sy * T, k4 = kk + 2 * sy * T;
+        const R hx = R(-sx) * R(0.5), hy = R(-sy) * R(0.5);
+        const R c0 = R(1) - R(3) * (u * hx + v * hy);
+        atomicAdd(&XbI[kk], Xb * c0); atomicAdd(&XbI[TT + kk], Yb * c0);
+        atomicAdd(&XbI[k1], Xb * R(4) * u * hx); atomicAdd(&XbI[TT + k1], Yb * R(4) * u * hx);
+        atomicAdd(&XbI[k2], -Xb * u * hx); atomicAdd(&XbI[TT + k2], -Yb * u * hx);
+        atomicAdd(&XbI[k3], Xb * R(4) * v * hy); atomicAdd(&XbI[TT + k3], Yb * R(4) * v * hy);
+        atomicAdd(&XbI[k4], -Xb * v * hy); atomicAdd(&XbI[TT + k4], -Yb * v * hy);
+        const R ub = -Xb * (R(1) + n.dXdx) - Yb * n.dYdx;
+        const R vb = -Xb * n.dXdy - Yb * (R(1) + n.dYdy);
+        // u = (sum c f + half-force) / rho
+        const R inv = R(1) / n.rho;
+#pragma unroll
+        for (int q = 0; q < 9; q++)
+            atomicAdd(&a.fb[q * P + n.c], ((R(cxq(q)) - u) * ub + (R(cyq(q)) - v) * vb) * inv);
+        atomicAdd(&a.cb[n.c], ub * inv);
+        atomicAdd(&a.cb[P + n.c], vb * inv);
+    };
+    // One layer after the other, G targets at a time; the next ones' plan is made between
+    // the arrival at a layer's barrier and the wait (the first barrier: the labels).  One
+    // place for each of the pieces: a launch runs through its code but once, and every line of it
+    // is fetched anew.
+    AdjPlan<R> p;
+    p.e = -1;
+    int l = NL + 1, k = 0, rounds = 1;  // rounds of the layer left
+    while (true) {
+        apply(l, p);
+        const bool last = --rounds == 0;
+        if (last) {
+            cluster_arrive();
+            if (--l == 0) break;
+            k = loff[l] + tid / L;
+            rounds = max((loff[l + 1] - loff[l] + G - 1) / G, 1);
+        } else {
+            k += G;
+        }
+        p = make(l, k);
+        if (last) cluster_wait();
+    }
+    // advected nodes
+    for (int i = tid;; i += RMT_ADJ_THREADS, wk.next()) {
+        const Adv n = adv_load(i);
+        if (i == tid) cluster_wait();  // layer 1's
+        if (i >= nadv) break;
+        adv_apply(n);
     }
 }
 

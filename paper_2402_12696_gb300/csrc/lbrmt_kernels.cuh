@@ -66,9 +66,11 @@ __host__ __device__ constexpr int rmt_wide_smem(int T, int nc, int NL, int real)
            2 * plan_cap(real) * plan_bytes(real) + 2 * real * strip_values(T, nc);
 }
 constexpr int RMT_SMEM_MAX = rmt_mask_bytes(TILE_SIDE_MAX, 1, 20) + RMT_LIST_BYTES;
-// Shared memory of the reverse sweep's K2: byte labels and layer lists.
-constexpr int LIST_CAP = 2048;
-constexpr int RMT_ADJ_SMEM_MAX = ((TILE_SIDE_MAX * TILE_SIDE_MAX + 15) & ~15) + 8 * LIST_CAP;
+// Threads and shared memory (the set S, a list, the layers of a strip and its halo) of the reverse sweep's K2.
+constexpr int RMT_ADJ_THREADS = 512, RMT_ADJ_LIST = 2048;
+__host__ __device__ constexpr int rmt_adj_smem(int T, int nc, int NL) {
+    return 4 * mask_words(T, nc, NL) + 4 * RMT_ADJ_LIST + ((2 * ((T + nc - 1) / nc + 4) + 2 * NL) * (T + 5) + 15 & ~15);
+}
 // Force pool, per registered tile, TILE_N values per plane: F_x and F_y of the
 // solid terms (without the body force), Delta rho as an unevaluated sum hi + lo
 // (two planes' worth, the pair of node lt at POOL_DRHO + 2 lt, read as one
@@ -1254,91 +1256,6 @@ struct BoxWalk {
     }
     __device__ __forceinline__ void next() { c += dc; r += dr; if (c >= w) { c -= w; r++; } }
 };
-
-// Layers 1..NL around the solid set S (label 0) in a tile's label bytes (-1
-// free): layer l = the allowed nodes l 4-neighbour dilation steps from S (Sec.
-// 3.2; nodes beyond the pad of a no-slip side never count).  The allowed cells
-// of a tile form a rectangle, where that number of steps is the L1 distance to
-// S, so the labels come from a separable L1 distance transform in place on the
-// label bytes, over the box of S grown by NL: a sweep per row, then one per
-// column (distances capped at NL + 1), then the nodes beyond NL or outside the
-// allowed cells are freed again.  cnt (shared, may be null): per-layer counts
-// are added to cnt[1..NL].  The caller synchronises before reading the labels.
-__device__ __forceinline__ void label_layers_l1(const SimParams &sp, signed char *lab, int T, int sx0, int sx1,
-                                                int sy0, int sy1, int2 oo, int NL, int *cnt) {
-    const int x0 = max(sx0 - NL, 0), x1 = min(sx1 + NL, T - 1), y0 = max(sy0 - NL, 0), y1 = min(sy1 + NL, T - 1);
-    const int cap = NL + 1;
-    for (int y = y0 + (int)threadIdx.x; y <= y1; y += blockDim.x) {
-        signed char *row = lab + y * T;
-        int last = -(1 << 20);
-        for (int x = x0; x <= x1; x++) {
-            if (row[x] == 0) last = x;
-            else row[x] = (signed char)min(x - last, cap);
-        }
-        last = 1 << 20;
-        for (int x = x1; x >= x0; x--) {
-            if (row[x] == 0) last = x;
-            else row[x] = (signed char)min((int)row[x], min(last - x, cap));
-        }
-    }
-    __syncthreads();
-    for (int x = x0 + (int)threadIdx.x; x <= x1; x += blockDim.x) {
-        int d = cap;
-        for (int y = y0; y <= y1; y++) {
-            signed char *q = lab + y * T + x;
-            d = min((int)*q, d + 1);
-            *q = (signed char)d;
-        }
-        d = cap;
-        for (int y = y1; y >= y0; y--) {
-            signed char *q = lab + y * T + x;
-            d = min((int)*q, d + 1);
-            *q = (signed char)d;
-        }
-    }
-    __syncthreads();
-    const int w = x1 - x0 + 1, n = w * (y1 - y0 + 1);
-    BoxWalk wk(w);
-    for (int k = threadIdx.x; k < n; k += blockDim.x, wk.next()) {
-        const int lx = x0 + wk.c, ly = y0 + wk.r, t = ly * T + lx;
-        const int d = lab[t];
-        if (d < 1) continue;
-        if (d <= NL && allowed_cell(sp, oo.x + lx, oo.y + ly)) {
-            if (cnt) atomicAdd(&cnt[d], 1);
-        } else {
-            lab[t] = -1;
-        }
-    }
-}
-
-// The nodes of layers 1..NL (labelled, in the box [x0, x1] x [y0, y1]) in one
-// list, layer l at lists[loff[l] .. loff[l + 1]) (packed lx | ly << 16), so
-// that a layer's targets fill whole warps.  cnt holds the per-layer counts of
-// label_layers_l1 and is used up.  False (and no list) when more than cap
-// nodes; the caller then scans the tile for each layer.  Synchronises.
-__device__ __forceinline__ bool list_layers(const signed char *lab, int T, int x0, int x1, int y0, int y1, int NL,
-                                            int *cnt, int *loff, int *lists, int cap) {
-    if (threadIdx.x == 0) {
-        loff[1] = 0;
-        for (int l = 1; l <= NL; l++) {
-            loff[l + 1] = loff[l] + cnt[l];
-            cnt[l] = loff[l];
-        }
-    }
-    __syncthreads();
-    const bool listed = loff[NL + 1] <= cap;
-    if (listed) {
-        const int w = x1 - x0 + 1, n = w * (y1 - y0 + 1);
-        BoxWalk wk(w);
-        for (int k = threadIdx.x; k < n; k += blockDim.x, wk.next()) {
-            const int lx = x0 + wk.c, ly = y0 + wk.r;
-            const int d = lab[ly * T + lx];
-            if (d >= 1) lists[atomicAdd(&cnt[d], 1)] = lx | (ly << 16);
-        }
-    }
-    __syncthreads();
-    return listed;
-}
 
 // Rows of a solid's band over the CTAs of a cluster (one CTA: all of them).
 struct Strips {
