@@ -138,7 +138,7 @@ struct ForceAdjArgs {
 };
 
 __host__ __device__ __forceinline__ int force_adj_smem_elems(int tx, int ty) {
-    return 6 * KMAX * force_patch_n(tx, ty) + 3 * ((tx + 1) * ty + tx * (ty + 1)) + 3 * TILE_N;
+    return 4 * KMAX * force_patch_n(tx, ty) + 9 * ((tx + 1) * ty + tx * (ty + 1)) + 3 * TILE_N;
 }
 __host__ __device__ __forceinline__ int force_adj_smem_max() {
     int m = 0;
@@ -168,61 +168,55 @@ __device__ __forceinline__ void stress_adjoint(R Axx, R Axy, R Ayx, R Ayy, R G, 
     Abyx += -Dbyx * inv - dlb * Axy;
 }
 
+// Sum of v over the warp into *s (shared), one addition per warp.
+__device__ __forceinline__ void warp_add_to(double *s, double v) {
+    if (__ballot_sync(0xffffffffu, __double_as_longlong(v) != 0ll) == 0u) return;  // (an FP64 compare would cost as an addition)
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+    if ((threadIdx.x & 31) == 0) atomicAdd(s, v);
+}
+
+// One registered tile.  Each half-edge's adjoints (of one solid's edge derivatives and edge
+// phi) go to shared memory, and each patch node gathers those of the half-edges whose
+// stencil holds it; the solids' sums meet once per warp.
+// Bound by latency: a tile or two per SM, in a chain of loads, edge terms and the gather.
+// (Scattered from the half-edges with atomics -- compare-and-swap loops on shared floats, and
+// on doubles with every thread of the tile at one address -- a disk of radius 39 took 55 us; gathered, 16;
+// 256 disks of radius 16 on 2048^2: 300 us less a step.)
 template <class R>
 __device__ void force_adjoint_tile(const SimParams &sp, const ForceAdjArgs<R> &a, const int tile, ForceShared<R> &fs,
-                                   double *sGb, double *sRb, R *dyn, bool node_only) {
-    const int TX = sp.tx, PX = TX + 2, PN = force_patch_n(TX, sp.ty);
-    const int NXE = (TX + 1) * sp.ty, NYE = TX * (sp.ty + 1);
-    R *sX = dyn, *sY = sX + KMAX * PN, *sP = sY + KMAX * PN;
-    R *bX = sP + KMAX * PN, *bY = bX + KMAX * PN, *bP = bY + KMAX * PN;
-    R *eTb = bP + KMAX * PN;          // [(NXE + NYE) * 3]
-    R *nF = eTb + 3 * (NXE + NYE);    // [3 * TILE_N]: F_x, F_y, Delta rho adjoints of the tile nodes
+                                   double *sGb, double *sRb, double *sRc, R *dyn, bool node_only) {
+    const int TX = sp.tx, TY = sp.ty, PX = TX + 2, PN = force_patch_n(TX, TY);
+    const int NXE = (TX + 1) * TY, NE = NXE + TX * (TY + 1);
+    R *sX = dyn, *sY = sX + KMAX * PN, *sP = sY + KMAX * PN, *bP = sP + KMAX * PN;
+    R *eS = bP + KMAX * PN;  // [4][NE]: adjoint of the half-edge's solid stress, and of its sum of lambda
+    R *eG = eS + 4 * NE;     // [5][NE]: of one solid's edge derivatives Xn, Xt, Yn, Yt and of its edge phi
+    R *nF = eG + 5 * NE;     // [3 * TILE_N]: F_x, F_y, Delta rho adjoints of the tile nodes
     const R eps = pick<R>(sp.eps, sp.eps_f), eta = pick<R>(sp.eta, sp.eta_f);
-    const R rho_f = pick<R>(sp.rho_f, sp.rho_f_f);
-    const int tx = tile % sp.ntx, ty = tile / sp.ntx;
-    const int i0 = tx * TX, j0 = ty * sp.ty;
-    if (threadIdx.x == 0) {
-        int n = min(a.reg_count[tile], sp.kmax);
-        for (int k = 0; k < n; k++) fs.ids[k] = a.reg_solids[tile * KMAX + k];
-        for (int k = 1; k < n; k++) {
-            int v = fs.ids[k], m = k - 1;
-            while (m >= 0 && fs.ids[m] > v) { fs.ids[m + 1] = fs.ids[m]; m--; }
-            fs.ids[m + 1] = v;
+    const int i0 = tile % sp.ntx * TX, j0 = tile / sp.ntx * TY;
+    __syncthreads();  // the previous tile's shared state is no longer read
+    if (threadIdx.x < 32) {  // slot = rank of the id, as the forward
+        const int k = threadIdx.x, n = min(a.reg_count[tile], sp.kmax);
+        const int id = k < n ? a.reg_solids[tile * KMAX + k] : 0x7fffffff;
+        int rank = 0;
+#pragma unroll
+        for (int m = 0; m < KMAX; m++) rank += __shfl_sync(0xffffffffu, id, m) < id ? 1 : 0;
+        if (k < n) {
+            const SolidDesc &sd = a.solids[id];
+            fs.ids[rank] = id;
+            fs.sfr[rank] = a.frame[id];
+            fs.sG[rank] = pick<R>(sd.G, sd.G_f);
+            fs.sD[rank] = pick<R>(sd.drho, sd.drho_f);
+            fs.sA[rank] = pick<R>(sd.accel, sd.accel_f);
+            fs.srq[rank] = Rsq<R>(sd);
+            fs.sT[rank] = sd.T;
+            fs.soff[rank] = sd.off;
+            sGb[rank] = 0.0;
+            sRb[rank] = 0.0;
+            // drho_s = rho_f (r - 1), a_s = -(1 - 1/r) g with r = rho_s / rho_f
+            const double ir = sp.rho_f / sd.rho_s;
+            sRc[rank] = sp.gravity * ir * ir;
         }
-        fs.nk = n;
-    }
-    __syncthreads();
-    const int n = fs.nk;
-    if (threadIdx.x < n) {
-        const SolidDesc &sd = a.solids[fs.ids[threadIdx.x]];
-        fs.sfr[threadIdx.x] = a.frame[fs.ids[threadIdx.x]];
-        fs.sG[threadIdx.x] = pick<R>(sd.G, sd.G_f);
-        fs.sD[threadIdx.x] = pick<R>(sd.drho, sd.drho_f);
-        fs.sA[threadIdx.x] = pick<R>(sd.accel, sd.accel_f);
-        fs.srq[threadIdx.x] = Rsq<R>(sd);
-        fs.sT[threadIdx.x] = sd.T;
-        fs.soff[threadIdx.x] = sd.off;
-        sGb[threadIdx.x] = 0.0;
-        sRb[threadIdx.x] = 0.0;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n * PN; idx += blockDim.x) {
-        const int ks = idx / PN, p = idx % PN;
-        const int px = p % PX, py = p / PX;
-        const int gx = i0 - 1 + px, gy = j0 - 1 + py;
-        const Frame fr = fs.sfr[ks];
-        const int T = fs.sT[ks];
-        const int lx = sp.wall_x ? gx - fr.ox : wrapi(gx - fr.ox, sp.nx);
-        const int ly = sp.wall_y ? gy - fr.oy : wrapi(gy - fr.oy, sp.ny);
-        R X = nanv<R>(), Y = nanv<R>(), Pv = nanv<R>();
-        if (in_box(fr, lx, ly)) {
-            const R *Xs = a.xi + fs.soff[ks];
-            X = Xs[ly * T + lx];
-            Y = Xs[T * T + ly * T + lx];
-            if (X == X) Pv = phi_eta(X, Y, lx, ly, fr, fs.srq[ks]);
-        }
-        sX[ks * PN + p] = X; sY[ks * PN + p] = Y; sP[ks * PN + p] = Pv;
-        bX[ks * PN + p] = R(0); bY[ks * PN + p] = R(0); bP[ks * PN + p] = R(0);
+        if (k == 0) fs.nk = n;
     }
     {
         const int lt = threadIdx.x;
@@ -234,214 +228,253 @@ __device__ void force_adjoint_tile(const SimParams &sp, const ForceAdjArgs<R> &a
         nF[2 * TILE_N + lt] = in ? a.Db[c] : R(0);
     }
     __syncthreads();
+    const int n = fs.nk;
+    for (int ks = 0; ks < n; ks++) {
+        const Frame fr = fs.sfr[ks];
+        const int T = fs.sT[ks];
+        const R *Xs = a.xi + fs.soff[ks];
+        BoxWalk wk(PX);
+        for (int p = threadIdx.x; p < PN; p += blockDim.x, wk.next()) {
+            const int gx = i0 - 1 + wk.c, gy = j0 - 1 + wk.r;
+            const int lx = sp.wall_x ? gx - fr.ox : wrapi(gx - fr.ox, sp.nx);
+            const int ly = sp.wall_y ? gy - fr.oy : wrapi(gy - fr.oy, sp.ny);
+            R X = nanv<R>(), Y = nanv<R>(), Pv = nanv<R>();
+            if (in_box(fr, lx, ly)) {
+                X = Xs[ly * T + lx];
+                Y = Xs[T * T + ly * T + lx];
+                if (X == X) Pv = phi_eta(X, Y, lx, ly, fr, fs.srq[ks]);
+            }
+            sX[ks * PN + p] = X; sY[ks * PN + p] = Y; sP[ks * PN + p] = Pv;
+            bP[ks * PN + p] = R(0);
+        }
+    }
+    __syncthreads();
     // Node terms: Delta rho = sum lam drho_s / max(1, L), A_y = sum lam a_s / max(1, L).
     {
-        const int lt = threadIdx.x, cx = lt & (TX - 1), cy = lt >> sp.lx;
-        const int p = (cy + 1) * PX + cx + 1;
+        const int lt = threadIdx.x, p = ((lt >> sp.lx) + 1) * PX + (lt & (TX - 1)) + 1;
         const R Dbar = nF[2 * TILE_N + lt], Aybar = nF[TILE_N + lt];
-        if (Dbar != R(0) || Aybar != R(0)) {
-            R L = 0, D = 0, Ay = 0;
-            for (int ks = 0; ks < n; ks++) {
-                const R ph = sP[ks * PN + p];
-                if (!(ph == ph)) continue;
+        R L = 0, D = 0, Ay = 0;
+        for (int ks = 0; ks < n; ks++) {
+            const R ph = sP[ks * PN + p];
+            if (!(ph == ph)) continue;
+            const R lam = R(1) - heaviside<R>(ph, eps);
+            L += lam; D += lam * fs.sD[ks]; Ay += lam * fs.sA[ks];
+        }
+        R Dr = Dbar, Ar = Aybar, Lb = R(0);
+        if (L > R(1)) {
+            Dr = Dbar / L; Ar = Aybar / L;
+            Lb = -(Dbar * (D / L) + Aybar * (Ay / L)) / L;
+        }
+        for (int ks = 0; ks < n; ks++) {  // uniform over the CTA
+            const R ph = sP[ks * PN + p];
+            double rb = 0.0;
+            if (ph == ph && (Dbar != R(0) || Aybar != R(0))) {
                 const R lam = R(1) - heaviside<R>(ph, eps);
-                L += lam; D += lam * fs.sD[ks]; Ay += lam * fs.sA[ks];
+                bP[ks * PN + p] = -dheaviside<R>(ph, eps) * (Dr * fs.sD[ks] + Ar * fs.sA[ks] + Lb);
+                if (lam != R(0)) rb = (double)lam * ((double)Dr * sp.rho_f - (double)Ar * sRc[ks]);
             }
-            R Dr = Dbar, Ar = Aybar, Lb = R(0);
-            if (L > R(1)) {
-                Dr = Dbar / L; Ar = Aybar / L;
-                Lb = -(Dbar * (D / L) + Aybar * (Ay / L)) / L;
-            }
-            for (int ks = 0; ks < n; ks++) {
-                const R ph = sP[ks * PN + p];
-                if (!(ph == ph)) continue;
-                const R lam = R(1) - heaviside<R>(ph, eps);
-                const R lamb = Dr * fs.sD[ks] + Ar * fs.sA[ks] + Lb;
-                atomicAdd(&bP[ks * PN + p], -dheaviside<R>(ph, eps) * lamb);
-                // drho_s = rho_f (r - 1), a_s = -(1 - 1/r) g with r = rho_s / rho_f
-                const SolidDesc &sd = a.solids[fs.ids[ks]];
-                const double r = sd.rho_s / sp.rho_f;
-                atomicAdd(&sRb[ks], (double)lam * ((double)Dr * (double)rho_f - (double)Ar * sp.gravity / (r * r)));
-            }
+            warp_add_to(&sRb[ks], rb);
         }
     }
     if (node_only) {
         __syncthreads();
         if (threadIdx.x < n) atomicAdd(&a.Rb[fs.ids[threadIdx.x]], sRb[threadIdx.x]);
-        __syncthreads();
         return;
     }
-    // Edge stress adjoints from the tile's nodes: F_x = d_x tau_xx + d_y tau_xy, F_y = d_x tau_xy + d_y tau_yy.
-    for (int e = threadIdx.x; e < NXE + NYE; e += blockDim.x) {
+    const unsigned xdiv = 0xffffffffu / (unsigned)(TX + 1) + 1u;  // e / (TX + 1) = umulhi(e, xdiv)
+    // The stencil of half-edge e: patch node p0 of its low side's first column (row), the
+    // steps along and across it, and whether its normal is x.
+    auto stencil = [&](int e, int &p0, int &al, int &ac) {
+        const bool xe = e < NXE;
+        const int f = e - NXE, ey = xe ? (int)__umulhi((unsigned)e, xdiv) : f >> sp.lx;
+        p0 = ey * PX + (xe ? e - ey * (TX + 1) : f & (TX - 1));
+        al = xe ? PX : 1;
+        ac = xe ? 1 : PX;
+        return xe;
+    };
+    // Solid ks on it: derivatives in x and y, edge phi; false where its stress does not enter.
+    auto edge = [&](int ks, int p0, int al, int ac, bool xe, R &Axx, R &Axy, R &Ayx, R &Ayy, R &ph) {
+        const R *P = sP + ks * PN + p0, *X = sX + ks * PN + p0, *Y = sY + ks * PN + p0;
+        ph = R(0.5) * (P[al] + P[ac + al]);
+        if (!(ph < eps)) return false;  // lambda = 0 and dlambda/dphi = 0: as the forward, no terms
+        R Xn, Xt, Yn, Yt;
+        edge_grad<R>(X[0], X[al], X[2 * al], X[ac], X[ac + al], X[ac + 2 * al], Xn, Xt);
+        if (!(Xt == Xt)) return false;
+        edge_grad<R>(Y[0], Y[al], Y[2 * al], Y[ac], Y[ac + al], Y[ac + 2 * al], Yn, Yt);
+        Axx = xe ? Xn : Xt; Axy = xe ? Xt : Xn; Ayx = xe ? Yn : Yt; Ayy = xe ? Yt : Yn;
+        return true;
+    };
+    if (n > 1) __syncthreads();  // the contact terms add to the node terms
+    // Each half-edge's stress adjoint from the tile's nodes (F_x = d_x tau_xx + d_y tau_xy, F_y =
+    // d_x tau_xy + d_y tau_yy), and through the blend; contact pairs.
+    for (int e = threadIdx.x; e < NE; e += blockDim.x) {
+        int p0, al, ac;
+        const bool xe = stencil(e, p0, al, ac);
         R bxx = 0, bxy = 0, byy = 0;
-        if (e < NXE) {
-            const int ex = e % (TX + 1), ey = e / (TX + 1);
-            if (ex >= 1) { const int l = ey * TX + ex - 1; bxx += nF[l]; bxy += nF[TILE_N + l]; }
-            if (ex < TX) { const int r = ey * TX + ex; bxx -= nF[r]; bxy -= nF[TILE_N + r]; }
+        if (xe) {
+            const int ey = (int)__umulhi((unsigned)e, xdiv), ex = e - ey * (TX + 1), r = ey * TX + ex;
+            if (ex >= 1) { bxx += nF[r - 1]; bxy += nF[TILE_N + r - 1]; }
+            if (ex < TX) { bxx -= nF[r]; bxy -= nF[TILE_N + r]; }
         } else {
-            const int f = e - NXE, ex = f % TX, ey = f / TX;
-            if (ey >= 1) { const int b = (ey - 1) * TX + ex; bxy += nF[b]; byy += nF[TILE_N + b]; }
-            if (ey < sp.ty) { const int t = ey * TX + ex; bxy -= nF[t]; byy -= nF[TILE_N + t]; }
+            const int t = e - NXE;  // ey TX + ex
+            if (t >= TX) { bxy += nF[t - TX]; byy += nF[TILE_N + t - TX]; }
+            if (t < TX * TY) { bxy -= nF[t]; byy -= nF[TILE_N + t]; }
         }
-        eTb[3 * e] = bxx; eTb[3 * e + 1] = bxy; eTb[3 * e + 2] = byy;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < NXE + NYE; e += blockDim.x) {
-        const R tbxx = eTb[3 * e], tbxy = eTb[3 * e + 1], tbyy = eTb[3 * e + 2];
-        if (tbxx == R(0) && tbxy == R(0) && tbyy == R(0)) continue;
-        int pa[3], pb[3];
-        const bool xedge = e < NXE;
-        if (xedge) {
-            const int ex = e % (TX + 1), ey = e / (TX + 1);
-            for (int k = 0; k < 3; k++) { pa[k] = (ey + k) * PX + ex; pb[k] = (ey + k) * PX + ex + 1; }
-        } else {
-            const int f = e - NXE, ex = f % TX, ey = f / TX;
-            for (int k = 0; k < 3; k++) { pa[k] = ey * PX + ex + k; pb[k] = (ey + 1) * PX + ex + k; }
-        }
-        // pass 1: the blended solid stress and sum lambda
-        R Sxx = 0, Sxy = 0, Syy = 0, L = 0;
-        unsigned okm = 0;
-        for (int ks = 0; ks < n; ks++) {
-            const R *X = sX + ks * PN, *Y = sY + ks * PN, *Pp = sP + ks * PN;
-            bool ok = true;
-            for (int k = 0; k < 3; k++) ok = ok && (Pp[pa[k]] == Pp[pa[k]]) && (Pp[pb[k]] == Pp[pb[k]]);
-            if (!ok) continue;
-            const R ph = R(0.5) * (Pp[pa[1]] + Pp[pb[1]]);
-            if (!(ph < eps)) continue;  // lambda = 0 and dlambda/dphi = 0: as the forward, no terms
-            const R lam = R(1) - heaviside<R>(ph, eps);
-            R dXn, dXt, dYn, dYt, txx, txy, tyy;
-            edge_grad<R>(X[pa[0]], X[pa[1]], X[pa[2]], X[pb[0]], X[pb[1]], X[pb[2]], dXn, dXt);
-            edge_grad<R>(Y[pa[0]], Y[pa[1]], Y[pa[2]], Y[pb[0]], Y[pb[1]], Y[pb[2]], dYn, dYt);
-            const bool good = xedge ? stress_from_grad<R>(dXn, dXt, dYn, dYt, fs.sG[ks], txx, txy, tyy)
-                                    : stress_from_grad<R>(dXt, dXn, dYt, dYn, fs.sG[ks], txx, txy, tyy);
-            if (!good) continue;
-            okm |= 1u << ks;
-            Sxx += lam * txx; Sxy += lam * txy; Syy += lam * tyy; L += lam;
-        }
-        R Sbxx = tbxx, Sbxy = tbxy, Sbyy = tbyy, Lb = R(0);
-        if (L > R(1)) {
-            Sbxx /= L; Sbxy /= L; Sbyy /= L;
-            Lb = -(tbxx * Sxx + tbxy * Sxy + tbyy * Syy) / (L * L);
-        }
-        // pass 2: each solid's stress and weight
-        for (int ks = 0; ks < n; ks++) {
-            if (!((okm >> ks) & 1u)) continue;
-            const R *X = sX + ks * PN, *Y = sY + ks * PN, *Pp = sP + ks * PN;
-            const R ph = R(0.5) * (Pp[pa[1]] + Pp[pb[1]]);
-            const R lam = R(1) - heaviside<R>(ph, eps);
-            R dXn, dXt, dYn, dYt, h_xx, h_xy, h_yy;
-            edge_grad<R>(X[pa[0]], X[pa[1]], X[pa[2]], X[pb[0]], X[pb[1]], X[pb[2]], dXn, dXt);
-            edge_grad<R>(Y[pa[0]], Y[pa[1]], Y[pa[2]], Y[pb[0]], Y[pb[1]], Y[pb[2]], dYn, dYt);
-            const R Axx = xedge ? dXn : dXt, Axy = xedge ? dXt : dXn, Ayx = xedge ? dYn : dYt, Ayy = xedge ? dYt : dYn;
-            stress_from_grad<R>(Axx, Axy, Ayx, Ayy, R(1), h_xx, h_xy, h_yy);  // stress per unit G
-            const R G = fs.sG[ks];
-            const R lamb = G * (Sbxx * h_xx + Sbxy * h_xy + Sbyy * h_yy) + Lb;
-            atomicAdd(&sGb[ks], (double)(lam * (Sbxx * h_xx + Sbxy * h_xy + Sbyy * h_yy)));
-            R Abxx = 0, Abxy = 0, Abyx = 0, Abyy = 0;
-            stress_adjoint<R>(Axx, Axy, Ayx, Ayy, G, lam * Sbxx, lam * Sbxy, lam * Sbyy, Abxx, Abxy, Abyx, Abyy);
-            // back to the 2x3 stencils: dn = b1 - a1, dt = (b2 + a2 - b0 - a0) / 4
-            const R bXn = xedge ? Abxx : Abxy, bXt = xedge ? Abxy : Abxx;
-            const R bYn = xedge ? Abyx : Abyy, bYt = xedge ? Abyy : Abyx;
-            R *gX = bX + ks * PN, *gY = bY + ks * PN, *gP = bP + ks * PN;
-            atomicAdd(&gX[pb[1]], bXn); atomicAdd(&gX[pa[1]], -bXn);
-            atomicAdd(&gX[pb[2]], bXt / R(4)); atomicAdd(&gX[pa[2]], bXt / R(4));
-            atomicAdd(&gX[pb[0]], -bXt / R(4)); atomicAdd(&gX[pa[0]], -bXt / R(4));
-            atomicAdd(&gY[pb[1]], bYn); atomicAdd(&gY[pa[1]], -bYn);
-            atomicAdd(&gY[pb[2]], bYt / R(4)); atomicAdd(&gY[pa[2]], bYt / R(4));
-            atomicAdd(&gY[pb[0]], -bYt / R(4)); atomicAdd(&gY[pa[0]], -bYt / R(4));
-            const R phb = -dheaviside<R>(ph, eps) * lamb;
-            atomicAdd(&gP[pa[1]], R(0.5) * phb);
-            atomicAdd(&gP[pb[1]], R(0.5) * phb);
-        }
-        // pass 3: contact pairs (Eq. 3_6_collision_stress), not normalised
-        for (int ks = 0; ks < n; ks++) {
-            if (!((okm >> ks) & 1u)) continue;
-            const R *Ps = sP + ks * PN;
-            const R phs = R(0.5) * (Ps[pa[1]] + Ps[pb[1]]);
-            if (!(phs < eps)) continue;
-            for (int kt = ks + 1; kt < n; kt++) {
-                if (!((okm >> kt) & 1u)) continue;
-                const R *Pt = sP + kt * PN;
-                const R pht = R(0.5) * (Pt[pa[1]] + Pt[pb[1]]);
-                if (!(pht < eps)) continue;
-                const R fsv = R(0.5) * (R(1) - phs / eps), ftv = R(0.5) * (R(1) - pht / eps);
-                const bool take_s = fsv < ftv;
-                const R fm = take_s ? fsv : ftv;
-                R gn, gt;
-                edge_grad<R>(Ps[pa[0]] - Pt[pa[0]], Ps[pa[1]] - Pt[pa[1]], Ps[pa[2]] - Pt[pa[2]],
-                             Ps[pb[0]] - Pt[pb[0]], Ps[pb[1]] - Pt[pb[1]], Ps[pb[2]] - Pt[pb[2]], gn, gt);
-                const R gxx = xedge ? gn : gt, gyy = xedge ? gt : gn;
-                const R nrm = rsqrt_<R>(gxx * gxx + gyy * gyy);
-                if (nrm == R(0)) continue;
-                const R nx_ = gxx / nrm, ny_ = gyy / nrm;
-                const R Gst = fs.sG[ks] + fs.sG[kt];
-                const R kk = -eta * fm * Gst;
-                const R kkb = tbxx * (nx_ * nx_ - R(0.5)) + tbxy * (nx_ * ny_) + tbyy * (ny_ * ny_ - R(0.5));
-                const R nbx = kk * (R(2) * tbxx * nx_ + tbxy * ny_), nby = kk * (tbxy * nx_ + R(2) * tbyy * ny_);
-                const R gG = -eta * fm * kkb;
-                atomicAdd(&sGb[ks], (double)gG);
-                atomicAdd(&sGb[kt], (double)gG);
-                const R fmb = -eta * Gst * kkb;
-                const int kw = take_s ? ks : kt;
-                const R phw = -fmb / (R(2) * eps);  // f = (1 - phi / eps) / 2
-                atomicAdd(&bP[kw * PN + pa[1]], R(0.5) * phw);
-                atomicAdd(&bP[kw * PN + pb[1]], R(0.5) * phw);
-                const R nd = nx_ * nbx + ny_ * nby;
-                const R gbx = (nbx - nx_ * nd) / nrm, gby = (nby - ny_ * nd) / nrm;
-                const R gbn = xedge ? gbx : gby, gbt = xedge ? gby : gbx;
-                // (gn, gt) = edge_grad(P_s - P_t)
-                const int ksk[2] = {ks, kt};
-                for (int w = 0; w < 2; w++) {
-                    const R sgn = w == 0 ? R(1) : R(-1);
-                    R *gP = bP + ksk[w] * PN;
-                    atomicAdd(&gP[pb[1]], sgn * gbn); atomicAdd(&gP[pa[1]], -sgn * gbn);
-                    atomicAdd(&gP[pb[2]], sgn * gbt / R(4)); atomicAdd(&gP[pa[2]], sgn * gbt / R(4));
-                    atomicAdd(&gP[pb[0]], -sgn * gbt / R(4)); atomicAdd(&gP[pa[0]], -sgn * gbt / R(4));
+        R Lb = R(0), Sbxx = bxx, Sbxy = bxy, Sbyy = byy;
+        if (n > 1 && (bxx != R(0) || bxy != R(0) || byy != R(0))) {
+            R Sxx = 0, Sxy = 0, Syy = 0, L = 0;
+            unsigned okm = 0;
+            for (int ks = 0; ks < n; ks++) {
+                R Axx, Axy, Ayx, Ayy, ph, txx, txy, tyy;
+                if (!edge(ks, p0, al, ac, xe, Axx, Axy, Ayx, Ayy, ph) ||
+                    !stress_from_grad<R>(Axx, Axy, Ayx, Ayy, fs.sG[ks], txx, txy, tyy))
+                    continue;
+                const R lam = R(1) - heaviside<R>(ph, eps);
+                okm |= 1u << ks;
+                Sxx += lam * txx; Sxy += lam * txy; Syy += lam * tyy; L += lam;
+            }
+            if (L > R(1)) {
+                Sbxx /= L; Sbxy /= L; Sbyy /= L;
+                Lb = -(bxx * Sxx + bxy * Sxy + byy * Syy) / (L * L);
+            }
+            // contact pairs (Eq. 3_6_collision_stress), not normalised
+            for (unsigned ms = okm; ms; ms &= ms - 1u) {
+                const int ks = __ffs(ms) - 1;
+                const R *Ps = sP + ks * PN + p0;
+                const R phs = R(0.5) * (Ps[al] + Ps[ac + al]);
+                for (unsigned mt = ms & (ms - 1u); mt; mt &= mt - 1u) {
+                    const int kt = __ffs(mt) - 1;
+                    const R *Pt = sP + kt * PN + p0;
+                    const R pht = R(0.5) * (Pt[al] + Pt[ac + al]);
+                    const R fsv = R(0.5) * (R(1) - phs / eps), ftv = R(0.5) * (R(1) - pht / eps);
+                    const bool take_s = fsv < ftv;
+                    const R fm = take_s ? fsv : ftv;
+                    R gn, gt;
+                    edge_grad<R>(Ps[0] - Pt[0], Ps[al] - Pt[al], Ps[2 * al] - Pt[2 * al], Ps[ac] - Pt[ac],
+                                 Ps[ac + al] - Pt[ac + al], Ps[ac + 2 * al] - Pt[ac + 2 * al], gn, gt);
+                    const R gxx = xe ? gn : gt, gyy = xe ? gt : gn;
+                    const R nrm = rsqrt_<R>(gxx * gxx + gyy * gyy);
+                    if (nrm == R(0)) continue;
+                    const R nx_ = gxx / nrm, ny_ = gyy / nrm;
+                    const R Gst = fs.sG[ks] + fs.sG[kt];
+                    const R kk = -eta * fm * Gst;
+                    const R kkb = bxx * (nx_ * nx_ - R(0.5)) + bxy * (nx_ * ny_) + byy * (ny_ * ny_ - R(0.5));
+                    const R nbx = kk * (R(2) * bxx * nx_ + bxy * ny_), nby = kk * (bxy * nx_ + R(2) * byy * ny_);
+                    const R gG = -eta * fm * kkb;
+                    atomicAdd(&sGb[ks], (double)gG);
+                    atomicAdd(&sGb[kt], (double)gG);
+                    const R phw = eta * Gst * kkb / (R(2) * eps);  // f = (1 - phi / eps) / 2
+                    R *const w = bP + (take_s ? ks : kt) * PN + p0;
+                    atomicAdd(&w[al], R(0.5) * phw);
+                    atomicAdd(&w[ac + al], R(0.5) * phw);
+                    const R nd = nx_ * nbx + ny_ * nby;
+                    const R gbx = (nbx - nx_ * nd) / nrm, gby = (nby - ny_ * nd) / nrm;
+                    const R gbn = xe ? gbx : gby, gbt = (xe ? gby : gbx) * R(0.25);
+                    for (int v = 0; v < 2; v++) {  // (gn, gt) = edge_grad(P_s - P_t)
+                        const R sn = v == 0 ? gbn : -gbn, st = v == 0 ? gbt : -gbt;
+                        R *const g = bP + (v == 0 ? ks : kt) * PN + p0;
+                        atomicAdd(&g[ac + al], sn); atomicAdd(&g[al], -sn);
+                        atomicAdd(&g[ac + 2 * al], st); atomicAdd(&g[2 * al], st);
+                        atomicAdd(&g[ac], -st); atomicAdd(&g[0], -st);
+                    }
                 }
             }
         }
+        eS[e] = Sbxx; eS[NE + e] = Sbxy; eS[2 * NE + e] = Sbyy; eS[3 * NE + e] = Lb;
     }
-    __syncthreads();
-    // phi = phi_0(xi): push the level-set adjoint onto xi and flush to the solids' adjoint tiles
-    for (int idx = threadIdx.x; idx < n * PN; idx += blockDim.x) {
-        const int ks = idx / PN, p = idx % PN;
-        R gx_ = bX[ks * PN + p], gy_ = bY[ks * PN + p];
-        const R pb_ = bP[ks * PN + p];
-        const R X = sX[ks * PN + p], Y = sY[ks * PN + p];
-        if (!(X == X)) continue;
-        const int px = p % PX, py = p / PX;
-        const Frame fr = fs.sfr[ks];
-        const int gxg = i0 - 1 + px, gyg = j0 - 1 + py;
-        const int lx = sp.wall_x ? gxg - fr.ox : wrapi(gxg - fr.ox, sp.nx);
-        const int ly = sp.wall_y ? gyg - fr.oy : wrapi(gyg - fr.oy, sp.ny);
-        if (pb_ != R(0)) {
-            R dx_, dy_;
-            dphi_deta<R>(X, Y, lx, ly, fr, dx_, dy_);
-            gx_ += pb_ * dx_;
-            gy_ += pb_ * dy_;
+    for (int ks = 0; ks < n; ks++) {
+        const R G = fs.sG[ks];
+        double gb = 0.0;
+        bool any = false;
+        for (int e = threadIdx.x; e < NE; e += blockDim.x) {  // the half-edges of the loop above
+            const R Sbxx = eS[e], Sbxy = eS[NE + e], Sbyy = eS[2 * NE + e], Lb = eS[3 * NE + e];
+            R g[5] = {0, 0, 0, 0, 0}, Axx, Axy, Ayx, Ayy, ph, hxx, hxy, hyy;
+            int p0, al, ac;
+            const bool xe = stencil(e, p0, al, ac);
+            if ((Sbxx != R(0) || Sbxy != R(0) || Sbyy != R(0)) && edge(ks, p0, al, ac, xe, Axx, Axy, Ayx, Ayy, ph) &&
+                stress_from_grad<R>(Axx, Axy, Ayx, Ayy, R(1), hxx, hxy, hyy)) {  // stress per unit G
+                const R lam = R(1) - heaviside<R>(ph, eps), tau = Sbxx * hxx + Sbxy * hxy + Sbyy * hyy;
+                gb += (double)(lam * tau);
+                R bxx = 0, bxy = 0, byx = 0, byy = 0;
+                stress_adjoint<R>(Axx, Axy, Ayx, Ayy, G, lam * Sbxx, lam * Sbxy, lam * Sbyy, bxx, bxy, byx, byy);
+                // of dn = b1 - a1 and dt = (b2 + a2 - b0 - a0) / 4 of both components
+                g[0] = xe ? bxx : bxy; g[1] = R(0.25) * (xe ? bxy : bxx);
+                g[2] = xe ? byx : byy; g[3] = R(0.25) * (xe ? byy : byx);
+                g[4] = R(-0.5) * dheaviside<R>(ph, eps) * (G * tau + Lb);
+                any = true;
+            }
+#pragma unroll
+            for (int k = 0; k < 5; k++) eG[k * NE + e] = g[k];
         }
-        if (gx_ == R(0) && gy_ == R(0)) continue;
+        warp_add_to(&sGb[ks], gb);
+        any = __syncthreads_or(any);
+        // Patch node (px, py) and the half-edges around it: x-edge (ex, ey) lies between the
+        // patch columns ex and ex + 1, along the rows ey .. ey + 2; y-edges with x and y exchanged.
+        const Frame fr = fs.sfr[ks];
         const int T = fs.sT[ks];
         R *Xb = a.xib + fs.soff[ks];
-        atomicAdd(&Xb[ly * T + lx], gx_);
-        atomicAdd(&Xb[T * T + ly * T + lx], gy_);
+        BoxWalk wk(PX);
+        for (int p = threadIdx.x; p < PN; p += blockDim.x, wk.next()) {
+            const int px = wk.c, py = wk.r;
+            const R X = sX[ks * PN + p], Y = sY[ks * PN + p];
+            if (!(X == X)) continue;
+            R gx = 0, gy = 0, gp = bP[ks * PN + p];
+            if (any) {
+#pragma unroll
+                for (int dir = 0; dir < 2; dir++) {
+                    const int pn = dir == 0 ? px : py, pt = dir == 0 ? py : px;      // across and along the edges
+                    const int nn = dir == 0 ? TX + 1 : TY + 1, nt = dir == 0 ? TY : TX;  // their number
+#pragma unroll
+                    for (int side = 0; side < 2; side++) {  // the node on the low (0) or the high side of the edge
+                        const int en = pn - side;
+                        if (en < 0 || en >= nn) continue;
+#pragma unroll
+                        for (int k = 0; k < 3; k++) {  // its place along the edge
+                            const int et = pt - k;
+                            if (et < 0 || et >= nt) continue;
+                            const R *q = eG + (dir == 0 ? et * (TX + 1) + en : NXE + en * TX + et);
+                            if (k == 1) {
+                                gx += side ? q[0] : -q[0];
+                                gy += side ? q[2 * NE] : -q[2 * NE];
+                                gp += q[4 * NE];
+                            } else {
+                                gx += k == 2 ? q[NE] : -q[NE];
+                                gy += k == 2 ? q[3 * NE] : -q[3 * NE];
+                            }
+                        }
+                    }
+                }
+            }
+            // phi = phi_0(xi): push the level-set adjoint onto xi, and to the solid's adjoint tile
+            const int gxg = i0 - 1 + px, gyg = j0 - 1 + py;
+            const int lx = sp.wall_x ? gxg - fr.ox : wrapi(gxg - fr.ox, sp.nx);
+            const int ly = sp.wall_y ? gyg - fr.oy : wrapi(gyg - fr.oy, sp.ny);
+            if (gp != R(0)) {
+                R dx_, dy_;
+                dphi_deta<R>(X, Y, lx, ly, fr, dx_, dy_);
+                gx += gp * dx_;
+                gy += gp * dy_;
+            }
+            if (gx == R(0) && gy == R(0)) continue;
+            atomicAdd(&Xb[ly * T + lx], gx);
+            atomicAdd(&Xb[T * T + ly * T + lx], gy);
+        }
+        __syncthreads();  // eG is free again
     }
-    __syncthreads();
     if (threadIdx.x < n) {
         atomicAdd(&a.Gb[fs.ids[threadIdx.x]], sGb[threadIdx.x]);
         atomicAdd(&a.Rb[fs.ids[threadIdx.x]], sRb[threadIdx.x]);
     }
-    __syncthreads();
 }
 
 template <class R>
 __global__ void __launch_bounds__(TILE_N) force_adjoint_kernel(SimParams sp, ForceAdjArgs<R> a, int node_only) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ ForceShared<R> fs;
-    __shared__ double sGb[KMAX], sRb[KMAX];
+    __shared__ double sGb[KMAX], sRb[KMAX], sRc[KMAX];
     const int nact = *a.reg_nactive;
     for (int it = blockIdx.x; it < nact; it += gridDim.x)
-        force_adjoint_tile<R>(sp, a, a.reg_active[it], fs, sGb, sRb, reinterpret_cast<R *>(smem), node_only != 0);
+        force_adjoint_tile<R>(sp, a, a.reg_active[it], fs, sGb, sRb, sRc, reinterpret_cast<R *>(smem), node_only != 0);
 }
 
 // ---------------------------------------------------------------------------
