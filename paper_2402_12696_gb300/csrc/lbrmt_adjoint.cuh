@@ -52,6 +52,8 @@ struct LbAdjArgs {
     R *fb, *cb;        // adjoint of f^n, of the half-force read at step n
     R *Fb, *Db;        // adjoint of F^(n) (2 planes) and Delta rho^(n)
     double *bodyb;     // adjoint of the body force field, accumulated (2 planes) or null
+    R *zero;           // cleared besides: the adjoint of xi^n, before the reverse K2 adds to it
+    long long nzero;
 };
 
 template <class R>
@@ -60,6 +62,7 @@ __global__ void __launch_bounds__(256) lb_adjoint_kernel(SimParams sp, LbAdjArgs
     const int nx = sp.nx, ny = sp.ny;
     const R omega = pick<R>(sp.omega, sp.omega_f), kf = pick<R>(sp.kf, sp.kf_f);
     const R lid = pick<R>(sp.lid_u, sp.lid_u_f);
+    for (long long k = blockIdx.x * 256ll + threadIdx.x; k < a.nzero; k += (long long)gridDim.x * 256) a.zero[k] = R(0);
     for (long long c = blockIdx.x * 256ll + threadIdx.x; c < P; c += (long long)gridDim.x * 256) {
         const int i = (int)(c % nx), j = (int)(c / nx);
         const R rho = a.tape[c], ux = a.tape[P + c], uy = a.tape[2 * P + c];
@@ -1067,7 +1070,7 @@ __global__ void centroid_seed_kernel(SimParams sp, const R *xi, const Frame *fra
         if (!in_box(fr, lx, ly) || !domain_cell(sp, fr.ox + lx, fr.oy + ly)) continue;
         if (!(X[t] == X[t])) continue;
         const R phi = phi_eta(X[t], Y[t], lx, ly, fr, rq);
-        if (!(phi < eps)) continue;
+        if (!(phi < eps) || phi <= -eps) continue;  // dH/dphi = 0 inside
         const R lamb = R((gx * (fr.ox + lx - cx) + gy * (fr.oy + ly - cy)) / lsum);
         const R phb = -dheaviside<R>(phi, eps) * lamb;
         R dx_, dy_;
