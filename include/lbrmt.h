@@ -327,7 +327,8 @@ int lbrmt_uses_overlap(const lbrmt_sim *sim);
 /* Form of the reference-map kernel (Sec. 3.1-3.2): 256, one CTA of 256 threads
  * per solid, or 1024, each solid spread over a cluster of up to 16 CTAs of 512
  * threads.  0 (default) takes the cluster when the solids number at most half the
- * SMs, else 256 (FP64 arithmetic takes it there too, and then reports
+ * SMs (FP32 arithmetic: at most the SMs, a CTA each, where the largest tile has 72 nodes a
+ * side or more), else 256 (FP64 arithmetic takes it there too, and then reports
  * 256); 256 or 1024 fix it (1024 falls back to 256 with FP64 arithmetic).  The results
  * do not depend on the form.  Any other value gives LBRMT_ERR_ARG.  Takes effect at the
  * next step; lbrmt_rmt_threads tells the form in use (after initialisation, else 0). */

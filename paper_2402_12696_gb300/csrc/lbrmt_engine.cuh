@@ -346,10 +346,13 @@ struct Engine {
         int nsm0 = 0, dev0 = 0;
         cudaGetDevice(&dev0);
         cudaDeviceGetAttribute(&nsm0, cudaDevAttrMultiProcessorCount, dev0);
-        // K2's form: the request, else the wide one when the solids number at most
-        // half the SMs.  FP64 takes it unasked only, and reports its 256-thread CTAs.
+        // K2's form: the request, else the wide one when the solids number at most half the
+        // SMs, in FP32 arithmetic also up to one a SM where the tiles are not the smallest: a
+        // CTA of 512 threads alone on its SM then beats the narrow form's 256 (110 disks of radius
+        // 10-20, T = 88, 73 -> 63 us; radius 30, 92 -> 81; radius 10, T = 64, 39.8 and 40.3; radius 5
+        // 35.1 and 38.6; in FP64 157 and 200 at radius 16).  FP64 takes it unasked only, and reports its 256-thread CTAs.
         int w = li->rmt_req;
-        const bool few = sp.nsolids > 0 && 2 * sp.nsolids <= nsm0;
+        const bool few = sp.nsolids > 0 && (2 * sp.nsolids <= nsm0 || (sizeof(R) == 4 && sp.nsolids <= nsm0 && tmax >= 72));
         if (w == 0) w = sizeof(R) == 4 && few ? RMT_THREADS_BIG : RMT_THREADS;
         if (w == RMT_THREADS_BIG && sizeof(R) != 4) w = RMT_THREADS;
         li->rmt_threads = w;

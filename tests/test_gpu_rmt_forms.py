@@ -45,6 +45,8 @@ CASES = {
     "shapes": lambda: scenarios.shapes_small(1),
     "twenty_layers": lambda: _box(120, 130, 0, 1, [_disk(60.2, 65.3, 9.0)], n_layers=20),
     "wide_margin": lambda: _box(200, 190, 0, 1, [_disk(100.2, 95.3, 8.0)], deform_margin=4.0),
+    "one_cta_each": lambda: _box(512, 500, 0, 1, [_disk(25.3 + 51 * (k % 10), 25.2 + 50 * (k // 10), 12.0 + 0.07 * k)
+                                                  for k in range(100)]),
     "long_layers": lambda: _box(430, 440, 1, 1, [_disk(214.3, 220.4, 170.0)], deform_margin=0.05),
 }
 
