@@ -457,6 +457,19 @@ __device__ __forceinline__ void cluster_ld2(const float2 *p, int rank, float &x,
 __device__ __forceinline__ void cluster_ld2(const double2 *p, int rank, double &x, double &y) {
     asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(x), "=d"(y) : "r"(cluster_addr(p, rank)) : "memory");
 }
+// Reductions into another CTA's shared memory.
+__device__ __forceinline__ void cluster_min(int *p, int rank, int v) {
+    asm volatile("red.relaxed.cluster.shared::cluster.min.s32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_max(int *p, int rank, int v) {
+    asm volatile("red.relaxed.cluster.shared::cluster.max.s32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_add(int *p, int rank, int v) {
+    asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_add(unsigned long long *p, int rank, unsigned long long v) {
+    asm volatile("red.relaxed.cluster.shared::cluster.add.u64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "l"(v) : "memory");
+}
 __device__ __forceinline__ void cluster_st(float *p, int rank, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "f"(v) : "memory");
 }
@@ -1511,6 +1524,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     const R *Yi = a.init ? nullptr : Xi + TT;
     const R *Pi = a.init ? nullptr : Yi + TT;  // phi^n, stored by the previous step's relabel
     const R eps = pick<R>(sp.eps, sp.eps_f);
+    if (CL && tid < 4) sbb[tid] = (tid & 1) ? -(1 << 29) : (1 << 29);
     if (tid < 12) bb[tid] = (tid & 1) ? -(1 << 29) : (1 << 29);
     else if (tid < 16) bb[tid] = 0;
     if (tid < 24) lcnt[tid] = 0;
@@ -1525,6 +1539,7 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     int acc[3] = {0, 0, 0};
     int sb[4] = {1 << 29, -(1 << 29), 1 << 29, -(1 << 29)};
     __syncthreads();
+    if constexpr (CL) cluster_arrive();  // every CTA's sbb is set
 
     // Pass 0: the advected set S = {domain nodes with phi^n < 0}, Eqs. 3_1_refmap_adv / 3_1_eno,
     // over this CTA's rows of the input tile's box (the whole tile at initialisation).
@@ -1612,21 +1627,21 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
         if (lane == 0) atomicAdd(&vsum[k - 1], (unsigned long long)((long long)hi * 65536 + lo));
     }
     if (lane == 0) atomicAdd(&bb[12], acc[0]);
-    solid_sync();
-
-    // The box of S over the cluster.
-    if constexpr (CL) {
-        if (warp == 0) {
-            for (int k = 0; k < 4; k++) {
-                int v = (int)cluster_ld(&bb[k], lane < nc ? lane : rank);
-                warp_minmax(v, (k & 1) == 0);
-                if (lane == 0) sbb[k] = v;
-            }
-        }
-    } else if (tid < 4) {
-        sbb[tid] = bb[tid];
-    }
     __syncthreads();
+
+    // The box of S over the cluster, each CTA's reduced into every other's.
+    if constexpr (CL) {
+        cluster_wait();
+        if (warp == 0 && lane < nc)
+            for (int k = 0; k < 4; k += 2) {
+                cluster_min(&sbb[k], lane, bb[k]);
+                cluster_max(&sbb[k + 1], lane, bb[k + 1]);
+            }
+        cluster_sync();
+    } else {
+        if (tid < 4) sbb[tid] = bb[tid];
+        __syncthreads();
+    }
     const int sx0 = sbb[0], sx1 = sbb[1], sy0 = sbb[2], sy1 = sbb[3];
     const bool any = sx0 <= sx1;
     if (!any && tid == 0) atomicOr(a.err, ERR_TILE_OVERFLOW);  // the solid vanished
@@ -1978,32 +1993,16 @@ __device__ void rmt_solid(const SimParams &sp, const RmtArgs<R, S> &a, const int
     for (int k = 0; k < 8; k++) warp_minmax(bx[k], (k & 1) == 0);
     if (lane == 0)
         for (int k = 0; k < 8; k += 2) { atomicMin(&bb[4 + k], bx[k]); atomicMax(&bb[5 + k], bx[k + 1]); }
-    solid_sync();
-    if constexpr (CL) {
-        // the first CTA gathers the boxes and sums of the others, which stay until it has
-        long long v0 = 0, v1 = 0;
-        if (rank == 0 && warp == 0) {
-            const int src = lane < nc ? lane : 0;
-            int v[12];
-            for (int k = 4; k < 12; k++) v[k] = (int)cluster_ld(&bb[k], src);
-            int nS = lane < nc ? (int)cluster_ld(&bb[12], src) : 0;
-            if (lane < nc) {
-                const unsigned *q = reinterpret_cast<const unsigned *>(vsum);
-                v0 = (long long)(((unsigned long long)cluster_ld(q + 1, src) << 32) | cluster_ld(q, src));
-                v1 = (long long)(((unsigned long long)cluster_ld(q + 3, src) << 32) | cluster_ld(q + 2, src));
-            }
-            for (int k = 4; k < 12; k++) warp_minmax(v[k], (k & 1) == 0);
-            nS = __reduce_add_sync(0xffffffffu, nS);
-            for (int d = 16; d > 0; d >>= 1) {
-                v0 += __shfl_down_sync(0xffffffffu, v0, d);
-                v1 += __shfl_down_sync(0xffffffffu, v1, d);
-            }
-            __syncwarp();
-            if (lane == 0) {
-                for (int k = 4; k < 12; k++) bb[k] = v[k];
-                bb[12] = nS;
-                vsum[0] = (unsigned long long)v0;
-                vsum[1] = (unsigned long long)v1;
+    __syncthreads();
+    if constexpr (CL) {  // the boxes and sums of the others go to the first CTA
+        if (rank != 0 && warp == 0) {
+            if (lane < 8) {
+                if (lane & 1) cluster_max(&bb[4 + lane], 0, bb[4 + lane]);
+                else cluster_min(&bb[4 + lane], 0, bb[4 + lane]);
+            } else if (lane == 8) {
+                cluster_add(&bb[12], 0, bb[12]);
+            } else if (lane < 11) {
+                cluster_add(&vsum[lane - 9], 0, vsum[lane - 9]);
             }
         }
         cluster_sync();
