@@ -3,7 +3,7 @@ against central differences in FP64 (directional derivatives of the final
 centroids with respect to the body force field and to one solid's density
 ratio, which the discrete adjoint reproduces to the differencing error):
 windows beyond 5x5 (a disk of a few nodes), a band of 20 layers, disks in
-contact, and a disk for each number of CTAs of a cluster from 16 to 1, down
+contact, disks across periodic edges, and a disk for each number of CTAs of a cluster from 16 to 1, down
 to one CTA whose layers need several rounds.
 """
 import numpy as np
@@ -25,7 +25,7 @@ def _built():
     build.build()
 
 
-def _scenario(n, r, count=1, pitch=0.0, **more):
+def _scenario(n, r, count=1, pitch=0.0, at=(), **more):
     sc = scenarios.adjoint_ldc(n, r=r, G=0.02, rho_ratio=1.3, body=scenarios.smooth_body_field(1, n, amp=2e-5))
     sc.update(more)
     if count > 1:
@@ -33,6 +33,8 @@ def _scenario(n, r, count=1, pitch=0.0, **more):
         # (centres off the nodes: a node on the interface would change sides under the differences)
         sc["solids"] = [{**one, "x": 4.13 + pitch * (k % per + 0.5) + 0.1 * (k % 3), "y": 4.37 + pitch * (k // per + 0.5)}
                         for k in range(count)]
+    if at:
+        sc["solids"] = [{**sc["solids"][0], "x": x, "y": y} for x, y in at]
     return sc
 
 
@@ -40,6 +42,7 @@ CASES = {
     "few_nodes": lambda: _scenario(48, 1.7),
     "twenty_layers": lambda: _scenario(96, 9.0, n_layers=20),
     "contact": lambda: _scenario(96, 9.0, count=4, pitch=18.6),
+    "across_edges": lambda: _scenario(96, 11.0, at=[(0.43, 95.63), (50.33, 0.71)], wall_x=0, wall_y=0, lid_u=0.0),
     "cluster_16": lambda: _scenario(192, 40.0),
     "cluster_8": lambda: _scenario(192, 20.0, count=9, pitch=61.0),
     "cluster_4": lambda: _scenario(160, 8.0, count=20, pitch=30.0),
