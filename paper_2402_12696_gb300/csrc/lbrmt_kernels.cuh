@@ -2184,26 +2184,33 @@ __host__ __device__ __forceinline__ int force_smem_max() {
 // arithmetic, the formula of lambda, and divisions by 3 and 4).
 constexpr int K3_ROUNDS = 3;  // of K3_THREADS threads: 642 edges and 520 patch nodes at most (128 x 2)
 constexpr unsigned K3_NO_NODE = 0x3fffu, K3_NO_EDGE = 0x3ffu;
+// Part `part` of 2^sl of a tile is a band of its rows: a thread outside it has none of them.
 struct ForceMap {
     unsigned nodes, edges;
+    __device__ __forceinline__ bool own() const { return (nodes >> 28) == 0u; }  // the thread's tile node is in the part
     __device__ __forceinline__ unsigned node(int k) const { return (nodes >> (14 * k)) & K3_NO_NODE; }
     __device__ __forceinline__ unsigned edge(int k) const { return (edges >> (10 * k)) & K3_NO_EDGE; }
 };
-__device__ __forceinline__ ForceMap force_map(const SimParams &sp) {
+__device__ __forceinline__ ForceMap force_map(const SimParams &sp, const int part = 0, const int sl = 0) {
     ForceMap m = {0u, 0u};
+    const int h = sp.ty >> sl, r0 = part * h;
     const int TX = sp.tx, PX = TX + 2, PN = force_patch_n(TX, sp.ty), NXE = (TX + 1) * sp.ty, NE = NXE + TX * (sp.ty + 1);
 #pragma unroll
     for (int k = 0; k < 2; k++) {
         const int p = threadIdx.x + k * K3_THREADS;
-        m.nodes |= (p < PN ? (unsigned)((p % PX) | ((p / PX) << 8)) : K3_NO_NODE) << (14 * k);
+        const int row = p / PX - r0;  // tile rows -1 .. h of the part
+        m.nodes |= (p < PN && row >= 0 && row < h + 2 ? (unsigned)((p % PX) | ((p / PX) << 8)) : K3_NO_NODE) << (14 * k);
     }
 #pragma unroll
     for (int k = 0; k < K3_ROUNDS; k++) {
         const int e = threadIdx.x + k * K3_THREADS, f = e - NXE;
         // x-edge between columns ex - 1 and ex (tile coordinates); y-edge between rows ey - 1 and ey
         const int p = e < NXE ? (e / (TX + 1)) * PX + e % (TX + 1) : (f >> sp.lx) * PX + (f & (TX - 1));
-        m.edges |= (e < NE ? (unsigned)p : K3_NO_EDGE) << (10 * k);
+        const int row = (e < NXE ? e / (TX + 1) : f >> sp.lx) - r0;
+        m.edges |= (e < NE && row >= 0 && row < (e < NXE ? h : h + 1) ? (unsigned)p : K3_NO_EDGE) << (10 * k);
     }
+    const int row = ((int)threadIdx.x >> sp.lx) - r0;
+    if (row < 0 || row >= h) m.nodes |= 1u << 28;
     return m;
 }
 
@@ -2364,7 +2371,7 @@ __device__ void force_tile(const SimParams &sp, const ForceArgs<R> &a, const For
         const int cx = threadIdx.x & (TX - 1), cy = threadIdx.x >> sp.lx;
         const int ty = tile / sp.ntx, tx = tile - ty * sp.ntx;
         const int i = tx * TX + cx, j = ty * sp.ty + cy;
-        if (threadIdx.x < TILE_N && i < sp.nx && j < sp.ny) {
+        if (threadIdx.x < TILE_N && fm.own() && i < sp.nx && j < sp.ny) {
             const R *tl = eT + 3 * (cy * (TX + 1) + cx), *tr = eT + 3 * (cy * (TX + 1) + cx + 1);
             const R *tb = eT + 3 * (NXE + cy * TX + cx), *tt = eT + 3 * (NXE + (cy + 1) * TX + cx);
             const R fsx = (tr[0] - tl[0]) + (tt[1] - tb[1]);
@@ -2440,12 +2447,19 @@ __global__ void __launch_bounds__(K3_THREADS) __maxnreg__(sizeof(R) == 4 ? REGS 
     int it = blockIdx.x;
     int tile = it < sp.ntx * sp.nty ? a.reg_active[it] : 0;  // read beside the count
     const int nact = *a.reg_nactive;
-    if (it >= nact) return;  // uniform over the CTA
-    const ForceMap fm = force_map(sp);
+    // FP64: a tile in 2 or 4 parts while the grid holds them all; a tile keeps its SM's FP64
+    // pipe busy, and few tiles then use more of the SMs (one disk of radius 13 on 64^2, 22 -> 14.7
+    // us; in FP32, where a tile is latency, 10.3 and 10.1).
+    int sl = 0;
+    if constexpr (sizeof(R) == 8)
+        while (sl < 2 && (nact << (sl + 1)) <= (int)gridDim.x && (sp.ty >> (sl + 1)) > 0) sl++;
+    if (it >= nact << sl) return;  // uniform over the CTA
+    if (sl > 0) tile = a.reg_active[it >> sl];
+    const ForceMap fm = force_map(sp, it & ((1 << sl) - 1), sl);
     if (threadIdx.x < 32) force_solids<R>(sp, a, tile, fs[0], threadIdx.x);
     __syncthreads();
-    for (int b = 0; it < nact; it += gridDim.x, b ^= 1) {
-        const int next = it + (int)gridDim.x < nact ? a.reg_active[it + gridDim.x] : -1;
+    for (int b = 0; it < nact << sl; it += gridDim.x, b ^= 1) {
+        const int next = it + (int)gridDim.x < nact << sl ? a.reg_active[it + gridDim.x] : -1;
         force_tile<R, true>(sp, a, fm, tile, fs[b], reinterpret_cast<R *>(smem), next, &fs[b ^ 1]);
         tile = next;
     }
